@@ -101,7 +101,7 @@ def draw(rng):
                         diam_x=diam, diam_y=diam, gains=rng.random() < 0.8)
     precision = rng.choice(["fp32", "fp32", "split_fp16", "fp16"]) if what in ("image", "series") else "fp32"
     P = 2 if precision != "fp32" else rng.choice([1, 2, 2, 2])
-    A = logint(16, 512) if what != "series" else logint(16, 256)
+    A = logint(16, 512) if what != "series" and precision == "fp32" else logint(16, 256)
     if precision != "fp32" or what == "efield":
         A = max(16, A & ~3)
     K = rng.choice([1, 3, 5, 7])
