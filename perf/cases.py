@@ -105,6 +105,8 @@ def draw(rng):
     if precision != "fp32" or what == "efield":
         A = max(16, A & ~3)
     K = rng.choice([1, 3, 5, 7])
+    if precision != "fp32" and K == 7:
+        A = min(A, 128)
     sides = rng.choice(["64", "96", "128", "128", "64/96/128"])
     if precision == "fp32" and what in ("image", "gains") and rng.random() < 0.2:
         sides = "32"
@@ -270,8 +272,9 @@ def work(case):
 
 
 def tolerance(case):
-    """About four times the error measured against the 64-bit results (2-norm: FP32 images 1.4e-6,
-    E-field images 1.3e-7, split FP16 1.5e-5, gains 7e-7, S/N 3.4e-6)."""
+    """About four times the error measured against the 64-bit results (2-norm: FP32 images 1.9e-6,
+    E-field images 1.3e-7, split FP16 1.5e-5, FP16 1.2e-3, gains 7e-7, S/N 3.4e-6; largest
+    difference over the root mean square: FP32 8e-5, split FP16 1e-4, FP16 2.2e-2)."""
     if case["what"] == "search":
         return {"rel": 1e-5, "max": 1e-4, "differ": 1e-4}   # best windows tie within a rounding of S/N
     if case["what"] == "gains":
@@ -279,10 +282,10 @@ def tolerance(case):
     if case["what"] == "efield":
         return {"rel": 1e-6, "max": 1e-5}
     if case["precision"] == "fp16":
-        return {"rel": 1e-2, "max": 1e-1}     # 11-bit operands
+        return {"rel": 5e-3, "max": 1e-1}     # 11-bit operands
     if case["precision"] == "split_fp16":
         return {"rel": 6e-5, "max": 6e-4}
-    return {"rel": 6e-6, "max": 1e-4}
+    return {"rel": 8e-6, "max": 3e-4}
 
 
 # ---------------------------------------------------------------- the same results in 64 bits
