@@ -17,6 +17,7 @@ constexpr int kMaxK = 15;
 constexpr int kMaxAP = 4096;           // n_ant * n_pol handled by one CTA's staging
 constexpr int kPairHelpers = 3;        // pair kernel (tc_pair128.cu): gridding-only warps beside its 8 TMEM warps
 constexpr int kPairGatherWarps = 8 + kPairHelpers;
+constexpr int kCompactGatherWarps = 4; // compact kernel (fp32_compact.cu): gridding warps beside its 8 transform warps
 
 // How one grid side N is imaged by the FP32 kernel: the sky is split into
 // Q1 x Q1 pixel classes l = (Q1 m + h) and each CTA owns one class, so it grids
@@ -70,6 +71,13 @@ struct GroupCfg {
     int2 *d_gchan = nullptr;           // device: [n_chan] (block start, block words)
     int gwords = 0;                    // largest channel block (words)
     bool gstage = false;               // blocks staged in shared memory
+    // FP32 plans whose aperture occupies at most 64 x 64 cells: the compact kernel (fp32_compact.cu)
+    bool compact = false;
+    bool cstage = false;               // its gather lists are staged in shared memory
+    int crows = 0, cwords = 0;         // most occupied rows, most list words of a channel
+    uint16_t *d_ltab = nullptr;        // device: gather lists (build_compact_lists)
+    int2 *d_lidx = nullptr;            // device: [n_chan][gridding warps] (first batch, batches)
+    int4 *d_lchan = nullptr;           // device: [n_chan][2] (block start, words, rows, columns), (origin x, y, 0, 0)
     // large grid sides (8 x 8 pixel classes): grid once per (channel, sample) into the occupied
     // alias blocks, fold all classes with one 8 x 8 DFT per folded cell (alias_fold_kernel), then
     // transform each class's loaded grid (fp32_fold64_kernel), in time batches of alias_tb samples
@@ -219,6 +227,15 @@ int launch_tc_pair(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const
 int build_gather_table(const std::vector<short2> &cells, int A, int K, int M, int P, const std::vector<int> &chans,
                        std::vector<uint32_t> &tab, std::vector<int4> &idx, std::vector<int2> &chan,
                        std::vector<unsigned long long> &rowmask, int threads = 0);
+// FP32 kernel for apertures of at most 64 x 64 cells, grid sides 64, 96, 128 (fp32_compact.cu)
+int build_compact_lists(const std::vector<short2> &cells, int A, int K, int P, const std::vector<int> &chans,
+                        std::vector<uint16_t> &tab, std::vector<int2> &idx, std::vector<int4> &chan);
+size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, int words);
+int prepare_compact(const epic_plan_s *plan, const GroupCfg &g);
+int launch_compact(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
+                   cudaStream_t stream);
+int launch_compact_efield(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T,
+                          float2 *out, long long stride, cudaStream_t stream);
 // Register-transform kernels, fold side M = 64 or 48 (fp32_reg64.cu)
 size_t reg64_smem_bytes(int M, int P, int TS, int A, int K, int nker);
 int launch_reg64(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
@@ -247,6 +264,7 @@ struct RawImage {
     int *status = nullptr;
 };
 int fp32_pick_tau(int n_items, int T, int sms);
+int compact_pick_tau(int n_chan, int n_items, int T, int sms);
 // time chunks of one launch: forced (image series), else autotuned for this T, else the cost model
 int choose_tau(const epic_plan_s *plan, const GroupCfg &g, int T);
 // large grid sides (GroupCfg::alias)

@@ -273,19 +273,20 @@ size_t smem_bytes(int A, int K, int nker = 1)
     return (b + 15) & ~static_cast<size_t>(15);
 }
 
-int pick_tau(int n_items, int T, int sms)
+int pick_tau(int n_items, int T, int sms, int n_min, double setup)
 {
     if (T <= 1) return 1;
     // Pick the time split that balances work across SMs: an SM's throughput is
     // about the same with one or two resident CTAs, so the integration takes
     // about (CTAs on the busiest SM) x (samples per CTA + ~2 samples of set-up
     // and partial write).
-    int best = 1;
+    n_min = std::max(1, std::min({n_min, kMaxTau, T}));
+    int best = n_min;
     double best_cost = 1e300;
-    for (int n = 1; n <= kMaxTau && n <= T; n++) {
+    for (int n = n_min; n <= kMaxTau && n <= T; n++) {
         const long long blocks = static_cast<long long>(n_items) * n;
         const long long waves = (blocks + sms - 1) / sms;
-        const double per = static_cast<double>((T + n - 1) / n) + 2.0;
+        const double per = static_cast<double>((T + n - 1) / n) + setup;
         const double cost = waves * per;
         if (cost < best_cost - 1e-9) {
             best_cost = cost;
@@ -338,13 +339,22 @@ int launch_raw(const RawImage &r, const uint8_t *v, const float2 *gains, cudaStr
 
 }  // namespace
 
-int fp32_pick_tau(int n_items, int T, int sms) { return pick_tau(n_items, T, sms); }
+int fp32_pick_tau(int n_items, int T, int sms) { return pick_tau(n_items, T, sms, 1, 2.0); }
+
+// The compact kernel's CTA images all classes of a channel: n_chan CTAs per time chunk, each
+// writing Q times the partial image (set-up and write cost ~4 samples).  No chunk is longer than
+// the per-class kernel's would be, so FP32 sums run over no more samples than there.
+int compact_pick_tau(int n_chan, int n_items, int T, int sms)
+{
+    return pick_tau(n_chan, T, sms, fp32_pick_tau(n_items, T, sms), 4.0);
+}
 
 int choose_tau(const epic_plan_s *plan, const GroupCfg &g, int T)
 {
     int n = plan->force_tau > 0                       ? plan->force_tau
             : (g.tuned_tau > 0 && g.tuned_T == T) ? g.tuned_tau
-                                                  : pick_tau(g.launch_items, T, plan->sm_count);
+            : g.compact                             ? compact_pick_tau(g.n_chan, g.n_items, T, plan->sm_count)
+                                                  : fp32_pick_tau(g.launch_items, T, plan->sm_count);
     return std::max(1, std::min(n, g.tau_cap));
 }
 
@@ -394,6 +404,7 @@ int launch_imaging(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const
     if (g.alias && plan->force_tau == 0) return launch_alias(plan, g, v, gains, T, n_tau, s);
     if (g.tensor && !g.tc_regular) return EPIC_ERR_UNSUPPORTED;   // e.g. an image series: no fold path there
     if (g.tensor) return g.pair ? launch_tc_pair(plan, g, v, gains, T, n_tau, s) : launch_tc_dual(plan, g, v, gains, T, n_tau, s);
+    if (g.compact) return launch_compact(plan, g, v, gains, T, n_tau, s);
     if (g.reg64) return launch_reg64(plan, g, v, gains, T, n_tau, s);
     switch (g.M * 4 + plan->P) {
     case 32 * 4 + 2: return launch_group<32, 2>(plan, g, v, gains, T, n_tau, s);

@@ -108,6 +108,9 @@ void free_plan(epic_plan_s *p)
         cudaFree(g.d_pidx);
         cudaFree(g.d_upper);
         cudaFree(g.d_ef_off);
+        cudaFree(g.d_ltab);
+        cudaFree(g.d_lidx);
+        cudaFree(g.d_lchan);
     }
     delete p;
 }
@@ -788,7 +791,33 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 }
             }
         }
-        if (g.reg64) {
+        // FP32 plans: the compact kernel where every channel's footprints span at most 64 x 64 cells
+        // (any 2x-padded array at sides up to 128) and its planes fit in shared memory
+        if (rc == EPIC_OK && !tensor && (g.N == 64 || g.N == 96 || g.N == 128)) {
+            std::vector<uint16_t> ltab;
+            std::vector<int2> lidx;
+            std::vector<int4> lchan;
+            if (epic::build_compact_lists(cells, n_ant, p->K, n_pol, g.chans, ltab, lidx, lchan) == EPIC_OK) {
+                for (int i = 0; i < g.n_chan; i++) {
+                    g.cwords = std::max(g.cwords, lchan[2 * i].y);
+                    g.crows = std::max(g.crows, lchan[2 * i].z);
+                }
+                auto fits = [&](int words) {   // + static shared memory and the system's share
+                    return epic::compact_smem_bytes(g.N, n_pol, g.crows, n_ant, p->K, p->nker, words) + 1024 <=
+                           static_cast<size_t>(smem_optin);
+                };
+                g.compact = fits(0);
+                g.cstage = fits(g.cwords) && !(diag & EPIC_DIAG_GATHER_GLOBAL);
+            }
+            if (g.compact) {
+                g.R1 = 1;
+                g.R2 = g.M;
+                rc = dev_upload(&g.d_ltab, ltab.data(), ltab.size());
+                if (rc == EPIC_OK) rc = dev_upload(&g.d_lidx, lidx.data(), lidx.size());
+                if (rc == EPIC_OK) rc = dev_upload(&g.d_lchan, lchan.data(), lchan.size());
+            }
+        }
+        if (g.reg64 && !g.compact) {
             g.R1 = 1;
             g.R2 = g.M;
             std::vector<uint32_t> desc;
@@ -881,8 +910,9 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 }
             }
         }
-        g.launch_items = g.pair ? g.n_chan * (g.Q1 == 2 ? 2 : 1) : g.n_items;
+        g.launch_items = g.pair ? g.n_chan * (g.Q1 == 2 ? 2 : 1) : g.compact ? g.n_chan : g.n_items;
         if (g.pair) g.tau_cap = std::max(g.tau_cap, epic::fp32_pick_tau(g.launch_items, max_spectra, p->sm_count));
+        if (g.compact) g.tau_cap = std::max(g.tau_cap, epic::compact_pick_tau(g.n_chan, g.n_items, max_spectra, p->sm_count));
         if (rc == EPIC_OK) rc = dev_upload(&g.d_chans, g.chans.data(), g.chans.size());
         if (rc == EPIC_OK) rc = dev_upload(&g.d_out_off, offs.data(), offs.size());
         if (rc == EPIC_OK) {
@@ -947,6 +977,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
     for (const auto &g : p->groups) {
         if (rc != EPIC_OK) break;
         if (!g.tensor) rc = epic::prepare_fp32(p, g);
+        if (rc == EPIC_OK && g.compact) rc = epic::prepare_compact(p, g);
         if (rc == EPIC_OK && g.alias) rc = epic::prepare_alias(p);
     }
     if (rc == EPIC_OK) {
@@ -1069,7 +1100,8 @@ int epic_autotune(epic_plan_t plan, int n_spectra, void *stream)
         auto add = [&](int n) {
             if (n >= 1 && n <= cap && std::find(cand.begin(), cand.end(), n) == cand.end()) cand.push_back(n);
         };
-        const int c0 = epic::fp32_pick_tau(g.launch_items, n_spectra, plan->sm_count);
+        const int c0 = g.compact ? epic::compact_pick_tau(g.n_chan, g.n_items, n_spectra, plan->sm_count)
+                                 : epic::fp32_pick_tau(g.launch_items, n_spectra, plan->sm_count);
         for (int d = -2; d <= 2; d++) add(c0 + d);
         for (int waves = 1; waves <= 4; waves++)
             add(static_cast<int>((static_cast<long long>(waves) * plan->sm_count) / std::max(1, g.launch_items)));
@@ -1188,7 +1220,8 @@ int epic_image_efield(epic_plan_t plan, const uint8_t *ci4, const float *gains, 
     const auto *g2 = reinterpret_cast<const float2 *>(gains);
     plan->delays = nullptr;
     for (const auto &g : plan->groups) {
-        const int rc = epic::launch_reg64_efield(plan, g, ci4, g2, n_spectra, o, plan->ef_stride, s);
+        const int rc = g.compact ? epic::launch_compact_efield(plan, g, ci4, g2, n_spectra, o, plan->ef_stride, s)
+                                 : epic::launch_reg64_efield(plan, g, ci4, g2, n_spectra, o, plan->ef_stride, s);
         if (rc != EPIC_OK) return rc;
     }
     return EPIC_OK;

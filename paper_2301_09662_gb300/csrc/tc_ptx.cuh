@@ -210,6 +210,12 @@ __device__ __forceinline__ void tmem_st16_issue(uint32_t taddr, const uint32_t (
                  : "memory");
 }
 
+__device__ __forceinline__ void tmem_st8_issue(uint32_t taddr, const uint32_t (&r)[8])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+                 : "memory");
+}
+
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // Barrier `id` (1..15) over `count` threads (a multiple of 32).
