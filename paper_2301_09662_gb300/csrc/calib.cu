@@ -8,10 +8,24 @@
 //
 // phi_a = exp(-2 pi i (kx_a lx + ky_a ly) / N) for a source at the image offset
 // (lx, ly) = (l N du, m N du) pixels (a source there has e_a ~ phi_a and appears
-// at +(lx, ly) in the image).  One CTA per (channel, polarisation); phi, the gains,
-// the integer |e|^2 sums and E(t) stay in shared memory.
+// at +(lx, ly) in the image).
+//
+// gain_solve_cluster_kernel (n_ant n_pol <= 1024): one thread-block cluster per channel, each CTA
+// a share of the samples.  A warp takes a sample at a time: its lanes hold the row's voltages
+// (words lane, lane + 32, ..), form E(t) of both polarisations by one warp reduction and add
+// E conj(e) to the sums of their own antennas in registers, so an iteration reads the voltages
+// once.  The CTAs' sums meet through distributed shared memory: each CTA finishes a slice of the
+// antennas and hands its gains to the others, so there is no workspace and one launch.  Bound by
+// issue (about 20 instructions a voltage and iteration).  256 antennas, 64 channels, two
+// polarisations, 1000 spectra, two iterations: 96 us, against 322 us for one CTA per channel and
+// polarisation, whose loads' latency was the limit.
+// gain_solve_kernel (larger arrays): one CTA per (channel, polarisation), E(t) of all samples in
+// shared memory, the voltages read twice per iteration.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
+
+#include <cooperative_groups.h>
 
 #include "dft_small.cuh"
 #include "epic_internal.cuh"
@@ -118,6 +132,263 @@ gain_solve_kernel(const uint8_t *__restrict__ v, const short2 *__restrict__ cell
     for (int a = tid; a < A; a += kCalThreads) gains[(static_cast<size_t>(c) * A + a) * P + p] = g[a];
 }
 
+constexpr int kCalWarps = kCalThreads / 32;
+
+// Byte b of four 4+4-bit voltages x (as ci4_decode), two instructions a part: with the sign bits
+// flipped a nibble is n + 8 in 0..15; or-ed into the mantissa of 2^23 at bit s it reads
+// 2^23 + (n + 8) 2^s, and one FMA takes the offset and the scale away, exactly.
+struct Ci4Word {
+    uint32_t lo, hi;
+    __device__ __forceinline__ explicit Ci4Word(uint32_t x) : lo(x ^ 0x88888888u), hi(lo >> 16) {}
+    template <int S>
+    static __device__ __forceinline__ float part(uint32_t y)
+    {
+        const float m = __uint_as_float((y & (0xFu << S)) | 0x4B000000u);
+        return fmaf(m, 1.f / static_cast<float>(1 << S), -(8388608.f / static_cast<float>(1 << S) + 8.f));
+    }
+    __device__ __forceinline__ float2 get(int b) const
+    {
+        const uint32_t y = b & 2 ? hi : lo;
+        return b & 1 ? make_float2(part<12>(y), part<8>(y)) : make_float2(part<4>(y), part<0>(y));
+    }
+};
+
+size_t cal_cluster_smem(int AP)   // sums of every warp, the CTA's sums, gains, phases, sum |e|^2
+{
+    return sizeof(float2) * static_cast<size_t>(AP) * (kCalWarps + 3) + sizeof(int) * static_cast<size_t>(AP) * (kCalWarps + 2);
+}
+
+// grid (cluster size x n_chan); R: words a lane holds of a sample's row (n_ant n_pol <= 128 R)
+template <int R>
+__global__ void __launch_bounds__(kCalThreads, R <= 4 ? 2 : 1)
+gain_solve_cluster_kernel(const uint8_t *__restrict__ v, const short2 *__restrict__ cells, const int *__restrict__ chans,
+                          int A, int C, int P, int T, int N, double lx, double ly, int n_iter, float2 *__restrict__ gains)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = static_cast<int>(cl.block_rank()), CL = static_cast<int>(cl.num_blocks());
+    extern __shared__ float2 sm[];
+    const int AP = A * P;
+    float2 *red = sm;                                // [warps][AP]
+    float2 *part = red + kCalWarps * AP;             // [AP] the CTA's sums
+    float2 *g = part + AP;                           // [AP]
+    float2 *phi = g + AP;                            // [AP] (per antenna, repeated per polarisation)
+    float *wden = reinterpret_cast<float *>(phi + AP);   // [warps][AP] exact sum |e|^2 of the first iteration
+    int *iden = reinterpret_cast<int *>(wden + kCalWarps * AP);   // [AP] the CTA's
+    int *den = iden + AP;                            // [AP] over the cluster
+    __shared__ float ss_part[2];                     // the CTA's slice of sum |g|^2 per polarisation
+    __shared__ float red2[kCalWarps][2];
+    __shared__ float2 ref[2];
+    __shared__ float scale[2];
+    const int c = chans[blockIdx.x / CL];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int i0 = static_cast<int>(static_cast<long long>(AP) * rank / CL);
+    const int i1 = static_cast<int>(static_cast<long long>(AP) * (rank + 1) / CL);
+
+    // the lattice phases of the CTA's slice, to every CTA of the cluster
+    for (int i = i0 + tid; i < i1; i += kCalThreads) {
+        const short2 k = cells[static_cast<size_t>(c) * A + i / P];
+        double turns = (static_cast<double>(k.x) * lx + static_cast<double>(k.y) * ly) / N;
+        turns -= rint(turns);
+        double s, co;
+        sincospi(-2.0 * turns, &s, &co);
+        const float2 f = make_float2(static_cast<float>(co), static_cast<float>(s));
+        for (int r = 0; r < CL; r++) cl.map_shared_rank(phi, r)[i] = f;
+    }
+    for (int i = tid; i < AP; i += kCalThreads) {
+        g[i] = make_float2(1.f, 0.f);
+    }
+    cl.sync();
+
+    const bool words = (AP & 3) == 0 && (reinterpret_cast<uintptr_t>(v) & 3) == 0;
+    const int step = CL * kCalWarps;
+    auto load = [&](int t, uint32_t (&x)[R]) {
+        const uint8_t *row = v + (static_cast<size_t>(t) * C + c) * AP;
+#pragma unroll
+        for (int r = 0; r < R; r++) {
+            const int w = lane + 32 * r;
+            x[r] = 0u;                               // decodes to zero
+            if (t >= T) continue;
+            if (words) {
+                if (4 * w < AP) x[r] = __ldg(reinterpret_cast<const uint32_t *>(row) + w);
+            } else {
+#pragma unroll
+                for (int b = 0; b < 4; b++)
+                    if (4 * w + b < AP) x[r] |= static_cast<uint32_t>(__ldg(row + 4 * w + b)) << (8 * b);
+            }
+        }
+    };
+    const float invA = 1.f / static_cast<float>(A);
+    // one iteration over the CTA's samples; FIRST adds up |e|^2 as well (FP32 holds these integers
+    // exactly: at most 128 a sample, far fewer than 2^17 samples a warp)
+    auto sweep = [&](auto first) {
+        constexpr bool FIRST = decltype(first)::value;
+        // w = g conj(phi) of the lane's values
+        float2 w[R][4], num[R][4];
+        float dd[FIRST ? R : 1][4];
+#pragma unroll
+        for (int r = 0; r < R; r++)
+#pragma unroll
+            for (int b = 0; b < 4; b++) {
+                const int i = 4 * (lane + 32 * r) + b;
+                w[r][b] = i < AP ? cmul(g[i], make_float2(phi[i].x, -phi[i].y)) : make_float2(0.f, 0.f);
+                num[r][b] = make_float2(0.f, 0.f);
+                if (FIRST) dd[r][b] = 0.f;
+            }
+        uint32_t x[R], xn[R];
+        load(rank * kCalWarps + warp, x);
+        for (int t = rank * kCalWarps + warp; t < T; t += step) {
+            load(t + step, xn);
+            // polarisation of value i = i mod P: with P = 2 the byte's parity
+            float2 e0 = make_float2(0.f, 0.f), e1 = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int r = 0; r < R; r++) {
+                const Ci4Word cw(x[r]);
+#pragma unroll
+                for (int b = 0; b < 4; b++) {
+                    const float2 e = cw.get(b);
+                    float2 &o = (b & 1) ? e1 : e0;
+                    o.x = fmaf(w[r][b].x, e.x, fmaf(-w[r][b].y, e.y, o.x));
+                    o.y = fmaf(w[r][b].x, e.y, fmaf(w[r][b].y, e.x, o.y));
+                }
+            }
+            if (P == 1) {
+                e0 = cadd(e0, e1);
+                e1 = e0;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                e0.x += __shfl_xor_sync(0xffffffffu, e0.x, o);
+                e0.y += __shfl_xor_sync(0xffffffffu, e0.y, o);
+                e1.x += __shfl_xor_sync(0xffffffffu, e1.x, o);
+                e1.y += __shfl_xor_sync(0xffffffffu, e1.y, o);
+            }
+            e0 = cscale(e0, invA);
+            e1 = cscale(e1, invA);
+#pragma unroll
+            for (int r = 0; r < R; r++) {
+                const Ci4Word cw(x[r]);
+#pragma unroll
+                for (int b = 0; b < 4; b++) {
+                    const float2 e = cw.get(b);
+                    const float2 E = (b & 1) ? e1 : e0;
+                    float2 &o = num[r][b];
+                    o.x = fmaf(E.x, e.x, fmaf(E.y, e.y, o.x));      // E conj(e)
+                    o.y = fmaf(E.y, e.x, fmaf(-E.x, e.y, o.y));
+                    if (FIRST) dd[r][b] = fmaf(e.x, e.x, fmaf(e.y, e.y, dd[r][b]));
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < R; r++) x[r] = xn[r];
+        }
+#pragma unroll
+        for (int r = 0; r < R; r++)
+#pragma unroll
+            for (int b = 0; b < 4; b++) {
+                const int i = 4 * (lane + 32 * r) + b;
+                if (i >= AP) continue;
+                red[warp * AP + i] = num[r][b];
+                if (FIRST) wden[warp * AP + i] = dd[r][b];
+            }
+    };
+    for (int it = 0; it < n_iter; it++) {
+        if (it == 0) sweep(std::true_type{});
+        else sweep(std::false_type{});
+        __syncthreads();
+        for (int i = tid; i < AP; i += kCalThreads) {
+            float2 s = red[i];
+            for (int k = 1; k < kCalWarps; k++) s = cadd(s, red[k * AP + i]);
+            part[i] = s;
+            if (it == 0) {
+                int d = 0;
+                for (int k = 0; k < kCalWarps; k++) d += static_cast<int>(wden[k * AP + i]);
+                iden[i] = d;
+            }
+        }
+        cl.sync();
+        // the CTA's slice: sums over the cluster in rank order, gains before normalisation
+        float s0 = 0.f, s1 = 0.f;
+        for (int i = i0 + tid; i < i1; i += kCalThreads) {
+            float2 s = make_float2(0.f, 0.f);
+            int dd = 0;
+            for (int r = 0; r < CL; r++) {
+                s = cadd(s, cl.map_shared_rank(part, r)[i]);
+                if (it == 0) dd += cl.map_shared_rank(iden, r)[i];
+            }
+            if (it == 0) den[i] = dd;
+            else dd = den[i];
+            const float2 gi = dd > 0 ? cscale(cmul(phi[i], s), 1.f / static_cast<float>(dd)) : make_float2(0.f, 0.f);
+            const float q = gi.x * gi.x + gi.y * gi.y;
+            if (P == 2 && (i & 1)) s1 += q;
+            else s0 += q;
+            for (int r = 0; r < CL; r++) cl.map_shared_rank(g, r)[i] = gi;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            s0 += __shfl_xor_sync(0xffffffffu, s0, o);
+            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+        }
+        if (lane == 0) {
+            red2[warp][0] = s0;
+            red2[warp][1] = s1;
+        }
+        __syncthreads();
+        if (tid < 2) {
+            float s = 0.f;
+            for (int k = 0; k < kCalWarps; k++) s += red2[k][tid];
+            ss_part[tid] = s;
+        }
+        cl.sync();
+        // antenna 0's phase to zero, then RMS amplitude to one
+        if (tid < P) {
+            float s = 0.f;
+            for (int r = 0; r < CL; r++) s += cl.map_shared_rank(ss_part, r)[tid];
+            const float rms = sqrtf(s * invA);
+            scale[tid] = rms > 0.f ? 1.f / rms : 1.f;
+            const float2 g0 = g[tid];
+            const float r = sqrtf(g0.x * g0.x + g0.y * g0.y);
+            ref[tid] = r > 0.f ? make_float2(g0.x / r, -g0.y / r) : make_float2(1.f, 0.f);
+        }
+        __syncthreads();
+        for (int i = tid; i < AP; i += kCalThreads) {
+            const int p = P == 2 ? i & 1 : 0;
+            g[i] = cscale(cmul(g[i], ref[p]), scale[p]);
+        }
+        __syncthreads();
+    }
+    for (int i = i0 + tid; i < i1; i += kCalThreads) gains[static_cast<size_t>(c) * AP + i] = g[i];
+    cl.sync();   // no CTA leaves while another may still read its shared memory
+}
+
+template <int R>
+int launch_cal_cluster(const epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, int T, double lx, double ly, int n_iter,
+                       float2 *gains, cudaStream_t s)
+{
+    const size_t smem = cal_cluster_smem(plan->A * plan->P);
+    const auto kfn = gain_solve_cluster_kernel<R>;
+    if (cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(cal_cluster_smem(128 * R))) !=
+        cudaSuccess)
+        return EPIC_ERR_CUDA;
+    // up to two CTAs an SM, in one wave; a CTA keeps at least a sample per warp
+    int cl = 1;
+    while (cl < 8 && cl * g.n_chan <= plan->sm_count && 2 * cl * kCalWarps <= T) cl *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(g.n_chan * cl));
+    cfg.blockDim = dim3(kCalThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = static_cast<unsigned>(cl);
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kfn, v, plan->d_cells, g.d_chans, plan->A, plan->C, plan->P, T, g.N, lx, ly, n_iter,
+                              gains) == cudaSuccess
+               ? EPIC_OK
+               : EPIC_ERR_CUDA;
+}
+
 size_t cal_smem(int A, int T) { return sizeof(float2) * (2 * static_cast<size_t>(A) + T) + sizeof(int) * A; }
 
 }  // namespace
@@ -137,6 +408,16 @@ extern "C" int epic_solve_gains(epic_plan_t plan, const uint8_t *ci4, int n_spec
     auto s = static_cast<cudaStream_t>(stream);
     for (const auto &g : plan->groups) {
         const double lx = l * g.N * plan->du, ly = m * g.N * plan->du;
+        const int AP = plan->A * plan->P;
+        if (AP <= 1024) {
+            auto *out = reinterpret_cast<float2 *>(gains_out);
+            const int rc = AP <= 128   ? epic::launch_cal_cluster<1>(plan, g, ci4, n_spectra, lx, ly, n_iter, out, s)
+                           : AP <= 256 ? epic::launch_cal_cluster<2>(plan, g, ci4, n_spectra, lx, ly, n_iter, out, s)
+                           : AP <= 512 ? epic::launch_cal_cluster<4>(plan, g, ci4, n_spectra, lx, ly, n_iter, out, s)
+                                       : epic::launch_cal_cluster<8>(plan, g, ci4, n_spectra, lx, ly, n_iter, out, s);
+            if (rc != EPIC_OK) return rc;
+            continue;
+        }
         epic::gain_solve_kernel<<<static_cast<unsigned>(g.n_chan * plan->P), epic::kCalThreads, smem, s>>>(
             ci4, plan->d_cells, g.d_chans, plan->A, plan->C, plan->P, n_spectra, g.N, lx, ly, n_iter,
             reinterpret_cast<float2 *>(gains_out));
