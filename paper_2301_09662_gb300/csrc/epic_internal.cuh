@@ -45,7 +45,7 @@ struct GroupCfg {
     std::vector<int> chans;            // plan channel indices in this group
     int *d_chans = nullptr;            // device copy of chans
     long long *d_out_off = nullptr;    // device: output offset (complex elements) per group channel
-    double *d_wpow = nullptr;          // device: |W^(l)|^2 on the shifted [N][N] layout
+    float2 *d_wpow = nullptr;          // device: |W^(l)|^2 on the shifted [N][N] layout, as FP32 pairs (hi, lo)
     double2 *d_tw64 = nullptr;         // per-antenna kernels: exp(+2 pi i k / N) in FP64
     double2 *d_Y = nullptr;            // per-antenna kernels: [n_chan][3][2K-1][N] partial auto images
     float2 *d_twN = nullptr;           // device: exp(+2 pi i k / N), k < N
@@ -126,7 +126,8 @@ struct epic_plan_s {
     uint8_t *d_dft48 = nullptr;        // the 48-point DFT in the same 128 x 128 operands (grid side 96)
     short2 *d_cells = nullptr;         // [C][A]
     float2 *d_kernel = nullptr;        // [K*K]
-    int *d_autoint = nullptr;          // [C][A][4] exact integer auto sums
+    int *d_autoint = nullptr;          // [chunk or image][C][A][4] exact integer auto sums
+    double *d_apq = nullptr;           // [image][C][4] A_pq: XX, YY, Re XY, Im XY (one shared kernel)
     int *d_status = nullptr;           // sticky device status word
     double f_ref = 0;                  // delay phases: reference frequency (mid-band, Hz)
     double du = 0.5;                   // grid cell size in wavelengths
@@ -145,7 +146,7 @@ struct epic_plan_s {
     // CUDA graph of one integration, re-captured when T, pointers or profiling change
     bool use_graph = true;
     cudaStream_t cap = nullptr;        // capture stream
-    std::vector<cudaStream_t> side;    // one branch per grid side
+    std::vector<cudaStream_t> side;    // one branch per grid side, beside the auto sums' branch
     cudaEvent_t ev_fork = nullptr, ev_auto = nullptr;
     std::vector<cudaEvent_t> ev_join;
     cudaGraphExec_t gexec = nullptr;
@@ -187,7 +188,8 @@ int prepare_fp32(const epic_plan_s *plan, const GroupCfg &g);
 int prepare_reg64(const epic_plan_s *plan, const GroupCfg &g);
 
 // shared pieces (image_common.cu)
-int launch_autopower(epic_plan_s *plan, const uint8_t *v, int T, cudaStream_t stream);
+int auto_chunks(const epic_plan_s *plan, int T);   // time chunks of its integer sums
+int launch_autopower(epic_plan_s *plan, const uint8_t *v, const float2 *gains, int T, cudaStream_t stream);
 int launch_epilogue(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T, int n_tau,
                     float2 *out, cudaStream_t stream);
 // per-antenna kernels: auto-correlation grid X(rho) -> Y(rho_y, l_x) per channel and product
@@ -195,7 +197,7 @@ int launch_auto_rho(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, c
 // delay table of the current call (plan->delays, [T][A] seconds) into plan->d_dtab
 int launch_delay_prep(epic_plan_s *plan, int T, cudaStream_t stream);
 // image series: per-image auto sums and one epilogue image per time chunk
-int launch_autopower_series(epic_plan_s *plan, const uint8_t *v, int spi, int n_img, cudaStream_t stream);
+int launch_autopower_series(epic_plan_s *plan, const uint8_t *v, const float2 *gains, int spi, int n_img, cudaStream_t stream);
 int launch_epilogue_series(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int spi, int n_img,
                            float2 *out, cudaStream_t stream);
 // imaging kernel of one group (FP32 or tensor form as the plan says)
@@ -257,7 +259,7 @@ struct RawImage {
     const float2 *kernel = nullptr;    // [K*K]
     const int *chans = nullptr;        // [C] identity channel list
     const long long *out_off = nullptr;  // [C]
-    const double *wpow = nullptr;      // [N][N]
+    const float2 *wpow = nullptr;      // [N][N], FP32 pairs
     const float2 *twN = nullptr;       // [N]
     float *partial = nullptr;          // [n_tau][n_items][M*M][NPF]
     int *autoint = nullptr;            // [C][A][4]
@@ -283,7 +285,7 @@ int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, cud
 // host tables shared by the plan and the static-scratch entry point
 int host_cell_map(const double *ant_xy_m, int n_ant, const double *freq_hz, int n_chan, const int *grid_n,
                   double du, int K, std::vector<short2> &cells);
-void host_kernel_power(const float *kern, int K, int N, std::vector<double> &out);
+void host_kernel_power(const float *kern, int K, int N, std::vector<float2> &out);
 // raise a kernel's dynamic shared-memory cap to the device limit (less its static shared memory);
 // EPIC_ERR_UNSUPPORTED if `need` does not fit
 int raise_dyn_smem_cap(const void *kfn, size_t need);

@@ -289,7 +289,7 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
         // ================ unpack, calibrate, grid
         const int gt = tid - kFT, gw = warp - kFW;
         const int2 my = lidx[ci * kGW + gw];                     // (first batch, batches)
-        const bool words = (AP & 3) == 0;
+        const bool words = (AP & 3) == 0 && (reinterpret_cast<uintptr_t>(v) & 3) == 0;
         const int APW = AP >> 2;
         uint32_t pre[TS][kPreC];
         // the bytes of sample t: words gt, gt + kGT, ..; or single bytes gt, gt + kGT, .. packed four to a word

@@ -438,7 +438,7 @@ int image_fp32(epic_plan_s *plan, const uint8_t *v, const float2 *gains, int T, 
     if (fork && cudaEventRecord(plan->ev_fork, stream) != cudaSuccess) return EPIC_ERR_CUDA;
     if (autosub) {
         prof_mark(plan, stream, stage, true);
-        rc = launch_autopower(plan, v, T, stream);
+        rc = launch_autopower(plan, v, gains, T, stream);
         prof_mark(plan, stream, stage++, false);
         if (rc != EPIC_OK) return rc;
         if (fork && cudaEventRecord(plan->ev_auto, stream) != cudaSuccess) return EPIC_ERR_CUDA;

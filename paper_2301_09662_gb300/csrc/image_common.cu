@@ -7,8 +7,10 @@
 // is A_pq |W^(l)|^2 with A_pq = sum_a g_ap g_aq^* sum_t e_ap e_aq^*.  The inner
 // time sum is exact in int32 (|e e^*| components <= 128, T <= 10^5); the
 // antenna sum and the subtraction run in FP64 because the auto term can be
-// much larger than what is left after it is removed.
+// much larger than what is left after it is removed (the subtraction in FP32
+// pairs of ~48 bits, see epilogue_kernel).
 #include <algorithm>
+#include <type_traits>
 
 #include "epic_internal.cuh"
 
@@ -21,152 +23,232 @@ __device__ __forceinline__ void ci4_parts(uint32_t b, int &re, int &im)
     im = static_cast<int>(static_cast<int8_t>((b << 4) & 0xF0u)) >> 4;
 }
 
-// grid (C, n_chunks): per antenna, integer sums over one time chunk
-//   [0] sum |e_X|^2   [1] sum |e_Y|^2   [2] Re sum e_X e_Y^*   [3] Im sum e_X e_Y^*
-__global__ void __launch_bounds__(kThreads)
-autopower_kernel(const uint8_t *__restrict__ v, int T, int C, int A, int P, int n_chunks,
-                 size_t chunk_stride, int *__restrict__ autoint)
+// sums of one antenna: [0] |e_X|^2  [1] |e_Y|^2  [2] Re e_X e_Y^*  [3] Im e_X e_Y^*
+template <int P>
+__device__ __forceinline__ void auto_add(uint32_t bx, uint32_t by, int (&s)[P == 2 ? 4 : 1])
 {
+    int xr, xi;
+    ci4_parts(bx, xr, xi);
+    s[0] += xr * xr + xi * xi;
+    if constexpr (P == 2) {
+        int yr, yi;
+        ci4_parts(by, yr, yi);
+        s[1] += yr * yr + yi * yi;
+        s[2] += xr * yr + xi * yi;
+        s[3] += xi * yr - xr * yi;
+    }
+}
+
+// grid (C, n_chunks): per antenna, the integer sums over one time chunk, from 32-bit words of the
+// rows (WORDS: n_ant n_pol a multiple of 4 and v aligned to it, 4 / P antennas a thread) or one antenna a thread.
+// chunk_stride 0: every chunk adds into one (cleared) sum; else each chunk stores its own.
+template <int P, bool WORDS>
+__global__ void __launch_bounds__(128)
+autopower_kernel(const uint8_t *__restrict__ v, int T, int C, int A, int n_chunks, size_t chunk_stride,
+                 int *__restrict__ autoint)
+{
+    constexpr int NA = WORDS ? 4 / P : 1, NS = P == 2 ? 4 : 1;
     const int c = blockIdx.x;
     const int chunk = blockIdx.y;
     const int t0 = static_cast<int>(static_cast<long long>(T) * chunk / n_chunks);
     const int t1 = static_cast<int>(static_cast<long long>(T) * (chunk + 1) / n_chunks);
-    for (int a = threadIdx.x; a < A; a += blockDim.x) {
-        int sxx = 0, syy = 0, sxyr = 0, sxyi = 0;
-        for (int t = t0; t < t1; t++) {
-            const uint8_t *row = v + (static_cast<size_t>(t) * C + c) * A * P + static_cast<size_t>(a) * P;
-            int xr, xi;
-            ci4_parts(row[0], xr, xi);
-            sxx += xr * xr + xi * xi;
-            if (P == 2) {
-                int yr, yi;
-                ci4_parts(row[1], yr, yi);
-                syy += yr * yr + yi * yi;
-                sxyr += xr * yr + xi * yi;
-                sxyi += xi * yr - xr * yi;
+    const size_t row = static_cast<size_t>(C) * A * P;
+    for (int u = threadIdx.x; u * NA < A; u += blockDim.x) {
+        int s[NA][NS];
+#pragma unroll
+        for (int n = 0; n < NA; n++)
+#pragma unroll
+            for (int k = 0; k < NS; k++) s[n][k] = 0;
+        const uint8_t *src = v + static_cast<size_t>(t0) * row + static_cast<size_t>(c) * A * P + static_cast<size_t>(u) * NA * P;
+#pragma unroll 8
+        for (int t = t0; t < t1; t++, src += row) {
+            if constexpr (WORDS) {
+                const uint32_t w = __ldg(reinterpret_cast<const uint32_t *>(src));
+#pragma unroll
+                for (int n = 0; n < NA; n++) auto_add<P>(w >> (8 * P * n), w >> (8 * P * n + 8), s[n]);
+            } else {
+                auto_add<P>(src[0], P == 2 ? src[P - 1] : 0u, s[0]);
             }
         }
-        // chunk_stride 0: every chunk adds into one sum; else one sum per chunk (image series)
-        int *dst = autoint + chunk * chunk_stride + (static_cast<size_t>(c) * A + a) * 4;
-        atomicAdd(dst + 0, sxx);
-        if (P == 2) {
-            atomicAdd(dst + 1, syy);
-            atomicAdd(dst + 2, sxyr);
-            atomicAdd(dst + 3, sxyi);
+#pragma unroll
+        for (int n = 0; n < NA; n++) {
+            int *dst = autoint + chunk * chunk_stride + (static_cast<size_t>(c) * A + u * NA + n) * 4;
+#pragma unroll
+            for (int k = 0; k < NS; k++) {
+                if (chunk_stride) dst[k] = s[n][k];
+                else atomicAdd(dst + k, s[n][k]);
+            }
         }
     }
 }
 
-// grid (pixel tiles, group channels).  Partial layout written by the imaging
+// A_pq = sum_a g_ap g_aq^* sum_t e_ap e_aq^* of channel c, by one block, in FP64 and a fixed order
+// (deterministic); sums of n_chunks chunks (exact integers) first.  Result in apq: XX, YY, Re XY, Im XY.
+template <int P>
+__device__ __forceinline__ void auto_reduce(const int *autoint, int n_chunks, size_t chunk_stride, const float2 *gains,
+                                            int A, int c, double (&red)[kThreads / 32][4], double (&apq)[4])
+{
+    double s[4] = {0, 0, 0, 0};
+    for (int a = threadIdx.x; a < A; a += kThreads) {
+        int ia[4] = {0, 0, 0, 0};
+        const int *src = autoint + (static_cast<size_t>(c) * A + a) * 4;
+#pragma unroll 4
+        for (int k = 0; k < n_chunks; k++) {
+            if constexpr (P == 2) {
+                const int4 q = *reinterpret_cast<const int4 *>(src + k * chunk_stride);
+                ia[0] += q.x;
+                ia[1] += q.y;
+                ia[2] += q.z;
+                ia[3] += q.w;
+            } else {
+                ia[0] += src[k * chunk_stride];
+            }
+        }
+        double gxr = 1, gxi = 0, gyr = 1, gyi = 0;
+        if (gains) {
+            const float2 gx = gains[(static_cast<size_t>(c) * A + a) * P];
+            gxr = gx.x;
+            gxi = gx.y;
+            if (P == 2) {
+                const float2 gy = gains[(static_cast<size_t>(c) * A + a) * P + 1];
+                gyr = gy.x;
+                gyi = gy.y;
+            }
+        }
+        s[0] += (gxr * gxr + gxi * gxi) * static_cast<double>(ia[0]);
+        if (P == 2) {
+            s[1] += (gyr * gyr + gyi * gyi) * static_cast<double>(ia[1]);
+            // g_x g_y^* (I_re + i I_im)
+            const double pr = gxr * gyr + gxi * gyi, pi = gxi * gyr - gxr * gyi;
+            s[2] += pr * ia[2] - pi * ia[3];
+            s[3] += pr * ia[3] + pi * ia[2];
+        }
+    }
+    // fixed-order tree: within each warp by shuffles, then the warps' sums by thread 0..3
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_down_sync(0xffffffffu, s[k], o);
+    if ((threadIdx.x & 31) == 0)
+        for (int k = 0; k < 4; k++) red[threadIdx.x >> 5][k] = s[k];
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        double tot = 0;
+        for (int i = 0; i < kThreads / 32; i++) tot += red[i][threadIdx.x];
+        apq[threadIdx.x] = tot;
+    }
+    __syncthreads();
+}
+
+// grid (C, images): A_pq once per channel and image, for the epilogue's blocks to read
+template <int P>
+__global__ void __launch_bounds__(kThreads)
+auto_sum_kernel(const int *__restrict__ autoint, int n_chunks, size_t chunk_stride, const float2 *__restrict__ gains, int A,
+                int C, double *__restrict__ apq_out)
+{
+    __shared__ double red[kThreads / 32][4];
+    __shared__ double apq[4];
+    auto_reduce<P>(autoint + static_cast<size_t>(blockIdx.y) * n_chunks * chunk_stride, n_chunks, chunk_stride, gains, A,
+                   blockIdx.x, red, apq);
+    if (threadIdx.x < 4) apq_out[(static_cast<size_t>(blockIdx.y) * C + blockIdx.x) * 4 + threadIdx.x] = apq[threadIdx.x];
+}
+
+// A number as an unevaluated FP32 pair (hi, lo), about 48 bits.
+__device__ __forceinline__ float2 to_pair(double x)
+{
+    const float hi = static_cast<float>(x);
+    return make_float2(hi, static_cast<float>(x - static_cast<double>(hi)));
+}
+// h + x exactly as (sum, error): the error is returned (Knuth's TwoSum)
+__device__ __forceinline__ float two_sum(float &h, float x)
+{
+    const float t = h + x;
+    const float bp = t - h;
+    const float e = (h - (t - bp)) + (x - bp);
+    h = t;
+    return e;
+}
+// s -= a b in pairs (a, b, s pairs of ~48 bits; the product's high part by an exact two-product)
+__device__ __forceinline__ void pair_msub(float2 &s, float2 a, float2 b)
+{
+    const float p = __fmul_rn(a.x, b.x);
+    const float e = fmaf(a.x, b.y, fmaf(a.y, b.x, fmaf(a.x, b.x, -p)));
+    const float r = two_sum(s.x, -p);
+    s.y += r - e;
+}
+
+// grid (pixel tiles, group channels, images).  Partial layout written by the imaging
 // kernels: [tau][item][pos][NPF] with item = ci * Q + (hy * Q1 + hx) and
 // pos = py * M + px, where folded frequency m sits at digit position
 // up (R2 (m mod R1) + m / R1) (R1 = 1, R2 = M for natural order; up = 2 when a
 // side-32 grid was transformed zero-padded to 64 points, whose even
 // frequencies are the 32-point transform).
-template <int M, int P>
+//
+// Bound by HBM (partials read once, image written once).  The subtraction
+// runs in FP32 pairs (~48 bits): GB300's FP64 pipe does ~2 operations a clock
+// and SM, and five FP64 operations and eight conversions a value made it, not
+// the memory, the limit; A_pq itself is summed in FP64, once per channel and
+// image (auto_sum_kernel), not in every block.  Whole calls: 25 Stokes images of
+// 64 channels of 128 x 128 5.21 -> 3.66 ms, 64 channels of 512 x 512 with 2048
+// antennas 21.75 -> 20.40 ms.
+template <int N, int M, int P>
 __global__ void __launch_bounds__(kThreads)
-epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int N, int Q1, int R1, int R2,
+epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R1, int R2,
                 const int *__restrict__ chans, const long long *__restrict__ out_off,
-                const double *__restrict__ wpow, const int *__restrict__ autoint,
-                const float2 *__restrict__ gains, int A, int T, unsigned flags, float2 *__restrict__ out,
-                size_t auto_stride, long long out_stride,
-                const double2 *__restrict__ Yauto, const double2 *__restrict__ tw64, int K, int up)
+                const float2 *__restrict__ wpow, const double *__restrict__ apq_tab, const int *__restrict__ autoint,
+                const float2 *__restrict__ gains, int A, int C, int T, unsigned flags, float2 *__restrict__ out,
+                long long out_stride, const double2 *__restrict__ Yauto, const double2 *__restrict__ tw64, int K)
 {
+    constexpr int NPF = P == 2 ? 4 : 1;          // sums and products per pixel
+    constexpr int up = N < M ? M / N : 1, Q1 = N < M ? 1 : N / M, Q = Q1 * Q1, NN = N * N;
     // blockIdx.z = image: it sums time chunks [z n_tau, (z + 1) n_tau) and uses
     // the auto sums and output block of index z (one image unless a series)
     const int img = blockIdx.z;
-    partial += static_cast<size_t>(img) * n_tau * n_items * (M * M) * (P == 2 ? 4 : 1);
-    autoint += img * auto_stride;
+    partial += static_cast<size_t>(img) * n_tau * n_items * (M * M) * NPF;
     out += img * out_stride;
-    constexpr int NPF = P == 2 ? 4 : 1;
-    constexpr int NP = P == 2 ? 4 : 1;
     const int ci = blockIdx.y;
     const int c = chans[ci];
     const bool autosub = !(flags & EPIC_NO_AUTOSUB);
-
-    // A_pq(c) in FP64, reduced in a fixed order (deterministic)
-    __shared__ double red[kThreads / 32][6];
-    __shared__ double apq[6];   // XX, YY, Re XY, Im XY (YX = conj XY)
     const bool ant_kernels = Yauto != nullptr;   // auto image from the per-antenna auto-correlation grid
-    if (autosub && !ant_kernels) {
-        double s[6] = {0, 0, 0, 0, 0, 0};
-        for (int a = threadIdx.x; a < A; a += kThreads) {
-            const int *ia = autoint + (static_cast<size_t>(c) * A + a) * 4;
-            double gxr = 1, gxi = 0, gyr = 1, gyi = 0;
-            if (gains) {
-                const float2 gx = gains[(static_cast<size_t>(c) * A + a) * P];
-                gxr = gx.x;
-                gxi = gx.y;
-                if (P == 2) {
-                    const float2 gy = gains[(static_cast<size_t>(c) * A + a) * P + 1];
-                    gyr = gy.x;
-                    gyi = gy.y;
-                }
-            }
-            s[0] += (gxr * gxr + gxi * gxi) * static_cast<double>(ia[0]);
-            if (P == 2) {
-                s[1] += (gyr * gyr + gyi * gyi) * static_cast<double>(ia[1]);
-                // g_x g_y^* (I_re + i I_im)
-                const double pr = gxr * gyr + gxi * gyi, pi = gxi * gyr - gxr * gyi;
-                s[2] += pr * ia[2] - pi * ia[3];
-                s[3] += pr * ia[3] + pi * ia[2];
-            }
-        }
-        // fixed-order tree: within each warp by shuffles, then the warps' sums by thread 0..3
+
+    __shared__ double red[kThreads / 32][4];
+    __shared__ double apq[4];   // XX, YY, Re XY, Im XY (YX = conj XY)
+    if (autosub && !ant_kernels && !apq_tab) auto_reduce<P>(autoint, 1, 0, gains, A, c, red, apq);
+    float2 aq[NPF];
 #pragma unroll
-        for (int k = 0; k < 4; k++)
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_down_sync(0xffffffffu, s[k], o);
-        if ((threadIdx.x & 31) == 0)
-            for (int k = 0; k < 4; k++) red[threadIdx.x >> 5][k] = s[k];
-        __syncthreads();
-        if (threadIdx.x < 4) {
-            double tot = 0;
-            for (int i = 0; i < kThreads / 32; i++) tot += red[i][threadIdx.x];
-            apq[threadIdx.x] = tot;
-        }
-        __syncthreads();
-    }
+    for (int k = 0; k < NPF; k++)
+        aq[k] = autosub && !ant_kernels ? to_pair(apq_tab ? apq_tab[(static_cast<size_t>(img) * C + c) * 4 + k] : apq[k])
+                                        : make_float2(0.f, 0.f);
 
     const double scale = ((flags & EPIC_MEAN) && T > 0) ? 1.0 / T : 1.0;
-    const int NN = N * N;
-    const int Q = Q1 * Q1;
     float2 *oc = out + out_off[ci];
     for (int pix = blockIdx.x * kThreads + threadIdx.x; pix < NN; pix += gridDim.x * kThreads) {
         const int i = pix / N, j = pix % N;
         const int ly = (i + N / 2) % N, lx = (j + N / 2) % N;   // (i - N/2) mod N
         const int hx = lx % Q1, mx = lx / Q1, hy = ly % Q1, my = ly / Q1;
         const int item = ci * Q + hy * Q1 + hx;
-        const int px = up * (R2 * (mx % R1) + mx / R1), py = up * (R2 * (my % R1) + my / R1);
+        const int px = up * (R1 == 1 ? mx : R2 * (mx % 8) + mx / 8), py = up * (R1 == 1 ? my : R2 * (my % 8) + my / 8);
         const size_t pos = static_cast<size_t>(py) * M + px;
         // time chunks added in time order as compensated FP32 (hi, lo) pairs: TwoSum keeps
-        // hi + lo equal to the exact running sum up to the roundings of lo, far below FP32;
-        // FP64 only for the pair and the auto-term subtraction (FP64 is ~2 ops/clock/SM here)
-        float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
-        auto two_sum = [](float &h, float &l, float x) {
-            const float t = h + x;
-            const float bp = t - h;
-            l += (h - (t - bp)) + (x - bp);
-            h = t;
-        };
+        // hi + lo equal to the exact running sum up to the roundings of lo, far below FP32
+        float2 s[NPF];
+#pragma unroll
+        for (int k = 0; k < NPF; k++) s[k] = make_float2(0.f, 0.f);
         const float *src0 = partial + (static_cast<size_t>(item) * (M * M) + pos) * NPF;
         const size_t tau_stride = static_cast<size_t>(n_items) * (M * M) * NPF;
+#pragma unroll 4
         for (int tau = 0; tau < n_tau; tau++) {
             const float *src = src0 + tau * tau_stride;
             if constexpr (P == 2) {
                 const float4 f = __ldg(reinterpret_cast<const float4 *>(src));
-                two_sum(hi[0], lo[0], f.x);
-                two_sum(hi[1], lo[1], f.y);
-                two_sum(hi[2], lo[2], f.z);
-                two_sum(hi[3], lo[3], f.w);
+                s[0].y += two_sum(s[0].x, f.x);
+                s[1].y += two_sum(s[1].x, f.y);
+                s[2].y += two_sum(s[2].x, f.z);
+                s[3].y += two_sum(s[3].x, f.w);
             } else {
-                two_sum(hi[0], lo[0], __ldg(src));
+                s[0].y += two_sum(s[0].x, __ldg(src));
             }
         }
-        double s[4];
-#pragma unroll
-        for (int k = 0; k < 4; k++) s[k] = static_cast<double>(hi[k]) + static_cast<double>(lo[k]);
-        const double w = wpow[pix];
         if (ant_kernels) {
             if (autosub) {
                 // auto_pq(l) = sum_{rho_y} Y_pq(rho_y, l_x) exp(+2 pi i rho_y l_y / N)
@@ -186,35 +268,53 @@ epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int N
                         axi += y2.x * tw.y + y2.y * tw.x;
                     }
                 }
-                s[0] -= ax;
-                if (P == 2) {
-                    s[1] -= ay;
-                    s[2] -= axr;
-                    s[3] -= axi;
+                const double au[4] = {ax, ay, axr, axi};
+#pragma unroll
+                for (int k = 0; k < NPF; k++) s[k] = to_pair((static_cast<double>(s[k].x) + static_cast<double>(s[k].y)) - au[k]);
+            }
+        } else {
+            const float2 w = __ldg(wpow + pix);
+            if (flags & EPIC_KERNEL_TAPER) {
+                // point-gridded sums: subtract the bare autos, then apply |W^(l)|^2
+#pragma unroll
+                for (int k = 0; k < NPF; k++) {
+                    float2 d = s[k];
+                    d.y += two_sum(d.x, -aq[k].x) - aq[k].y;
+                    const float p = __fmul_rn(d.x, w.x);
+                    s[k] = make_float2(p, fmaf(d.x, w.y, fmaf(d.y, w.x, fmaf(d.x, w.x, -p))));
                 }
-            }
-        } else if (flags & EPIC_KERNEL_TAPER) {
-            // point-gridded sums: subtract the bare autos, then apply |W^(l)|^2
-            for (int k = 0; k < (P == 2 ? 4 : 1); k++) s[k] = (s[k] - (autosub ? apq[k] : 0.0)) * w;
-        } else if (autosub) {
-            s[0] -= apq[0] * w;
-            if (P == 2) {
-                s[1] -= apq[1] * w;
-                s[2] -= apq[2] * w;
-                s[3] -= apq[3] * w;
+            } else if (autosub) {
+#pragma unroll
+                for (int k = 0; k < NPF; k++) pair_msub(s[k], aq[k], w);
             }
         }
-        if (P == 2 && (flags & EPIC_STOKES)) {
-            // I = XX + YY, Q = XX - YY, U = 2 Re XY, V = 2 Im XY
-            const double st[4] = {s[0] + s[1], s[0] - s[1], 2.0 * s[2], 2.0 * s[3]};
-            for (int k = 0; k < 4; k++) oc[k * NN + pix] = make_float2(static_cast<float>(st[k] * scale), 0.f);
-            continue;
+        if constexpr (P == 2) {
+            if (flags & EPIC_STOKES) {
+                // I = XX + YY, Q = XX - YY, U = 2 Re XY, V = 2 Im XY
+                float2 si = s[0], sq = s[0];
+                si.y += two_sum(si.x, s[1].x) + s[1].y;
+                sq.y += two_sum(sq.x, -s[1].x) - s[1].y;
+                s[0] = si;
+                s[1] = sq;
+                s[2] = make_float2(2.f * s[2].x, 2.f * s[2].y);
+                s[3] = make_float2(2.f * s[3].x, 2.f * s[3].y);
+            }
         }
-        oc[pix] = make_float2(static_cast<float>(s[0] * scale), 0.f);
-        if constexpr (NP == 4) {
-            oc[NN + pix] = make_float2(static_cast<float>(s[1] * scale), 0.f);
-            oc[2 * NN + pix] = make_float2(static_cast<float>(s[2] * scale), static_cast<float>(s[3] * scale));
-            oc[3 * NN + pix] = make_float2(static_cast<float>(s[2] * scale), static_cast<float>(-s[3] * scale));
+        float r[NPF];
+#pragma unroll
+        for (int k = 0; k < NPF; k++)
+            r[k] = scale == 1.0 ? s[k].x + s[k].y
+                                : static_cast<float>((static_cast<double>(s[k].x) + static_cast<double>(s[k].y)) * scale);
+        oc[pix] = make_float2(r[0], 0.f);
+        if constexpr (P == 2) {
+            oc[NN + pix] = make_float2(r[1], 0.f);
+            if (flags & EPIC_STOKES) {
+                oc[2 * NN + pix] = make_float2(r[2], 0.f);
+                oc[3 * NN + pix] = make_float2(r[3], 0.f);
+            } else {
+                oc[2 * NN + pix] = make_float2(r[2], r[3]);
+                oc[3 * NN + pix] = make_float2(r[2], -r[3]);
+            }
         }
     }
 }
@@ -284,33 +384,59 @@ auto_rho_kernel(const int *__restrict__ autoint, const float2 *__restrict__ gain
     }
 }
 
-template <int M, int P>
-int launch_epi(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T, int n_tau, float2 *out,
-               cudaStream_t stream)
+// The instantiation for a grid side, its folded side and the polarisations
+template <class F>
+int epi_dispatch(int N, int M, int P, F &&f)
 {
-    const int NN = g.N * g.N;
-    // 8 pixels a thread: fewer blocks, each reducing the channel's auto-power sums once
-    const int tiles = (NN + kThreads * 8 - 1) / (kThreads * 8);
-    const dim3 grid(static_cast<unsigned>(tiles), static_cast<unsigned>(g.n_chan));
-    epilogue_kernel<M, P><<<grid, kThreads, 0, stream>>>(g.d_partial, n_tau, g.n_items, g.N, g.Q1, g.R1, g.R2,
-                                                         g.d_chans,
-                                                         g.d_out_off, g.d_wpow, plan->d_autoint, gains, plan->A, T,
-                                                         plan->flags, out, 0, 0,
-                                                         plan->nker > 1 ? g.d_Y : nullptr, g.d_tw64, plan->K, g.up);
-    return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
+    auto with_p = [&](auto n_, auto m_) {
+        return P == 2 ? f(n_, m_, std::integral_constant<int, 2>{}) : f(n_, m_, std::integral_constant<int, 1>{});
+    };
+    auto side = [&](auto n_, auto m_) { return with_p(n_, m_); };
+#define EPI_SIDE(n, m) \
+    if (N == n && M == m) return side(std::integral_constant<int, n>{}, std::integral_constant<int, m>{})
+    EPI_SIDE(32, 32);
+    EPI_SIDE(32, 64);
+    EPI_SIDE(64, 64);
+    EPI_SIDE(96, 48);
+    EPI_SIDE(128, 64);
+    EPI_SIDE(256, 64);
+    EPI_SIDE(512, 64);
+#undef EPI_SIDE
+    return EPIC_ERR_UNSUPPORTED;
 }
 
-template <int M, int P>
-int launch_epi_raw(const RawImage &r, const float2 *gains, float2 *out, cudaStream_t stream)
+int epi_tiles(int N, int per_thread) { return (N * N + kThreads * per_thread - 1) / (kThreads * per_thread); }
+
+// n_img images of n_tau time chunks each
+int launch_epi(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T, int n_tau, int n_img, float2 *out,
+               cudaStream_t stream)
 {
-    const int NN = r.N * r.N;
-    const int tiles = (NN + kThreads * 4 - 1) / (kThreads * 4);
-    const dim3 grid(static_cast<unsigned>(tiles), static_cast<unsigned>(r.C));
-    epilogue_kernel<M, P><<<grid, kThreads, 0, stream>>>(r.partial, r.n_tau, r.n_items, r.N, r.Q1, 8, M / 8,
-                                                         r.chans,
-                                                         r.out_off, r.wpow, r.autoint, gains, r.A, r.T, r.flags,
-                                                         out, 0, 0, nullptr, nullptr, 0, 1);
-    return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
+    return epi_dispatch(g.N, g.M, plan->P, [&](auto n_, auto m_, auto p_) {
+        constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
+        const dim3 grid(static_cast<unsigned>(epi_tiles(N, 4)), static_cast<unsigned>(g.n_chan), static_cast<unsigned>(n_img));
+        epilogue_kernel<N, M, P><<<grid, kThreads, 0, stream>>>(
+            g.d_partial, n_tau, g.n_items, g.R1, g.R2, g.d_chans, g.d_out_off, g.d_wpow, plan->d_apq, plan->d_autoint, gains,
+            plan->A, plan->C, T, plan->flags, out, static_cast<long long>(plan->out_floats / 2),
+            plan->nker > 1 ? g.d_Y : nullptr, g.d_tw64, plan->K);
+        return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
+    });
+}
+
+template <class F>
+int auto_dispatch(int P, bool words, F &&f)
+{
+    if (P == 2) return words ? f(autopower_kernel<2, true>) : f(autopower_kernel<2, false>);
+    return words ? f(autopower_kernel<1, true>) : f(autopower_kernel<1, false>);
+}
+
+int launch_auto(const uint8_t *v, int T, int C, int A, int P, int chunks, size_t stride, int *autoint, cudaStream_t stream)
+{
+    const bool words = (A * P) % 4 == 0 && reinterpret_cast<uintptr_t>(v) % 4 == 0;
+    const dim3 grid(static_cast<unsigned>(C), static_cast<unsigned>(chunks));
+    return auto_dispatch(P, words, [&](auto kfn) {
+        kfn<<<grid, 128, 0, stream>>>(v, T, C, A, chunks, stride, autoint);
+        return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
+    });
 }
 
 // Per (t, antenna): the FP64 part of the delay phase, once per integration,
@@ -332,65 +458,50 @@ __global__ void delay_prep_kernel(const double *__restrict__ delays, int n, doub
 int launch_autopower_raw(const RawImage &r, const uint8_t *v, int sm_count, cudaStream_t stream)
 {
     if (r.T == 0) return EPIC_OK;
-    int chunks = (4 * sm_count + r.C - 1) / r.C;
-    if (chunks > r.T) chunks = r.T;
-    if (chunks < 1) chunks = 1;
-    const dim3 grid(static_cast<unsigned>(r.C), static_cast<unsigned>(chunks));
-    autopower_kernel<<<grid, kThreads, 0, stream>>>(v, r.T, r.C, r.A, r.P, chunks, 0, r.autoint);
-    return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
+    const int chunks = std::max(1, std::min((4 * sm_count + r.C - 1) / r.C, r.T));
+    return launch_auto(v, r.T, r.C, r.A, r.P, chunks, 0, r.autoint, stream);
 }
 
 int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, cudaStream_t stream)
 {
-    switch (r.M * 4 + r.P) {
-    case 32 * 4 + 1: return launch_epi_raw<32, 1>(r, gains, out, stream);
-    case 32 * 4 + 2: return launch_epi_raw<32, 2>(r, gains, out, stream);
-    case 48 * 4 + 1: return launch_epi_raw<48, 1>(r, gains, out, stream);
-    case 48 * 4 + 2: return launch_epi_raw<48, 2>(r, gains, out, stream);
-    case 64 * 4 + 1: return launch_epi_raw<64, 1>(r, gains, out, stream);
-    case 64 * 4 + 2: return launch_epi_raw<64, 2>(r, gains, out, stream);
-    default: return EPIC_ERR_UNSUPPORTED;
-    }
+    return epi_dispatch(r.N, r.M, r.P, [&](auto n_, auto m_, auto p_) {
+        constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
+        const dim3 grid(static_cast<unsigned>(epi_tiles(N, 4)), static_cast<unsigned>(r.C));
+        epilogue_kernel<N, M, P><<<grid, kThreads, 0, stream>>>(r.partial, r.n_tau, r.n_items, 8, M / 8, r.chans, r.out_off,
+                                                                r.wpow, nullptr, r.autoint, gains, r.A, r.C, r.T, r.flags,
+                                                                out, 0, nullptr, nullptr, 0);
+        return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
+    });
 }
 
-template <int M, int P>
-int launch_epi_series(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int spi, int n_img, float2 *out,
-                      cudaStream_t stream)
+// Time chunks of one integration's auto sums: enough blocks to fill the GPU, at least four samples
+// each, few enough that summing them (auto_sum_kernel, one block a channel) stays short.
+int auto_chunks(const epic_plan_s *plan, int T)
 {
-    const int NN = g.N * g.N;
-    const int tiles = (NN + kThreads * 4 - 1) / (kThreads * 4);
-    const dim3 grid(static_cast<unsigned>(tiles), static_cast<unsigned>(g.n_chan), static_cast<unsigned>(n_img));
-    epilogue_kernel<M, P><<<grid, kThreads, 0, stream>>>(g.d_partial, 1, g.n_items, g.N, g.Q1, g.R1, g.R2, g.d_chans,
-                                                         g.d_out_off, g.d_wpow, plan->d_autoint, gains, plan->A, spi,
-                                                         plan->flags, out,
-                                                         static_cast<size_t>(plan->C) * plan->A * 4,
-                                                         static_cast<long long>(plan->out_floats / 2), nullptr,
-                                                         nullptr, 0, g.up);
+    return std::max(1, std::min({(8 * plan->sm_count + plan->C - 1) / plan->C, T / 4, 32}));
+}
+
+// A_pq of n_img images from the auto sums of chunks chunks each
+static int launch_auto_sum(epic_plan_s *plan, const float2 *gains, int chunks, int n_img, cudaStream_t stream)
+{
+    const dim3 grid(static_cast<unsigned>(plan->C), static_cast<unsigned>(n_img));
+    const size_t stride = static_cast<size_t>(plan->C) * plan->A * 4;
+    if (plan->P == 2) auto_sum_kernel<2><<<grid, kThreads, 0, stream>>>(plan->d_autoint, chunks, stride, gains, plan->A, plan->C, plan->d_apq);
+    else auto_sum_kernel<1><<<grid, kThreads, 0, stream>>>(plan->d_autoint, chunks, stride, gains, plan->A, plan->C, plan->d_apq);
     return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
 }
 
-int launch_autopower_series(epic_plan_s *plan, const uint8_t *v, int spi, int n_img, cudaStream_t stream)
+int launch_autopower_series(epic_plan_s *plan, const uint8_t *v, const float2 *gains, int spi, int n_img, cudaStream_t stream)
 {
     const size_t stride = static_cast<size_t>(plan->C) * plan->A * 4;
-    if (cudaMemsetAsync(plan->d_autoint, 0, stride * n_img * sizeof(int), stream) != cudaSuccess) return EPIC_ERR_CUDA;
-    const dim3 grid(static_cast<unsigned>(plan->C), static_cast<unsigned>(n_img));
-    autopower_kernel<<<grid, kThreads, 0, stream>>>(v, spi * n_img, plan->C, plan->A, plan->P, n_img, stride,
-                                                    plan->d_autoint);
-    return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
+    const int rc = launch_auto(v, spi * n_img, plan->C, plan->A, plan->P, n_img, stride, plan->d_autoint, stream);
+    return rc != EPIC_OK ? rc : launch_auto_sum(plan, gains, 1, n_img, stream);
 }
 
 int launch_epilogue_series(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int spi, int n_img,
                            float2 *out, cudaStream_t stream)
 {
-    switch (g.M * 4 + plan->P) {
-    case 32 * 4 + 1: return launch_epi_series<32, 1>(plan, g, gains, spi, n_img, out, stream);
-    case 32 * 4 + 2: return launch_epi_series<32, 2>(plan, g, gains, spi, n_img, out, stream);
-    case 48 * 4 + 1: return launch_epi_series<48, 1>(plan, g, gains, spi, n_img, out, stream);
-    case 48 * 4 + 2: return launch_epi_series<48, 2>(plan, g, gains, spi, n_img, out, stream);
-    case 64 * 4 + 1: return launch_epi_series<64, 1>(plan, g, gains, spi, n_img, out, stream);
-    case 64 * 4 + 2: return launch_epi_series<64, 2>(plan, g, gains, spi, n_img, out, stream);
-    default: return EPIC_ERR_UNSUPPORTED;
-    }
+    return launch_epi(plan, g, gains, spi, 1, n_img, out, stream);
 }
 
 int launch_delay_prep(epic_plan_s *plan, int T, cudaStream_t stream)
@@ -411,36 +522,22 @@ int launch_auto_rho(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, c
     return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
 }
 
-int launch_autopower(epic_plan_s *plan, const uint8_t *v, int T, cudaStream_t stream)
+int launch_autopower(epic_plan_s *plan, const uint8_t *v, const float2 *gains, int T, cudaStream_t stream)
 {
     const size_t n = static_cast<size_t>(plan->C) * plan->A * 4;
-    if (cudaMemsetAsync(plan->d_autoint, 0, n * sizeof(int), stream) != cudaSuccess) return EPIC_ERR_CUDA;
-    if (T == 0) return EPIC_OK;
-    int chunks = (4 * plan->sm_count + plan->C - 1) / plan->C;
-    if (chunks > T) chunks = T;
-    if (chunks < 1) chunks = 1;
-    const dim3 grid(static_cast<unsigned>(plan->C), static_cast<unsigned>(chunks));
-    autopower_kernel<<<grid, kThreads, 0, stream>>>(v, T, plan->C, plan->A, plan->P, chunks, 0, plan->d_autoint);
-    return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
+    const int chunks = auto_chunks(plan, T);
+    if (plan->nker > 1) {   // the per-antenna auto image takes one sum per antenna
+        if (cudaMemsetAsync(plan->d_autoint, 0, n * sizeof(int), stream) != cudaSuccess) return EPIC_ERR_CUDA;
+        return T == 0 ? EPIC_OK : launch_auto(v, T, plan->C, plan->A, plan->P, chunks, 0, plan->d_autoint, stream);
+    }
+    const int rc = launch_auto(v, T, plan->C, plan->A, plan->P, chunks, n, plan->d_autoint, stream);
+    return rc != EPIC_OK ? rc : launch_auto_sum(plan, gains, chunks, 1, stream);
 }
 
 int launch_epilogue(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T, int n_tau, float2 *out,
                     cudaStream_t stream)
 {
-    if (plan->P == 2) {
-        switch (g.M) {
-        case 32: return launch_epi<32, 2>(plan, g, gains, T, n_tau, out, stream);
-        case 48: return launch_epi<48, 2>(plan, g, gains, T, n_tau, out, stream);
-        case 64: return launch_epi<64, 2>(plan, g, gains, T, n_tau, out, stream);
-        }
-    } else {
-        switch (g.M) {
-        case 32: return launch_epi<32, 1>(plan, g, gains, T, n_tau, out, stream);
-        case 48: return launch_epi<48, 1>(plan, g, gains, T, n_tau, out, stream);
-        case 64: return launch_epi<64, 1>(plan, g, gains, T, n_tau, out, stream);
-        }
-    }
-    return EPIC_ERR_UNSUPPORTED;
+    return launch_epi(plan, g, gains, T, n_tau, 1, out, stream);
 }
 
 }  // namespace epic

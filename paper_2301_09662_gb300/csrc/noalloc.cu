@@ -93,7 +93,7 @@ extern "C" int epic_image_static(const double *ant_xy_m, int n_ant, int n_pol, c
     int rc = host_cell_map(ant_xy_m, n_ant, freq_hz, n_chan, gn.data(), du, K, cells);
     if (rc != EPIC_OK) return rc;
     const int N = grid_n, M = N / Q1, NP = n_pol == 2 ? 4 : 1, NPF = n_pol == 2 ? 4 : 1;
-    std::vector<double> wpow;
+    std::vector<float2> wpow;
     host_kernel_power(kernel_c64, K, N, wpow);
 
     // ---- scratch layout (all offsets 256-byte aligned)
@@ -103,7 +103,7 @@ extern "C" int epic_image_static(const double *ant_xy_m, int n_ant, int n_pol, c
     const size_t o_kernel = off;   off = align256(off + static_cast<size_t>(K) * K * sizeof(float2));
     const size_t o_chans = off;    off = align256(off + static_cast<size_t>(n_chan) * sizeof(int));
     const size_t o_outoff = off;   off = align256(off + static_cast<size_t>(n_chan) * sizeof(long long));
-    const size_t o_wpow = off;     off = align256(off + wpow.size() * sizeof(double));
+    const size_t o_wpow = off;     off = align256(off + wpow.size() * sizeof(float2));
     const size_t o_twN = off;      off = align256(off + static_cast<size_t>(N) * sizeof(float2));
     const size_t table_bytes = off;
     const size_t o_auto = off;     off = align256(off + static_cast<size_t>(n_chan) * n_ant * 4 * sizeof(int));
@@ -132,7 +132,7 @@ extern "C" int epic_image_static(const double *ant_xy_m, int n_ant, int n_pol, c
         chans[c] = c;
         outoff[c] = static_cast<long long>(c) * NP * N * N;
     }
-    std::memcpy(img.data() + o_wpow, wpow.data(), wpow.size() * sizeof(double));
+    std::memcpy(img.data() + o_wpow, wpow.data(), wpow.size() * sizeof(float2));
     auto *tw = reinterpret_cast<float2 *>(img.data() + o_twN);
     for (int k = 0; k < N; k++) {
         const double ang = 2.0 * M_PI * k / N;
@@ -167,7 +167,7 @@ extern "C" int epic_image_static(const double *ant_xy_m, int n_ant, int n_pol, c
     r.kernel = reinterpret_cast<const float2 *>(scratch + o_kernel);
     r.chans = reinterpret_cast<const int *>(scratch + o_chans);
     r.out_off = reinterpret_cast<const long long *>(scratch + o_outoff);
-    r.wpow = reinterpret_cast<const double *>(scratch + o_wpow);
+    r.wpow = reinterpret_cast<const float2 *>(scratch + o_wpow);
     r.twN = reinterpret_cast<const float2 *>(scratch + o_twN);
     r.autoint = reinterpret_cast<int *>(scratch + o_auto);
     r.partial = reinterpret_cast<float *>(scratch + o_partial);

@@ -67,6 +67,7 @@ void free_plan(epic_plan_s *p)
     cudaFree(p->d_dft48);
     cudaFree(p->d_bauto);
     cudaFree(p->d_autoint);
+    cudaFree(p->d_apq);
     cudaFree(p->d_status);
     cudaFree(p->d_dfreq);
     cudaFree(p->d_dtab);
@@ -175,7 +176,16 @@ int host_cell_map(const double *ant_xy_m, int n_ant, const double *freq_hz, int 
     return EPIC_OK;
 }
 
-void host_kernel_power(const float *kern, int K, int N, std::vector<double> &out) { kernel_power(kern, K, N, out); }
+void host_kernel_power(const float *kern, int K, int N, std::vector<float2> &out)
+{
+    std::vector<double> w;
+    kernel_power(kern, K, N, w);
+    out.resize(w.size());
+    for (size_t i = 0; i < w.size(); i++) {
+        const float hi = static_cast<float>(w[i]);
+        out[i] = make_float2(hi, static_cast<float>(w[i] - static_cast<double>(hi)));
+    }
+}
 
 // A kernel's dynamic shared-memory cap holds for the whole process, so it is
 // raised to the most the device allows beside the kernel's static shared
@@ -759,8 +769,8 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
         g.n_items = g.n_chan * g.Q;
         std::vector<long long> offs(g.n_chan);
         for (int i = 0; i < g.n_chan; i++) offs[i] = p->out_off[g.chans[i]];
-        std::vector<double> wpow;
-        kernel_power(kernel_c64, K, g.N, wpow);
+        std::vector<float2> wpow;
+        epic::host_kernel_power(kernel_c64, K, g.N, wpow);
         std::vector<float2> tw(g.N);
         for (int k = 0; k < g.N; k++) {
             const double ang = 2.0 * M_PI * k / g.N;
@@ -943,13 +953,15 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
         for (const auto &g : p->groups) any = any || g.tensor;
         if (!any) rc = EPIC_ERR_UNSUPPORTED;
     }
-    // exact auto sums: one set per image of a series batch (slot 0 for epic_image)
+    // exact auto sums: one set per image of a series batch, or per time chunk of one integration
     p->series_cap = epic::kMaxTau;
     for (const auto &g : p->groups) p->series_cap = std::min(p->series_cap, g.tau_cap);
     p->series_cap = std::max(p->series_cap, 1);
     if (rc == EPIC_OK)
         rc = dev_upload(&p->d_autoint, static_cast<const int *>(nullptr),
-                        static_cast<size_t>(p->series_cap) * n_chan * n_ant * 4);
+                        static_cast<size_t>(std::max(p->series_cap, epic::auto_chunks(p, max_spectra))) * n_chan * n_ant * 4);
+    if (rc == EPIC_OK && !ant_kernels)
+        rc = dev_upload(&p->d_apq, static_cast<const double *>(nullptr), static_cast<size_t>(p->series_cap) * n_chan * 4);
     if (rc == EPIC_OK && tensor) {
         // both 64-point DFT stages on the tensor cores (tc_dual64.cu)
         std::vector<uint16_t> ops;
@@ -993,21 +1005,20 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
             cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&p->ev_auto, cudaEventDisableTiming) != cudaSuccess)
             rc = EPIC_ERR_CUDA;
-        if (p->groups.size() > 1) {
-            for (size_t i = 0; i < p->groups.size() && rc == EPIC_OK; i++) {
-                cudaStream_t st;
-                cudaEvent_t ev;
-                if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
-                    rc = EPIC_ERR_CUDA;
-                    break;
-                }
-                p->side.push_back(st);
-                if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
-                    rc = EPIC_ERR_CUDA;
-                    break;
-                }
-                p->ev_join.push_back(ev);
+        // one branch per group, also for a single one: its imaging runs beside the auto sums
+        for (size_t i = 0; i < p->groups.size() && rc == EPIC_OK; i++) {
+            cudaStream_t st;
+            cudaEvent_t ev;
+            if (cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) != cudaSuccess) {
+                rc = EPIC_ERR_CUDA;
+                break;
             }
+            p->side.push_back(st);
+            if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) != cudaSuccess) {
+                rc = EPIC_ERR_CUDA;
+                break;
+            }
+            p->ev_join.push_back(ev);
         }
     }
     if (rc != EPIC_OK) {
@@ -1091,7 +1102,7 @@ int epic_autotune(epic_plan_t plan, int n_spectra, void *stream)
     const double *saved_delays = plan->delays;
     plan->delays = nullptr;
     const bool autosub = !(plan->flags & EPIC_NO_AUTOSUB);
-    if (rc == EPIC_OK && autosub) rc = epic::launch_autopower(plan, v, n_spectra, s);
+    if (rc == EPIC_OK && autosub) rc = epic::launch_autopower(plan, v, nullptr, n_spectra, s);
     for (auto &g : plan->groups) {
         if (rc != EPIC_OK) break;
         if (g.alias) continue;               // one time chunk, batched by the plan: nothing to tune
@@ -1187,7 +1198,7 @@ int epic_image_series_ex(epic_plan_t plan, const uint8_t *ci4, const float *gain
         const int b = std::min(plan->series_cap, n_img - i0);
         const uint8_t *vb = ci4 + static_cast<size_t>(i0) * spi * row_bytes;
         float2 *ob = out2 + static_cast<size_t>(i0) * (img_floats / 2);
-        if (!(plan->flags & EPIC_NO_AUTOSUB)) rc = epic::launch_autopower_series(plan, vb, spi, b, s);
+        if (!(plan->flags & EPIC_NO_AUTOSUB)) rc = epic::launch_autopower_series(plan, vb, g2, spi, b, s);
         // the batch's delays, time-indexed from the batch's first spectrum like its voltages
         plan->delays = delays_s ? delays_s + static_cast<size_t>(i0) * spi * plan->A : nullptr;
         if (rc == EPIC_OK && plan->delays) rc = epic::launch_delay_prep(plan, spi * b, s);
