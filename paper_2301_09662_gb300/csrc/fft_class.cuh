@@ -50,31 +50,48 @@ constexpr ClassTwiddle<M> make_class_twiddle()
 __constant__ const ClassTwiddle<64> c_cls64 = make_class_twiddle<64>();
 __constant__ const ClassTwiddle<48> c_cls48 = make_class_twiddle<48>();
 
-// x(i), i < n (n <= 64, the same in every lane), from line[i * STRIDE], folded to M and turned for class h
+// x(i), i < 8 nb (nb <= 8, the same in every lane; the positions past the last occupied one are
+// zeros in memory), from line[i * STRIDE], folded to M for class h.  Whole blocks of eight: a test
+// per position took as many instructions as the loads.
 template <int M, int STRIDE>
-__device__ __forceinline__ void class_load(float2 (&x)[M], const float2 *line, int n, int h)
+__device__ __forceinline__ void class_load(float2 (&x)[M], const float2 *line, int nb, int h)
 {
 #pragma unroll
-    for (int i = 0; i < M; i++) x[i] = i < n ? line[i * STRIDE] : make_float2(0.f, 0.f);
+    for (int b = 0; b < M / 8; b++) {
+        if (b < nb) {
+#pragma unroll
+            for (int i = 8 * b; i < 8 * b + 8; i++) x[i] = line[i * STRIDE];
+        } else {
+#pragma unroll
+            for (int i = 8 * b; i < 8 * b + 8; i++) x[i] = make_float2(0.f, 0.f);
+        }
+    }
     if constexpr (M == 48) {
         // w_96^{(i + 48) h} = (-1)^h w_96^{i h}
-        if (n > 48) {
-            const float2 sg = h ? make_float2(-1.f, -1.f) : make_float2(1.f, 1.f);
+        const float2 sg = h ? make_float2(-1.f, -1.f) : make_float2(1.f, 1.f);
 #pragma unroll
-            for (int i = 0; i < 16; i++)
-                if (i + 48 < n) x[i] = pfma(line[(i + 48) * STRIDE], sg, x[i]);
+        for (int b = 0; b < 2; b++) {
+            if (b + 6 < nb) {
+#pragma unroll
+                for (int i = 8 * b; i < 8 * b + 8; i++) x[i] = pfma(line[(i + 48) * STRIDE], sg, x[i]);
+            }
         }
     }
 }
 
 template <int M>
-__device__ __forceinline__ void class_turn(float2 (&x)[M], int h)
+__device__ __forceinline__ void class_turn(float2 (&x)[M], int nb, int h)
 {
     if (h) {
 #pragma unroll
-        for (int i = 1; i < M; i++) {
-            if constexpr (M == 64) x[i] = pfma(pswap(x[i]), c_cls64.ni[i], pmul(x[i], c_cls64.rr[i]));
-            else x[i] = pfma(pswap(x[i]), c_cls48.ni[i], pmul(x[i], c_cls48.rr[i]));
+        for (int b = 0; b < M / 8; b++) {
+            if (b < nb) {
+#pragma unroll
+                for (int i = b ? 8 * b : 1; i < 8 * b + 8; i++) {
+                    if constexpr (M == 64) x[i] = pfma(pswap(x[i]), c_cls64.ni[i], pmul(x[i], c_cls64.rr[i]));
+                    else x[i] = pfma(pswap(x[i]), c_cls48.ni[i], pmul(x[i], c_cls48.rr[i]));
+                }
+            }
         }
     }
 }

@@ -29,13 +29,13 @@
 //    transformed.  G is free as soon as the row transforms hold their inputs.
 //
 // Measured against the per-class kernel (one GB300, whole calls): 256 antennas, 64 channels of
-// 128 x 128, 1000 spectra 5.78 -> 3.20 ms; the same as 25 Stokes images with delays 8.30 -> 5.21 ms;
-// E-field images of 50 spectra 0.535 -> 0.406 ms; per-antenna kernels, 250 spectra 2.55 -> 1.55 ms;
-// 37 channels at 64, 96 and 128 0.67 -> 0.47 ms.  Bound by the transform warps' issue: the FMA
+// 128 x 128, 1000 spectra 5.78 -> 3.10 ms; the same as 25 Stokes images with delays 8.30 -> 3.61 ms;
+// E-field images of 50 spectra 0.535 -> 0.402 ms; per-antenna kernels, 250 spectra 2.55 -> 1.55 ms;
+// 37 channels at 64, 96 and 128 0.67 -> 0.46 ms.  Bound by the transform warps' issue: the FMA
 // pipe is active 51 % of the time (42 % there, for half the work), 8 transform warps an SM.
 //
 // Shared memory: G [P][rows][65], R [P][rows][N + 1], voltages of two samples,
-// gains, tap pairs, the gather lists if they fit (else they are read through L1).
+// gains, taps and gather lists (read through L1 where they do not fit).
 // Side 64 takes two samples at a time, so that its transforms fill the 8 warps.
 #include <algorithm>
 #include <type_traits>
@@ -56,17 +56,21 @@ constexpr int kBarFFT = 1, kBarGrid = 2;      // named barriers of the transform
 constexpr int kPreC = 4;                     // voltage words a gridding thread holds per sample (A P <= 2048)
 constexpr uint16_t kNoCell = 0xFFFFu, kOddRow = 0x8000u;
 
-// Byte offsets of the shared-memory regions.
+// Rows of R: whole blocks of eight (class_load), the last ones zeros.
+__host__ __device__ inline int compact_pad(int rows) { return (rows + 7) & ~7; }
+
+// Byte offsets of the shared-memory regions (taps: with a kernel per antenna, the kernels are staged).
 struct CompactSmem {
     unsigned R, es, gp, taps, tab, total;
 };
-__host__ __device__ inline CompactSmem compact_smem(int P, int TS, int N, int rows, int A, int K, int nker, int words)
+__host__ __device__ inline CompactSmem compact_smem(int P, int TS, int N, int rows, int A, int K, int nker, bool taps,
+                                                    int words)
 {
     auto up = [](unsigned b) { return (b + 15u) & ~15u; };
     CompactSmem s;
     const unsigned planes = static_cast<unsigned>(TS * P * rows);
     s.R = up(planes * kCS * 8u);
-    unsigned r = planes * (N + 1) * 8u;
+    unsigned r = static_cast<unsigned>(TS * P * compact_pad(rows)) * (N + 1) * 8u;
     if (TS == 2) {   // the two samples' time sums are added through R at the end
         const unsigned sum = static_cast<unsigned>(N * N) * (P == 2 ? 16u : 4u);
         r = r > sum ? r : sum;
@@ -74,7 +78,7 @@ __host__ __device__ inline CompactSmem compact_smem(int P, int TS, int N, int ro
     s.es = s.R + up(r);
     s.gp = s.es + up(2u * TS * A * P * 8u);
     s.taps = s.gp + up(static_cast<unsigned>(A * P) * 8u);
-    s.tab = s.taps + (nker > 1 ? up(static_cast<unsigned>(nker * K * K) * 8u)
+    s.tab = s.taps + (nker > 1 ? (taps ? up(static_cast<unsigned>(nker * K * K) * 8u) : 0u)
                                : static_cast<unsigned>(K * (K + 1) + 1) * 8u * 16u);
     s.total = s.tab + up(static_cast<unsigned>(words) * 2u);
     return s;
@@ -94,6 +98,7 @@ struct CompactShape {
     static __device__ __forceinline__ int cls(int task, int k) { return (task + k) % Q; }
 };
 
+// staged: bit 0 the gather lists, bit 1 the antennas' kernels (AK) are in shared memory
 template <int M, int Q, int P, int TS, bool AK, bool EF>
 __global__ void __launch_bounds__(kCThreads, 1)
 fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gains, const float2 *__restrict__ kern,
@@ -110,15 +115,15 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
     // G holds a sample (gridding warps arrive); G has been read, R has been read (transform warps)
     __shared__ __align__(8) uint64_t bar_full, bar_free, bar_read;
     const int AP = A * P, KK = K * K, TPN = K * (K + 1);
-    const CompactSmem L = compact_smem(P, TS, N, rmax, A, K, AK ? A : 1, 0);
+    const CompactSmem L = compact_smem(P, TS, N, rmax, A, K, AK ? A : 1, (staged & 2) != 0, 0);
     float2 *G = reinterpret_cast<float2 *>(smem_c);              // [TS][P][rmax][65]
     float2 *R = reinterpret_cast<float2 *>(smem_c + L.R);        // [TS][P][rmax][N + 1]
     float2 *es = reinterpret_cast<float2 *>(smem_c + L.es);      // [2][TS][A P]
     float2 *gp = reinterpret_cast<float2 *>(smem_c + L.gp);      // [A P]
     float4 *tw2 = reinterpret_cast<float4 *>(smem_c + L.taps);   // [K (K + 1) + 1][8 copies] (one kernel)
-    float2 *tapw = reinterpret_cast<float2 *>(smem_c + L.taps);  // [A][K K] (a kernel per antenna)
+    const float2 *tapw = staged & 2 ? reinterpret_cast<const float2 *>(smem_c + L.taps) : kern;   // [A][K K] (a kernel per antenna)
     uint16_t *stab = reinterpret_cast<uint16_t *>(smem_c + L.tab);
-    const int gplane = rmax * kCS, rplane = rmax * RS;
+    const int gplane = rmax * kCS, rplane = compact_pad(rmax) * RS;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ci = blockIdx.x % n_chan, tau = blockIdx.x / n_chan;
@@ -138,10 +143,13 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
     }
     // ---- set-up: a zero G (the cells no list names stay zero), gains, taps, lists
     for (int i = tid; i < TS * P * gplane; i += kCThreads) G[i] = make_float2(0.f, 0.f);
+    const int rpad = (compact_pad(rows) - rows) * RS;            // R's rows past the channel's stay zero
+    for (int i = tid; i < TS * P * rpad; i += kCThreads) R[(i / rpad) * rplane + rows * RS + i % rpad] = make_float2(0.f, 0.f);
     for (int i = tid; i < AP; i += kCThreads)
         gp[i] = gains ? gains[static_cast<size_t>(c) * AP + i] : make_float2(1.f, 0.f);
     if constexpr (AK) {
-        for (int i = tid; i < A * KK; i += kCThreads) tapw[i] = kern[i];
+        if (staged & 2)
+            for (int i = tid; i < A * KK; i += kCThreads) reinterpret_cast<float2 *>(smem_c + L.taps)[i] = kern[i];
     } else {
         // tap pairs (w(dy, dxl), w(dy, dxl + 1)), zero outside the footprint row; eight interleaved
         // copies, so the eight lanes of one 16-byte request never share a bank group; the last slot
@@ -156,7 +164,7 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
             tw2[i] = make_float4(w[0].x, w[0].y, w[1].x, w[1].y);
         }
     }
-    if (staged)
+    if (staged & 1)
         for (int i = tid; i < ch.y; i += kCThreads) stab[i] = __ldg(ltab + ch.x + i);
     if constexpr (!EF) tc::fence_before_sync();
     __syncthreads();
@@ -200,9 +208,9 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
                 const bool ok = q < rows * P;
                 const int p = ok ? q / rows : 0, y = ok ? q - p * rows : 0;
                 float2 x[M];
-                class_load<M, 1>(x, G + (ts * P + p) * gplane + y * kCS, cols, h);
+                class_load<M, 1>(x, G + (ts * P + p) * gplane + y * kCS, (cols + 7) >> 3, h);
                 if (task + kFW >= n_row) arrive(bar_free);       // this warp has read G
-                class_turn<M>(x, h);
+                class_turn<M>(x, (cols + 7) >> 3, h);
                 float2 *dst = R + (ts * P + p) * rplane + y * RS + h;
                 if (!r_free) {
                     wait(bar_read, ph ^ 1u);                     // the columns of the sample before have been read
@@ -225,9 +233,9 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
                 const int h = S::cls(task, k), blk = (task / Q) % (N / S::CB), ts = task / (Q * (N / S::CB));
                 const int p = lane / S::CB, col = blk * S::CB + lane % S::CB;
                 float2 x[M];
-                class_load<M, RS>(x, R + (ts * P + p) * rplane + col, rows, h);
+                class_load<M, RS>(x, R + (ts * P + p) * rplane + col, (rows + 7) >> 3, h);
                 if (k == last_k) arrive(bar_read);
-                class_turn<M>(x, h);
+                class_turn<M>(x, (rows + 7) >> 3, h);
                 if constexpr (EF) {
                     // F(l) of the corner-based array times w_N^{x0 lx + y0 ly}, on the shifted layout
                     const int4 org = lchan[2 * ci + 1];
@@ -342,7 +350,7 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
         // gather of the warp's batches: [d][32 left-cell offsets, bit 15: odd row, 0xFFFF: empty lane]
         // [d x 32 entries tp << 10 | a]; empty steps name the zero tap slot
         auto gather = [&](int buf) {
-            const uint16_t *bt = (staged ? stab : ltab + ch.x) + my.x;
+            const uint16_t *bt = (staged & 1 ? stab : ltab + ch.x) + my.x;
             auto ld = [](const uint16_t *q) -> uint32_t { return *q; };   // shared or global
             const float2 *e0 = es + buf * TS * AP;
             const uint32_t empty = static_cast<uint32_t>(TPN) << 10;
@@ -552,10 +560,10 @@ template <int M, int Q, int P, int TS, bool AK, bool EF>
 int launch_compact_t(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int n_tau,
                      cudaStream_t stream, float2 *ef_out, long long ef_stride)
 {
-    const CompactSmem L = compact_smem(P, TS, g.N, g.crows, plan->A, plan->K, plan->nker, g.cstage ? g.cwords : 0);
+    const CompactSmem L = compact_smem(P, TS, g.N, g.crows, plan->A, plan->K, plan->nker, g.ctaps, g.cstage ? g.cwords : 0);
     fp32_compact_kernel<M, Q, P, TS, AK, EF><<<static_cast<unsigned>(g.n_chan * n_tau), kCThreads, L.total, stream>>>(
         v, gains, plan->d_kernel, plan->K, g.d_chans, g.d_ltab, g.d_lidx, g.d_lchan, plan->A, plan->C, T, g.n_chan, n_tau,
-        g.crows, g.cstage ? 1 : 0, g.d_partial, plan->d_dfreq, !EF && plan->delays ? plan->d_dtab : nullptr, g.d_twN,
+        g.crows, (g.cstage ? 1 : 0) | (g.ctaps ? 2 : 0), g.d_partial, plan->d_dfreq, !EF && plan->delays ? plan->d_dtab : nullptr, g.d_twN,
         ef_out, g.d_ef_off, ef_stride, plan->d_status, plan->wait_budget);
     return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
 }
@@ -658,14 +666,14 @@ int build_compact_lists(const std::vector<short2> &cells, int A, int K, int P, c
     return EPIC_OK;
 }
 
-size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, int words)
+size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words)
 {
-    return compact_smem(P, N == 64 ? 2 : 1, N, rows, A, K, nker, words).total;
+    return compact_smem(P, N == 64 ? 2 : 1, N, rows, A, K, nker, taps, words).total;
 }
 
 int prepare_compact(const epic_plan_s *plan, const GroupCfg &g)
 {
-    const size_t need = compact_smem_bytes(g.N, plan->P, g.crows, plan->A, plan->K, plan->nker, g.cstage ? g.cwords : 0);
+    const size_t need = compact_smem_bytes(g.N, plan->P, g.crows, plan->A, plan->K, plan->nker, g.ctaps, g.cstage ? g.cwords : 0);
     return compact_dispatch(g, plan->P, [&](auto m_, auto q_, auto p_, auto ts_) {
         constexpr int M = decltype(m_)::value, Q = decltype(q_)::value, P = decltype(p_)::value, TS = decltype(ts_)::value;
         auto both = [&](auto ak) {
