@@ -74,6 +74,7 @@ struct GroupCfg {
     // FP32 plans whose aperture occupies at most 64 x 64 cells: the compact kernel (fp32_compact.cu)
     bool compact = false;
     bool cstage = false;               // its gather lists are staged in shared memory
+    bool ctaps = false;                // and, with a kernel per antenna, the kernels
     int crows = 0, cwords = 0;         // most occupied rows, most list words of a channel
     uint16_t *d_ltab = nullptr;        // device: gather lists (build_compact_lists)
     int2 *d_lidx = nullptr;            // device: [n_chan][gridding warps] (first batch, batches)
@@ -87,6 +88,15 @@ struct GroupCfg {
     short2 *d_j0 = nullptr;            // device: [n_chan] first occupied alias block (x, y)
     uint32_t *d_bseg = nullptr;        // device: footprint rows (a << 8 | dyi) per (channel, 8-row band)
     int *d_boff = nullptr;             // device: [n_chan * 8 + 1] offsets into d_bseg
+    // FP32, grid sides 256 and 512, dual polarisation, at most 128 x 128 occupied cells: rows into a
+    // workspace, then columns (fp32_wide.cu), in groups of wcb channels and batches of wtb samples
+    bool wide = false;
+    bool wgains = false, wforce = false;   // gains staged in shared memory; the path taken for any work (tests)
+    int wrpad = 0, wbands = 0, wstages = 0, wcb = 0, wtb = 0;   // rows kept (padded), bands of 64 rows, tile buffers
+    uint32_t *d_wtab = nullptr;        // device: gather lists (build_wide_lists)
+    int2 *d_widx = nullptr;
+    int4 *d_wchan = nullptr;
+    float2 *d_wws = nullptr;           // device: [wcb][wtb][N / 64][2][64][wrpad] row transforms
     // grid sides 128 and 64 in a tensor plan: the pair kernel (tc_pair128.cu)
     bool pair = false;
     PairSchedule psched;               // how its lists are dealt to the warps (epic_autotune measures a few)
@@ -232,12 +242,22 @@ int build_gather_table(const std::vector<short2> &cells, int A, int K, int M, in
 // FP32 kernel for apertures of at most 64 x 64 cells, grid sides 64, 96, 128 (fp32_compact.cu)
 int build_compact_lists(const std::vector<short2> &cells, int A, int K, int P, const std::vector<int> &chans,
                         std::vector<uint16_t> &tab, std::vector<int2> &idx, std::vector<int4> &chan);
-size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, int words);
+size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words);
 int prepare_compact(const epic_plan_s *plan, const GroupCfg &g);
 int launch_compact(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
                    cudaStream_t stream);
 int launch_compact_efield(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T,
                           float2 *out, long long stride, cudaStream_t stream);
+// FP32 kernels for sides 256 and 512, apertures of at most 128 x 128 cells (fp32_wide.cu)
+int build_wide_lists(const std::vector<short2> &cells, int A, int K, const std::vector<int> &chans, int &bands,
+                     std::vector<uint32_t> &tab, std::vector<int2> &idx, std::vector<int4> &chan, int threads = 0);
+size_t wide_rows_smem_bytes(int A, int K, bool gains);
+bool wide_pays(const epic_plan_s *plan, const GroupCfg &g, int T);
+int wide_stages(int rpad, size_t smem_optin);
+int wide_pick_tau(const GroupCfg &g, int T, int sms);
+int prepare_wide(const epic_plan_s *plan, const GroupCfg &g);
+int launch_wide(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
+                cudaStream_t stream);
 // Register-transform kernels, fold side M = 64 or 48 (fp32_reg64.cu)
 size_t reg64_smem_bytes(int M, int P, int TS, int A, int K, int nker);
 int launch_reg64(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,

@@ -401,6 +401,8 @@ int prepare_fp32(const epic_plan_s *plan, const GroupCfg &g)
 int launch_imaging(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
                    cudaStream_t s)
 {
+    if (g.wide && plan->force_tau == 0 && wide_pays(plan, g, T))
+        return launch_wide(plan, g, v, gains, T, n_tau, s);
     if (g.alias && plan->force_tau == 0) return launch_alias(plan, g, v, gains, T, n_tau, s);
     if (g.tensor && !g.tc_regular) return EPIC_ERR_UNSUPPORTED;   // e.g. an image series: no fold path there
     if (g.tensor) return g.pair ? launch_tc_pair(plan, g, v, gains, T, n_tau, s) : launch_tc_dual(plan, g, v, gains, T, n_tau, s);

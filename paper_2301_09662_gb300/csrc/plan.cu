@@ -112,6 +112,10 @@ void free_plan(epic_plan_s *p)
         cudaFree(g.d_ltab);
         cudaFree(g.d_lidx);
         cudaFree(g.d_lchan);
+        cudaFree(g.d_wtab);
+        cudaFree(g.d_widx);
+        cudaFree(g.d_wchan);
+        cudaFree(g.d_wws);
     }
     delete p;
 }
@@ -812,12 +816,14 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                     g.cwords = std::max(g.cwords, lchan[2 * i].y);
                     g.crows = std::max(g.crows, lchan[2 * i].z);
                 }
-                auto fits = [&](int words) {   // + static shared memory and the system's share
-                    return epic::compact_smem_bytes(g.N, n_pol, g.crows, n_ant, p->K, p->nker, words) + 1024 <=
+                auto fits = [&](bool taps, int words) {   // + static shared memory
+                    return epic::compact_smem_bytes(g.N, n_pol, g.crows, n_ant, p->K, p->nker, taps, words) + 64 <=
                            static_cast<size_t>(smem_optin);
                 };
-                g.compact = fits(0);
-                g.cstage = fits(g.cwords) && !(diag & EPIC_DIAG_GATHER_GLOBAL);
+                // the planes must fit; then the antennas' kernels, then the lists (else through L1)
+                g.compact = fits(false, 0);
+                g.ctaps = p->nker > 1 && fits(true, 0);
+                g.cstage = fits(g.ctaps, g.cwords) && !(diag & EPIC_DIAG_GATHER_GLOBAL);
             }
             if (g.compact) {
                 g.R1 = 1;
@@ -857,12 +863,51 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 if (diag & EPIC_DIAG_GATHER_GLOBAL) g.gstage = false;   // the unstaged form
             }
             if (rc == EPIC_OK) rc = dev_upload(&g.d_rowmask, rows.data(), rows.size());
+            // FP32, sides 256 and 512: rows into a workspace, then columns, where the aperture spans at
+            // most 128 x 128 cells (64 channels of 512 x 512, 2048 antennas, 7 x 7 kernel, 100 spectra:
+            // 6.96 ms against 20.40 on the fold path below); the per-class tables above stay for image
+            // series, E-field images and the smallest integrations (wide_pays)
+            if (rc == EPIC_OK && !tensor && n_pol == 2 && p->nker == 1 && (g.N == 256 || g.N == 512) &&
+                max_spectra > 0 && !(diag & EPIC_DIAG_NO_ALIAS) &&
+                epic::wide_rows_smem_bytes(n_ant, p->K, false) + 64 <= static_cast<size_t>(smem_optin)) {
+                std::vector<uint32_t> wtab;
+                std::vector<int2> widx;
+                std::vector<int4> wchan;
+                const int wrc = epic::build_wide_lists(cells, n_ant, p->K, g.chans, g.wbands, wtab, widx, wchan);
+                if (wrc == EPIC_ERR_NOMEM) rc = wrc;
+                if (wrc == EPIC_OK) {
+                    int rows_max = 0;
+                    for (const int4 &ch : wchan) rows_max = std::max(rows_max, ch.x);
+                    g.wrpad = (rows_max + 15) & ~15;
+                    g.wstages = epic::wide_stages(g.wrpad, static_cast<size_t>(smem_optin));
+                }
+                if (wrc == EPIC_OK && g.wstages > 0) {
+                    // channels per group and samples per batch within the workspace; whole integrations first
+                    const size_t per = static_cast<size_t>(g.N) * 2 * g.wrpad * sizeof(float2);
+                    constexpr size_t kBudget = size_t(4) << 30;
+                    g.wtb = static_cast<int>(std::max<size_t>(1, std::min<size_t>(max_spectra, kBudget / per)));
+                    const int cap_tb = static_cast<int>((diag >> 16) & 255u);   // as for the fold path
+                    if (cap_tb > 0) g.wtb = std::min(g.wtb, cap_tb);
+                    const int most = static_cast<int>(std::max<size_t>(1, kBudget / (per * g.wtb)));
+                    const int n_grp = (g.n_chan + most - 1) / most;
+                    g.wcb = (g.n_chan + n_grp - 1) / n_grp;
+                    g.wide = true;
+                    g.wforce = cap_tb > 0;
+                    g.wgains = epic::wide_rows_smem_bytes(n_ant, p->K, true) + 64 <= static_cast<size_t>(smem_optin);
+                    g.tau_cap = std::max(g.tau_cap, epic::wide_pick_tau(g, max_spectra, p->sm_count));
+                    rc = dev_upload(&g.d_wtab, wtab.data(), wtab.size());
+                    if (rc == EPIC_OK) rc = dev_upload(&g.d_widx, widx.data(), widx.size());
+                    if (rc == EPIC_OK) rc = dev_upload(&g.d_wchan, wchan.data(), wchan.size());
+                    if (rc == EPIC_OK)
+                        rc = dev_upload(&g.d_wws, static_cast<const float2 *>(nullptr), per / sizeof(float2) * g.wcb * g.wtb);
+                }
+            }
             // large sides with one shared kernel of more than one tap: grid once per (channel,
             // sample) and fold all classes (alias_fold.cu), for the FP32 and the two-stage tensor
             // kernel.  With one tap (the taper) re-gridding per class is cheaper than moving the
             // folded grids through HBM (measured at N = 512: 0.24 s against 0.44 s per dense
             // integration).  EPIC_NO_ALIAS=1 keeps the per-class gridding.
-            if (rc == EPIC_OK && fold_ok) {
+            if (rc == EPIC_OK && fold_ok && !g.wide) {
                 std::vector<short2> j0;
                 std::vector<uint32_t> bseg;
                 std::vector<int> boff;
@@ -990,6 +1035,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
         if (rc != EPIC_OK) break;
         if (!g.tensor) rc = epic::prepare_fp32(p, g);
         if (rc == EPIC_OK && g.compact) rc = epic::prepare_compact(p, g);
+        if (rc == EPIC_OK && g.wide) rc = epic::prepare_wide(p, g);
         if (rc == EPIC_OK && g.alias) rc = epic::prepare_alias(p);
     }
     if (rc == EPIC_OK) {
@@ -1105,7 +1151,7 @@ int epic_autotune(epic_plan_t plan, int n_spectra, void *stream)
     if (rc == EPIC_OK && autosub) rc = epic::launch_autopower(plan, v, nullptr, n_spectra, s);
     for (auto &g : plan->groups) {
         if (rc != EPIC_OK) break;
-        if (g.alias) continue;               // one time chunk, batched by the plan: nothing to tune
+        if (g.alias || g.wide) continue;     // time chunks set by the plan: nothing to tune
         const int cap = std::max(1, std::min(g.tau_cap, n_spectra));
         std::vector<int> cand;
         auto add = [&](int n) {
