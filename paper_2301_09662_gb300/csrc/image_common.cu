@@ -196,6 +196,7 @@ __global__ void __launch_bounds__(kThreads)
 epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R1, int R2,
                 const int *__restrict__ chans, const long long *__restrict__ out_off,
                 const float2 *__restrict__ wpow, const double *__restrict__ apq_tab, const int *__restrict__ autoint,
+                int auto_n, size_t auto_stride,
                 const float2 *__restrict__ gains, int A, int C, int T, unsigned flags, float2 *__restrict__ out,
                 long long out_stride, const double2 *__restrict__ Yauto, const double2 *__restrict__ tw64, int K)
 {
@@ -213,7 +214,8 @@ epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R
 
     __shared__ double red[kThreads / 32][4];
     __shared__ double apq[4];   // XX, YY, Re XY, Im XY (YX = conj XY)
-    if (autosub && !ant_kernels && !apq_tab) auto_reduce<P>(autoint, 1, 0, gains, A, c, red, apq);
+    if (autosub && !ant_kernels && !apq_tab)
+        auto_reduce<P>(autoint + static_cast<size_t>(img) * auto_n * auto_stride, auto_n, auto_stride, gains, A, c, red, apq);
     float2 aq[NPF];
 #pragma unroll
     for (int k = 0; k < NPF; k++)
@@ -236,7 +238,7 @@ epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R
         for (int k = 0; k < NPF; k++) s[k] = make_float2(0.f, 0.f);
         const float *src0 = partial + (static_cast<size_t>(item) * (M * M) + pos) * NPF;
         const size_t tau_stride = static_cast<size_t>(n_items) * (M * M) * NPF;
-#pragma unroll 4
+#pragma unroll 8
         for (int tau = 0; tau < n_tau; tau++) {
             const float *src = src0 + tau * tau_stride;
             if constexpr (P == 2) {
@@ -405,18 +407,30 @@ int epi_dispatch(int N, int M, int P, F &&f)
     return EPIC_ERR_UNSUPPORTED;
 }
 
-int epi_tiles(int N, int per_thread) { return (N * N + kThreads * per_thread - 1) / (kThreads * per_thread); }
+// Pixel tiles: four pixels a thread, one where that would leave SMs idle.
+int epi_tiles(int N, int images, int sms)
+{
+    const int one = (N * N + kThreads - 1) / kThreads, four = (one + 3) / 4;
+    return four * images >= 4 * sms ? four : one;
+}
 
-// n_img images of n_tau time chunks each
-int launch_epi(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T, int n_tau, int n_img, float2 *out,
-               cudaStream_t stream)
+// A_pq summed by the epilogue's own blocks (small arrays: the sums are shorter than a launch) or by
+// auto_sum_kernel.  16 antennas, 4 channels of 32 x 32, 64 spectra, whole
+// call: 26.4 us with the extra kernel, 18.6 us without it and with one pixel a thread.
+bool auto_in_epilogue(const epic_plan_s *plan) { return plan->A <= 64; }
+
+// n_img images of n_tau time chunks each, their auto sums in auto_n chunks each
+int launch_epi(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T, int n_tau, int n_img, int auto_n,
+               float2 *out, cudaStream_t stream)
 {
     return epi_dispatch(g.N, g.M, plan->P, [&](auto n_, auto m_, auto p_) {
         constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
-        const dim3 grid(static_cast<unsigned>(epi_tiles(N, 4)), static_cast<unsigned>(g.n_chan), static_cast<unsigned>(n_img));
+        const dim3 grid(static_cast<unsigned>(epi_tiles(N, g.n_chan * n_img, plan->sm_count)), static_cast<unsigned>(g.n_chan),
+                        static_cast<unsigned>(n_img));
         epilogue_kernel<N, M, P><<<grid, kThreads, 0, stream>>>(
-            g.d_partial, n_tau, g.n_items, g.R1, g.R2, g.d_chans, g.d_out_off, g.d_wpow, plan->d_apq, plan->d_autoint, gains,
-            plan->A, plan->C, T, plan->flags, out, static_cast<long long>(plan->out_floats / 2),
+            g.d_partial, n_tau, g.n_items, g.R1, g.R2, g.d_chans, g.d_out_off, g.d_wpow,
+            auto_in_epilogue(plan) ? nullptr : plan->d_apq, plan->d_autoint, auto_n, static_cast<size_t>(plan->C) * plan->A * 4,
+            gains, plan->A, plan->C, T, plan->flags, out, static_cast<long long>(plan->out_floats / 2),
             plan->nker > 1 ? g.d_Y : nullptr, g.d_tw64, plan->K);
         return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
     });
@@ -466,9 +480,9 @@ int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, cud
 {
     return epi_dispatch(r.N, r.M, r.P, [&](auto n_, auto m_, auto p_) {
         constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
-        const dim3 grid(static_cast<unsigned>(epi_tiles(N, 4)), static_cast<unsigned>(r.C));
+        const dim3 grid(static_cast<unsigned>(epi_tiles(N, r.C, 148)), static_cast<unsigned>(r.C));
         epilogue_kernel<N, M, P><<<grid, kThreads, 0, stream>>>(r.partial, r.n_tau, r.n_items, 8, M / 8, r.chans, r.out_off,
-                                                                r.wpow, nullptr, r.autoint, gains, r.A, r.C, r.T, r.flags,
+                                                                r.wpow, nullptr, r.autoint, 1, 0, gains, r.A, r.C, r.T, r.flags,
                                                                 out, 0, nullptr, nullptr, 0);
         return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
     });
@@ -478,12 +492,13 @@ int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, cud
 // each, few enough that summing them (auto_sum_kernel, one block a channel) stays short.
 int auto_chunks(const epic_plan_s *plan, int T)
 {
-    return std::max(1, std::min({(8 * plan->sm_count + plan->C - 1) / plan->C, T / 4, 32}));
+    return std::max(1, std::min({(8 * plan->sm_count + plan->C - 1) / plan->C, T / 4, plan->A <= 64 ? 8 : 32}));
 }
 
 // A_pq of n_img images from the auto sums of chunks chunks each
 static int launch_auto_sum(epic_plan_s *plan, const float2 *gains, int chunks, int n_img, cudaStream_t stream)
 {
+    if (auto_in_epilogue(plan)) return EPIC_OK;
     const dim3 grid(static_cast<unsigned>(plan->C), static_cast<unsigned>(n_img));
     const size_t stride = static_cast<size_t>(plan->C) * plan->A * 4;
     if (plan->P == 2) auto_sum_kernel<2><<<grid, kThreads, 0, stream>>>(plan->d_autoint, chunks, stride, gains, plan->A, plan->C, plan->d_apq);
@@ -501,7 +516,7 @@ int launch_autopower_series(epic_plan_s *plan, const uint8_t *v, const float2 *g
 int launch_epilogue_series(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int spi, int n_img,
                            float2 *out, cudaStream_t stream)
 {
-    return launch_epi(plan, g, gains, spi, 1, n_img, out, stream);
+    return launch_epi(plan, g, gains, spi, 1, n_img, 1, out, stream);
 }
 
 int launch_delay_prep(epic_plan_s *plan, int T, cudaStream_t stream)
@@ -537,7 +552,7 @@ int launch_autopower(epic_plan_s *plan, const uint8_t *v, const float2 *gains, i
 int launch_epilogue(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T, int n_tau, float2 *out,
                     cudaStream_t stream)
 {
-    return launch_epi(plan, g, gains, T, n_tau, 1, out, stream);
+    return launch_epi(plan, g, gains, T, n_tau, 1, auto_chunks(plan, T), out, stream);
 }
 
 }  // namespace epic
