@@ -308,23 +308,42 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
-def tensor_roofline(wl, form, img_ms, peaks, pair=True):
+def occupied_k_blocks(wl, c, fold, K):
+    """16-deep k-blocks of the folded side that hold occupied columns and rows of
+    channel c (the pair kernel leaves the others out); all of them for a workload
+    without geometry."""
+    if getattr(wl, "ant_xy", None) is None:
+        return fold // 16, fold // 16
+    import numpy as np
+    x = (np.asarray(wl.ant_xy) - np.mean(wl.ant_xy, axis=0)) * wl.freq_hz[c] / (299792458.0 * wl.du)
+    cell = np.sign(x) * np.floor(np.abs(x) + 0.5)
+    span = np.minimum(cell.max(axis=0) - cell.min(axis=0) + K, fold)
+    return int(math.ceil(span[0] / 16)), int(math.ceil(span[1] / 16))
+
+
+def tensor_roofline(wl, form, img_ms, peaks, pair=True, taper=False):
     """Executed tensor FLOPs of the tensor-core imaging launch over its time.
     Each 64-point DFT stage of one sample is 8 k-blocks x terms MMAs of
-    128 x 128 x 16 (a side-96 48-point stage skips 2 of the 8 k-blocks).
-    Grid sides 128 and 96 run two pixel classes per CTA from one row stage
-    (pair kernel): 3 stage GEMMs per two classes; other sides (and these with
-    EPIC_DIAG_NO_PAIR): 2 per class.  Also the method's algorithmic FLOPs (the
-    FP32 FFT form's count) over the same time."""
+    128 x 128 x 16, of which the pair kernel (grid sides 128, 96 and 64) issues
+    those with occupied columns (row stage) or rows (column stages).  Sides 128
+    and 96 run two CTAs per channel, each a row stage and two column stages; side
+    64 one CTA, a row and a column stage; other sides (and these with
+    EPIC_DIAG_NO_PAIR) 2 stages per class.  Also the method's algorithmic FLOPs
+    (the FP32 FFT form's count) over the same time."""
     terms = 1 if form == "tc_fp16" else 3
     stage = 8 * terms * 2.0 * 128 * 128 * 16          # one 64-point stage: 8 k-blocks x terms MMAs
+    K = 1 if taper else wl.K
     stages = 0.0
-    for n in wl.grid_n:
+    for c, n in enumerate(wl.grid_n):
         n = int(n)
-        fold = 48 if n == 96 else 64                    # side 96: 48-point DFTs, 6 of the 8 k-blocks
+        fold = 48 if n == 96 else 64                    # side 96: 48-point DFTs
         classes = max(1, n // fold) ** 2
-        per_class = 1.5 if (pair and n in (128, 96)) else 2.0
-        stages += classes * per_class * (6.0 / 8.0 if n == 96 else 1.0)
+        if pair and n in (128, 96, 64):
+            kx, ky = occupied_k_blocks(wl, c, fold, K)
+            ctas = 1 if n == 64 else 2
+            stages += ctas * (2 * kx + ctas * 2 * ky) / 8.0
+        else:
+            stages += classes * 2.0 * (6.0 / 8.0 if n == 96 else 1.0)
     flops = stages * wl.T * stage
     ach = flops / (img_ms / 1e3) / 1e12
     peak = float(peaks.get("bf16_tflops", 1892.1))
@@ -462,7 +481,7 @@ def time_variants(wl, v, g, out, flush, args, stream):
             img = max((x for k, x in stages.items() if k.startswith("image[")), default=None)
             if img:
                 entry["roofline"] = tensor_roofline(wl, name.replace("_taper", "").replace("_one_class", ""), img,
-                                                    peaks, pair=name != "tc_split_fp16_one_class")
+                                                    peaks, pair=name != "tc_split_fp16_one_class", taper="_taper" in name)
         if name == "fp32" and stages:
             entry["roofline"] = fp32_roofline(wl, stages, peaks, sm_count)
             entry["roofline"]["traffic"] = ncu_record(NCU_TRAFFIC, "lwa", "fp32")

@@ -109,6 +109,9 @@ struct GroupCfg {
     uint16_t *d_ptab = nullptr;        // device: pair-kernel gather lists (build_pair_tables)
     int2 *d_pchan = nullptr;           // device: [n_chan] (block start, block words)
     int4 *d_pidx = nullptr;            // device: [n_chan][8 warps] (half 1 offset, batches, half 2 offset, batches)
+    std::vector<short2> h_pcells;      // host: [C][A] cells moved to the aperture's corner (pair_origin)
+    short2 *d_pcells = nullptr;        // device copy
+    int2 *d_pkblk = nullptr;           // device: [n_chan] 16-deep k-blocks with occupied columns, rows
     unsigned long long *d_upper = nullptr;  // device: [n_chan] folded rows whose cells lie in unfolded rows 64..127
     long long *d_ef_off = nullptr;     // device (E-field images): per group channel, complex offset within a sample
 };
@@ -164,7 +167,6 @@ struct epic_plan_s {
     void *g_out = nullptr;
     int g_T = -1;
     bool g_prof = false;
-    std::vector<short2> h_cells;       // host copy of the cell map, kept when a group uses the pair kernel
     // host-buffer entry point staging (allocated on first use)
     uint8_t *d_stage_v = nullptr;
     float *d_stage_g = nullptr;
@@ -224,6 +226,8 @@ int launch_tc_dual_fold(epic_plan_s *plan, const GroupCfg &g, const float2 *gain
 int launch_tc_dual(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
                    cudaStream_t stream);
 // grid sides 128 and 64: the gather-gridding pair kernel (tc_pair128.cu)
+void pair_origin(const std::vector<short2> &cells, int A, int K, const std::vector<int> &chans, int M,
+                 std::vector<short2> &moved, std::vector<int2> &kblk);
 int build_pair_tables(const std::vector<short2> &cells, int A, int K, const std::vector<int> &chans,
                       const std::vector<uint32_t> &tab32, const std::vector<int4> &idx32,
                       const std::vector<int2> &chan32, std::vector<uint16_t> &tab, std::vector<int4> &idx,

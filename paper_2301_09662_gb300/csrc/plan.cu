@@ -108,6 +108,8 @@ void free_plan(epic_plan_s *p)
         cudaFree(g.d_pchan);
         cudaFree(g.d_pidx);
         cudaFree(g.d_upper);
+        cudaFree(g.d_pcells);
+        cudaFree(g.d_pkblk);
         cudaFree(g.d_ef_off);
         cudaFree(g.d_ltab);
         cudaFree(g.d_lidx);
@@ -938,9 +940,12 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 std::vector<int2> chan32, pchan;
                 std::vector<unsigned long long> rows32, upper;
                 std::vector<uint16_t> ptab;
-                if (epic::build_gather_table(cells, n_ant, p->K, g.M, 2, g.chans, tab32, idx32, chan32, rows32) ==
+                std::vector<short2> pcells;
+                std::vector<int2> pkblk;
+                epic::pair_origin(cells, n_ant, p->K, g.chans, g.M, pcells, pkblk);
+                if (epic::build_gather_table(pcells, n_ant, p->K, g.M, 2, g.chans, tab32, idx32, chan32, rows32) ==
                         EPIC_OK &&
-                    epic::build_pair_tables(cells, n_ant, p->K, g.chans, tab32, idx32, chan32, ptab, pidx, pchan,
+                    epic::build_pair_tables(pcells, n_ant, p->K, g.chans, tab32, idx32, chan32, ptab, pidx, pchan,
                                             upper, epic::PairSchedule(), g.M) == EPIC_OK) {
                     int words = 0;
                     for (const int2 &ch : pchan) words = std::max(words, ch.y);
@@ -954,10 +959,12 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                         g.h_tab32 = std::move(tab32);
                         g.h_idx32 = std::move(idx32);
                         g.h_chan32 = std::move(chan32);
-                        if (p->h_cells.empty()) p->h_cells = cells;
                         g.ptab_n = ptab.size();
                         g.pidx_n = pidx.size();
+                        g.h_pcells = std::move(pcells);
                         rc = dev_upload(&g.d_ptab, ptab.data(), ptab.size());
+                        if (rc == EPIC_OK) rc = dev_upload(&g.d_pcells, g.h_pcells.data(), g.h_pcells.size());
+                        if (rc == EPIC_OK) rc = dev_upload(&g.d_pkblk, pkblk.data(), pkblk.size());
                         if (rc == EPIC_OK) rc = dev_upload(&g.d_pidx, pidx.data(), pidx.size());
                         if (rc == EPIC_OK) rc = dev_upload(&g.d_pchan, pchan.data(), pchan.size());
                         if (rc == EPIC_OK) rc = dev_upload(&g.d_upper, upper.data(), upper.size());
@@ -1117,7 +1124,7 @@ int repack_pair(epic_plan_s *plan, epic::GroupCfg &g, const epic::PairSchedule &
     std::vector<int2> pchan;
     std::vector<unsigned long long> upper;
     std::vector<uint16_t> ptab;
-    int rc = epic::build_pair_tables(plan->h_cells, plan->A, plan->K, g.chans, g.h_tab32, g.h_idx32, g.h_chan32,
+    int rc = epic::build_pair_tables(g.h_pcells, plan->A, plan->K, g.chans, g.h_tab32, g.h_idx32, g.h_chan32,
                                      ptab, pidx, pchan, upper, ps, g.M);
     if (rc != EPIC_OK) return rc;
     if (ptab.size() != g.ptab_n || pidx.size() != g.pidx_n) return EPIC_ERR_UNSUPPORTED;

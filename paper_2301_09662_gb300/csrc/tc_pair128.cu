@@ -167,7 +167,7 @@ tc_pair128_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gain
                   const short2 *__restrict__ cells, const float2 *__restrict__ kern, int K,
                   const int *__restrict__ chans, const float2 *__restrict__ twN,
                   const uint16_t *__restrict__ ptab, const int2 *__restrict__ pchan, const int4 *__restrict__ pidx,
-                  const unsigned long long *__restrict__ upper,
+                  const unsigned long long *__restrict__ upper, const int2 *__restrict__ kblk,
                   const uint8_t *__restrict__ dft_ops, int A, int C, int T, int n_items_out, int n_tau,
                   float *__restrict__ partial, int *__restrict__ status, long long wait_budget, int withhold_mma,
                   const float *__restrict__ dfreq, const float4 *__restrict__ dtab)
@@ -208,6 +208,7 @@ tc_pair128_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gain
     const int t0 = static_cast<int>(static_cast<long long>(T) * tau / n_tau);
     const int t1 = static_cast<int>(static_cast<long long>(T) * (tau + 1) / n_tau);
     const int2 my_chan = pchan[ci];
+    const int2 nk = kblk[ci];                    // 16-deep k-blocks that hold occupied columns (x) and rows (y)
 
     if (warp == 0) tc::tmem_alloc(&tmem_slot, 512);
     if (tid == 0) {
@@ -334,7 +335,7 @@ tc_pair128_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gain
                 if (!withhold_mma) {
 #pragma unroll
                     for (int kb = 0; kb < 8; kb++) {
-                        if (MF < 64 && (kb & 3) * 16 >= MF) continue;   // k beyond the folded side: zeros
+                        if ((kb & 3) >= nk.x) continue;   // no occupied column: zeros
                         const uint64_t g_hi = tc::smem_desc(g_base + kb * 256, kLBO, kSBO);
                         const uint64_t x_hi = tc::smem_desc(x_base + kb * 256, kLBO, kSBO);
                         tc::mma_f16(taddr + col_r(t), g_hi, x_hi, idesc_row, kb > 0 ? 1u : 0u);
@@ -365,7 +366,7 @@ tc_pair128_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gain
                         const uint32_t d2 = taddr + (hy ? col_r(t) : col_a(t));
 #pragma unroll
                         for (int kb = 0; kb < 8; kb++) {
-                            if (MF < 64 && (kb & 3) * 16 >= MF) continue;
+                            if ((kb & 3) >= nk.y) continue;   // no occupied row: zeros
                             const uint64_t h_hi = tc::smem_desc(h_base + kb * 256, kLBO, kSBO);
                             const uint64_t h_lo = tc::smem_desc(h_base + kPart + kb * 256, kLBO, kSBO);
                             if (hy == 0) {
@@ -687,6 +688,31 @@ const void *pair_kernel(int cls, int mf)
 }
 
 }  // namespace
+
+// Cells of the group's channels moved so that the first occupied column and row are 0, and per
+// channel the 16-deep k-blocks of the folded side that then hold occupied columns and rows.  The move
+// multiplies F(l) by one unit factor common to both polarisations, which cancels in every product;
+// an aperture that occupies 48 of 64 folded rows then leaves a k-block of zeros out of every column
+// stage (and out of the row stages by its columns), wherever on the grid it lies.
+void pair_origin(const std::vector<short2> &cells, int A, int K, const std::vector<int> &chans, int M,
+                 std::vector<short2> &moved, std::vector<int2> &kblk)
+{
+    const int h = (K - 1) / 2;
+    moved = cells;
+    kblk.assign(chans.size(), make_int2(M / 16, M / 16));
+    for (size_t ci = 0; ci < chans.size(); ci++) {
+        short2 *cc = moved.data() + static_cast<size_t>(chans[ci]) * A;
+        int x0 = 1 << 20, x1 = -1, y0 = 1 << 20, y1 = -1;
+        for (int a = 0; a < A; a++) {
+            x0 = std::min(x0, cc[a].x - h);
+            x1 = std::max(x1, cc[a].x + h);
+            y0 = std::min(y0, cc[a].y - h);
+            y1 = std::max(y1, cc[a].y + h);
+        }
+        for (int a = 0; a < A; a++) cc[a] = make_short2(static_cast<short>(cc[a].x - x0), static_cast<short>(cc[a].y - y0));
+        kblk[ci] = make_int2((std::min(x1 - x0 + 1, M) + 15) / 16, (std::min(y1 - y0 + 1, M) + 15) / 16);
+    }
+}
 
 // The gather lists of the pair kernel, rebuilt from the FP32 kernel's table of
 // the same channels (build_gather_table, fold side 64, dual polarisation: per
@@ -1080,8 +1106,8 @@ int launch_tc_pair(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const
         constexpr int V = decltype(vv)::value;
         auto kfn = cls == 1 ? tc_pair128_kernel<V, 1, 64> : g.M == 48 ? tc_pair128_kernel<V, 2, 48> : tc_pair128_kernel<V, 2, 64>;
         kfn<<<grid, kPairThreads, smem, stream>>>(
-            v, gains, plan->d_cells, plan->d_kernel, plan->K, g.d_chans, g.d_twN, g.d_ptab, g.d_pchan, g.d_pidx,
-            g.d_upper, dft, plan->A, plan->C, T, g.n_items, n_tau, g.d_partial, plan->d_status,
+            v, gains, g.d_pcells, plan->d_kernel, plan->K, g.d_chans, g.d_twN, g.d_ptab, g.d_pchan, g.d_pidx,
+            g.d_upper, g.d_pkblk, dft, plan->A, plan->C, T, g.n_items, n_tau, g.d_partial, plan->d_status,
             plan->wait_budget, plan->test_withhold_mma, plan->d_dfreq, plan->delays ? plan->d_dtab : nullptr);
         return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
     });
