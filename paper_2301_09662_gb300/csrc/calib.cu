@@ -16,8 +16,8 @@
 // E conj(e) to the sums of their own antennas in registers, so an iteration reads the voltages
 // once.  The CTAs' sums meet through distributed shared memory: each CTA finishes a slice of the
 // antennas and hands its gains to the others, so there is no workspace and one launch.  Bound by
-// issue (about 20 instructions a voltage and iteration).  256 antennas, 64 channels, two
-// polarisations, 1000 spectra, two iterations: 96 us, against 322 us for one CTA per channel and
+// issue and latency (packed pairs: about 12 instructions a voltage and iteration; 36 % issue).  256 antennas, 64 channels, two
+// polarisations, 1000 spectra, two iterations: 91 us, against 322 us for one CTA per channel and
 // polarisation, whose loads' latency was the limit.
 // gain_solve_kernel (larger arrays): one CTA per (channel, polarisation), E(t) of all samples in
 // shared memory, the voltages read twice per iteration.
@@ -134,24 +134,23 @@ gain_solve_kernel(const uint8_t *__restrict__ v, const short2 *__restrict__ cell
 
 constexpr int kCalWarps = kCalThreads / 32;
 
-// Byte b of four 4+4-bit voltages x (as ci4_decode), two instructions a part: with the sign bits
-// flipped a nibble is n + 8 in 0..15; or-ed into the mantissa of 2^23 at bit s it reads
-// 2^23 + (n + 8) 2^s, and one FMA takes the offset and the scale away, exactly.
-struct Ci4Word {
-    uint32_t lo, hi;
-    __device__ __forceinline__ explicit Ci4Word(uint32_t x) : lo(x ^ 0x88888888u), hi(lo >> 16) {}
-    template <int S>
-    static __device__ __forceinline__ float part(uint32_t y)
-    {
-        const float m = __uint_as_float((y & (0xFu << S)) | 0x4B000000u);
-        return fmaf(m, 1.f / static_cast<float>(1 << S), -(8388608.f / static_cast<float>(1 << S) + 8.f));
-    }
-    __device__ __forceinline__ float2 get(int b) const
-    {
-        const uint32_t y = b & 2 ? hi : lo;
-        return b & 1 ? make_float2(part<12>(y), part<8>(y)) : make_float2(part<4>(y), part<0>(y));
-    }
+// Bytes 2 k and 2 k + 1 of four 4+4-bit voltages x (as ci4_decode) as pairs (re, re), (im, im): with the
+// sign bits flipped a nibble is n + 8 in 0..15; or-ed into the mantissa of 2^23 at bit s it reads
+// 2^23 + (n + 8) 2^s, and one packed FMA takes the offsets and the scales away, exactly.
+struct Ci4Pair {
+    float2 re, im;
 };
+__device__ __forceinline__ Ci4Pair ci4_pair(uint32_t x, int k)
+{
+    const uint32_t y = (k ? x >> 16 : x) ^ 0x8888u;
+    auto bits = [&](int s) { return __uint_as_float((y & (0xFu << s)) | 0x4B000000u); };
+    constexpr float o0 = -(8388608.f + 8.f), o4 = -(8388608.f / 16.f + 8.f), o8 = -(8388608.f / 256.f + 8.f),
+                    o12 = -(8388608.f / 4096.f + 8.f);
+    Ci4Pair e;
+    e.re = pfma(make_float2(bits(4), bits(12)), make_float2(1.f / 16.f, 1.f / 4096.f), make_float2(o4, o12));
+    e.im = pfma(make_float2(bits(0), bits(8)), make_float2(1.f, 1.f / 256.f), make_float2(o0, o8));
+    return e;
+}
 
 size_t cal_cluster_smem(int AP)   // sums of every warp, the CTA's sums, gains, phases, sum |e|^2
 {
@@ -223,73 +222,75 @@ gain_solve_cluster_kernel(const uint8_t *__restrict__ v, const short2 *__restric
     // exactly: at most 128 a sample, far fewer than 2^17 samples a warp)
     auto sweep = [&](auto first) {
         constexpr bool FIRST = decltype(first)::value;
-        // w = g conj(phi) of the lane's values
-        float2 w[R][4], num[R][4];
-        float dd[FIRST ? R : 1][4];
+        // w = g conj(phi) of the lane's values, two bytes (both polarisations, or two antennas) to a packed pair
+        float2 wr[R][2], wi[R][2], wn[R][2], nr[R][2], ni[R][2];
+        float2 dd[FIRST ? R : 1][2];
+        const float2 zero = make_float2(0.f, 0.f);
 #pragma unroll
         for (int r = 0; r < R; r++)
 #pragma unroll
-            for (int b = 0; b < 4; b++) {
-                const int i = 4 * (lane + 32 * r) + b;
-                w[r][b] = i < AP ? cmul(g[i], make_float2(phi[i].x, -phi[i].y)) : make_float2(0.f, 0.f);
-                num[r][b] = make_float2(0.f, 0.f);
-                if (FIRST) dd[r][b] = 0.f;
+            for (int k = 0; k < 2; k++) {
+                float2 w[2];
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    const int i = 4 * (lane + 32 * r) + 2 * k + u;
+                    w[u] = i < AP ? cmul(g[i], make_float2(phi[i].x, -phi[i].y)) : zero;
+                }
+                wr[r][k] = make_float2(w[0].x, w[1].x);
+                wi[r][k] = make_float2(w[0].y, w[1].y);
+                wn[r][k] = make_float2(-w[0].y, -w[1].y);
+                nr[r][k] = ni[r][k] = zero;
+                if (FIRST) dd[r][k] = zero;
             }
         uint32_t x[R], xn[R];
         load(rank * kCalWarps + warp, x);
         for (int t = rank * kCalWarps + warp; t < T; t += step) {
             load(t + step, xn);
-            // polarisation of value i = i mod P: with P = 2 the byte's parity
-            float2 e0 = make_float2(0.f, 0.f), e1 = make_float2(0.f, 0.f);
+            // the halves of a pair: polarisations 0 and 1 (P = 2), or antennas of one polarisation
+            float2 er = zero, ei = zero;
 #pragma unroll
-            for (int r = 0; r < R; r++) {
-                const Ci4Word cw(x[r]);
+            for (int r = 0; r < R; r++)
 #pragma unroll
-                for (int b = 0; b < 4; b++) {
-                    const float2 e = cw.get(b);
-                    float2 &o = (b & 1) ? e1 : e0;
-                    o.x = fmaf(w[r][b].x, e.x, fmaf(-w[r][b].y, e.y, o.x));
-                    o.y = fmaf(w[r][b].x, e.y, fmaf(w[r][b].y, e.x, o.y));
+                for (int k = 0; k < 2; k++) {
+                    const Ci4Pair e = ci4_pair(x[r], k);
+                    er = pfma(wr[r][k], e.re, pfma(wn[r][k], e.im, er));
+                    ei = pfma(wr[r][k], e.im, pfma(wi[r][k], e.re, ei));
                 }
-            }
             if (P == 1) {
-                e0 = cadd(e0, e1);
-                e1 = e0;
+                er = make_float2(er.x + er.y, er.x + er.y);
+                ei = make_float2(ei.x + ei.y, ei.x + ei.y);
             }
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
-                e0.x += __shfl_xor_sync(0xffffffffu, e0.x, o);
-                e0.y += __shfl_xor_sync(0xffffffffu, e0.y, o);
-                e1.x += __shfl_xor_sync(0xffffffffu, e1.x, o);
-                e1.y += __shfl_xor_sync(0xffffffffu, e1.y, o);
+                er = padd(er, make_float2(__shfl_xor_sync(0xffffffffu, er.x, o), __shfl_xor_sync(0xffffffffu, er.y, o)));
+                ei = padd(ei, make_float2(__shfl_xor_sync(0xffffffffu, ei.x, o), __shfl_xor_sync(0xffffffffu, ei.y, o)));
             }
-            e0 = cscale(e0, invA);
-            e1 = cscale(e1, invA);
+            er = pmul(er, make_float2(invA, invA));
+            ei = pmul(ei, make_float2(invA, invA));
+            const float2 en = make_float2(-er.x, -er.y);
 #pragma unroll
-            for (int r = 0; r < R; r++) {
-                const Ci4Word cw(x[r]);
+            for (int r = 0; r < R; r++)
 #pragma unroll
-                for (int b = 0; b < 4; b++) {
-                    const float2 e = cw.get(b);
-                    const float2 E = (b & 1) ? e1 : e0;
-                    float2 &o = num[r][b];
-                    o.x = fmaf(E.x, e.x, fmaf(E.y, e.y, o.x));      // E conj(e)
-                    o.y = fmaf(E.y, e.x, fmaf(-E.x, e.y, o.y));
-                    if (FIRST) dd[r][b] = fmaf(e.x, e.x, fmaf(e.y, e.y, dd[r][b]));
+                for (int k = 0; k < 2; k++) {
+                    const Ci4Pair e = ci4_pair(x[r], k);
+                    nr[r][k] = pfma(er, e.re, pfma(ei, e.im, nr[r][k]));      // E conj(e)
+                    ni[r][k] = pfma(ei, e.re, pfma(en, e.im, ni[r][k]));
+                    if (FIRST) dd[r][k] = pfma(e.re, e.re, pfma(e.im, e.im, dd[r][k]));
                 }
-            }
 #pragma unroll
             for (int r = 0; r < R; r++) x[r] = xn[r];
         }
 #pragma unroll
         for (int r = 0; r < R; r++)
 #pragma unroll
-            for (int b = 0; b < 4; b++) {
-                const int i = 4 * (lane + 32 * r) + b;
-                if (i >= AP) continue;
-                red[warp * AP + i] = num[r][b];
-                if (FIRST) wden[warp * AP + i] = dd[r][b];
-            }
+            for (int k = 0; k < 2; k++)
+#pragma unroll
+                for (int u = 0; u < 2; u++) {
+                    const int i = 4 * (lane + 32 * r) + 2 * k + u;
+                    if (i >= AP) continue;
+                    red[warp * AP + i] = u ? make_float2(nr[r][k].y, ni[r][k].y) : make_float2(nr[r][k].x, ni[r][k].x);
+                    if (FIRST) wden[warp * AP + i] = u ? dd[r][k].y : dd[r][k].x;
+                }
     };
     for (int it = 0; it < n_iter; it++) {
         if (it == 0) sweep(std::true_type{});
