@@ -75,6 +75,7 @@ struct GroupCfg {
     bool compact = false;
     bool cstage = false;               // its gather lists are staged in shared memory
     bool ctaps = false;                // and, with a kernel per antenna, the kernels
+    bool estage = false, etaps = false;   // the same for its E-field form (fp32_efield.cu)
     int crows = 0, cwords = 0;         // most occupied rows, most list words of a channel
     uint16_t *d_ltab = nullptr;        // device: gather lists (build_compact_lists)
     int2 *d_lidx = nullptr;            // device: [n_chan][gridding warps] (first batch, batches)
@@ -248,6 +249,8 @@ int build_compact_lists(const std::vector<short2> &cells, int A, int K, int P, c
                         std::vector<uint16_t> &tab, std::vector<int2> &idx, std::vector<int4> &chan);
 size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words);
 int prepare_compact(const epic_plan_s *plan, const GroupCfg &g);
+size_t efield_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words);
+int prepare_efield(const epic_plan_s *plan, const GroupCfg &g);
 int launch_compact(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
                    cudaStream_t stream);
 int launch_compact_efield(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T,

@@ -5,7 +5,7 @@
 // The occupied cells are gridded into a compact array whose corner is the first
 // occupied cell.  Moving the origin multiplies F(l) by one unit factor common to
 // both polarisations, which cancels in every product, so nothing is folded and
-// no class phase is needed (E-field images put the factor back).  Rows are
+// no class phase is needed (E-field images: fp32_efield.cu).  Rows are
 // transformed to all N columns, then columns to all N rows, each N-point
 // transform as N / M classes of M-point register transforms (fft_class.cuh).
 //
@@ -30,7 +30,7 @@
 //
 // Measured against the per-class kernel (one GB300, whole calls): 256 antennas, 64 channels of
 // 128 x 128, 1000 spectra 5.78 -> 3.10 ms; the same as 25 Stokes images with delays 8.30 -> 3.61 ms;
-// E-field images of 50 spectra 0.535 -> 0.402 ms; per-antenna kernels, 250 spectra 2.55 -> 1.55 ms;
+// per-antenna kernels, 250 spectra 2.55 -> 1.55 ms;
 // 37 channels at 64, 96 and 128 0.67 -> 0.46 ms.  Bound by the transform warps' issue: the FMA
 // pipe is active 51 % of the time (42 % there, for half the work), 8 transform warps an SM.
 //
@@ -99,14 +99,13 @@ struct CompactShape {
 };
 
 // staged: bit 0 the gather lists, bit 1 the antennas' kernels (AK) are in shared memory
-template <int M, int Q, int P, int TS, bool AK, bool EF>
+template <int M, int Q, int P, int TS, bool AK>
 __global__ void __launch_bounds__(kCThreads, 1)
 fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gains, const float2 *__restrict__ kern,
                     int K, const int *__restrict__ chans, const uint16_t *__restrict__ ltab,
                     const int2 *__restrict__ lidx, const int4 *__restrict__ lchan, int A, int C, int T, int n_chan,
                     int n_tau, int rmax, int staged, float *__restrict__ partial, const float *__restrict__ dfreq,
-                    const float4 *__restrict__ dtab, const float2 *__restrict__ twN, float2 *__restrict__ ef_out,
-                    const long long *__restrict__ ef_off, long long ef_stride, int *__restrict__ status, long long wait_budget)
+                    const float4 *__restrict__ dtab, int *__restrict__ status, long long wait_budget)
 {
     using S = CompactShape<M, Q, P, TS>;
     constexpr int N = S::N, RS = N + 1, KO = M / 8, KH = KO / P;   // outputs per group; pixels a lane keeps of it
@@ -133,8 +132,7 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
     const int4 ch = lchan[2 * ci];                               // (block start, block words, rows, columns)
     const int rows = ch.z, cols = ch.w;
 
-    if constexpr (!EF)
-        if (warp == 0) tc::tmem_alloc(&tmem_slot, S::COLS);
+    if (warp == 0) tc::tmem_alloc(&tmem_slot, S::COLS);
     if (tid == 0) {
         tc::mbar_init(&bar_full, kGW);
         tc::mbar_init(&bar_free, kFW);
@@ -166,10 +164,10 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
     }
     if (staged & 1)
         for (int i = tid; i < ch.y; i += kCThreads) stab[i] = __ldg(ltab + ch.x + i);
-    if constexpr (!EF) tc::fence_before_sync();
+    tc::fence_before_sync();
     __syncthreads();
-    if constexpr (!EF) tc::fence_after_sync();
-    const uint32_t taddr = EF ? 0u : tmem_slot;
+    tc::fence_after_sync();
+    const uint32_t taddr = tmem_slot;
     // Waits are bounded: a warp whose wait runs out records it and waits no more, so the block ends
     // (its output undefined) and nothing hangs.
     bool dead = false;
@@ -187,13 +185,11 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
     if (warp < kFW) {
         // ================ transforms
         const uint32_t tw0 = taddr + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + (warp >> 2) * (S::SL * S::CW);
-        if constexpr (!EF) {
-            uint32_t z[32];
+        uint32_t z[32];
 #pragma unroll
-            for (int j = 0; j < 32; j++) z[j] = 0u;
-            for (int cc = 0; cc < S::SL * S::CW; cc += 32) tc::tmem_st32_issue(tw0 + cc, z);
-            tc::tmem_wait_st();
-        }
+        for (int j = 0; j < 32; j++) z[j] = 0u;
+        for (int cc = 0; cc < S::SL * S::CW; cc += 32) tc::tmem_st32_issue(tw0 + cc, z);
+        tc::tmem_wait_st();
         const int rb = (rows * P + 31) >> 5;                     // row tasks per sample and class
         const int n_row = TS * Q * rb;
         const int last_k = (S::TASKS - 1 - warp) / kFW;          // the warp's last column task (TASKS - 1 < warp: none)
@@ -236,61 +232,43 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
                 class_load<M, RS>(x, R + (ts * P + p) * rplane + col, (rows + 7) >> 3, h);
                 if (k == last_k) arrive(bar_read);
                 class_turn<M>(x, (rows + 7) >> 3, h);
-                if constexpr (EF) {
-                    // F(l) of the corner-based array times w_N^{x0 lx + y0 ly}, on the shifted layout
-                    const int4 org = lchan[2 * ci + 1];
-                    const long long NN = static_cast<long long>(N) * N;
-                    float2 *dst = ef_out + static_cast<long long>(t + ts) * ef_stride + ef_off[ci] + p * NN +
-                                  (col >= N / 2 ? col - N / 2 : col + N / 2);
-                    const bool ok = t + ts < t1;
-                    fft_groups<M>(x, [&](int k1, auto &o) {
+                const uint32_t at = tw0 + k * S::CW;
+                fft_groups<M>(x, [&](int k1, auto &o) {
+                    if constexpr (P == 2) {
+                        uint32_t s[16];
+                        tc::tmem_ld16_issue(at + 16 * k1, s);
+                        float bx[KH], by[KH];
 #pragma unroll
-                        for (int k2 = 0; k2 < KO; k2++) {
-                            const int ly = Q * (k1 + 8 * k2) + h;
-                            const float2 w = __ldg(twN + (org.x * col + org.y * ly) % N);
-                            const int i = ly >= N / 2 ? ly - N / 2 : ly + N / 2;
-                            if (ok) dst[static_cast<long long>(i) * N] = cmul(o[k2], w);
+                        for (int j = 0; j < KH; j++) {
+                            bx[j] = __shfl_xor_sync(0xffffffffu, o[j + KH].x, 16);
+                            by[j] = __shfl_xor_sync(0xffffffffu, o[j + KH].y, 16);
                         }
-                    });
-                } else {
-                    const uint32_t at = tw0 + k * S::CW;
-                    fft_groups<M>(x, [&](int k1, auto &o) {
-                        if constexpr (P == 2) {
-                            uint32_t s[16];
-                            tc::tmem_ld16_issue(at + 16 * k1, s);
-                            float bx[KH], by[KH];
+                        tc::tmem_wait_ld();
+                        tc::reg_fence16(s);
+                        // own |F|^2, the other polarisation's |F|^2, Re and Im of F_X F_Y^* (Im with the
+                        // lane's sign: own F_Y on the Y lanes)
 #pragma unroll
-                            for (int j = 0; j < KH; j++) {
-                                bx[j] = __shfl_xor_sync(0xffffffffu, o[j + KH].x, 16);
-                                by[j] = __shfl_xor_sync(0xffffffffu, o[j + KH].y, 16);
-                            }
-                            tc::tmem_wait_ld();
-                            tc::reg_fence16(s);
-                            // own |F|^2, the other polarisation's |F|^2, Re and Im of F_X F_Y^* (Im with the
-                            // lane's sign: own F_Y on the Y lanes)
-#pragma unroll
-                            for (int j = 0; j < KH; j++) {
-                                const float2 a = o[j];
-                                const float cx = bx[j], cy = by[j];
-                                s[4 * j] = __float_as_uint(fmaf(a.x, a.x, fmaf(a.y, a.y, __uint_as_float(s[4 * j]))));
-                                s[4 * j + 1] = __float_as_uint(fmaf(cx, cx, fmaf(cy, cy, __uint_as_float(s[4 * j + 1]))));
-                                s[4 * j + 2] = __float_as_uint(fmaf(a.x, cx, fmaf(a.y, cy, __uint_as_float(s[4 * j + 2]))));
-                                s[4 * j + 3] = __float_as_uint(fmaf(a.y, cx, fmaf(-a.x, cy, __uint_as_float(s[4 * j + 3]))));
-                            }
-                            tc::tmem_st16_issue(at + 16 * k1, s);
-                        } else {
-                            uint32_t s[8];
-                            tc::tmem_ld8_issue(at + 8 * k1, s);
-                            tc::tmem_wait_ld();
-                            tc::reg_fence8(s);
-#pragma unroll
-                            for (int j = 0; j < KO; j++)
-                                s[j] = __float_as_uint(fmaf(o[j].x, o[j].x, fmaf(o[j].y, o[j].y, __uint_as_float(s[j]))));
-                            tc::tmem_st8_issue(at + 8 * k1, s);
+                        for (int j = 0; j < KH; j++) {
+                            const float2 a = o[j];
+                            const float cx = bx[j], cy = by[j];
+                            s[4 * j] = __float_as_uint(fmaf(a.x, a.x, fmaf(a.y, a.y, __uint_as_float(s[4 * j]))));
+                            s[4 * j + 1] = __float_as_uint(fmaf(cx, cx, fmaf(cy, cy, __uint_as_float(s[4 * j + 1]))));
+                            s[4 * j + 2] = __float_as_uint(fmaf(a.x, cx, fmaf(a.y, cy, __uint_as_float(s[4 * j + 2]))));
+                            s[4 * j + 3] = __float_as_uint(fmaf(a.y, cx, fmaf(-a.x, cy, __uint_as_float(s[4 * j + 3]))));
                         }
-                    });
-                    tc::tmem_wait_st();
-                }
+                        tc::tmem_st16_issue(at + 16 * k1, s);
+                    } else {
+                        uint32_t s[8];
+                        tc::tmem_ld8_issue(at + 8 * k1, s);
+                        tc::tmem_wait_ld();
+                        tc::reg_fence8(s);
+#pragma unroll
+                        for (int j = 0; j < KO; j++)
+                            s[j] = __float_as_uint(fmaf(o[j].x, o[j].x, fmaf(o[j].y, o[j].y, __uint_as_float(s[j]))));
+                        tc::tmem_st8_issue(at + 8 * k1, s);
+                    }
+                });
+                tc::tmem_wait_st();
             }
         }
     } else {
@@ -434,7 +412,7 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
                 }
                 if (off != kNoCell) {
                     float2 *cell = G + (off & 0x7FFFu);
-                    const float sg = !EF && P == 2 && (off & kOddRow) ? -1.f : 1.f;   // (-1)^y on Y
+                    const float sg = P == 2 && (off & kOddRow) ? -1.f : 1.f;   // (-1)^y on Y
 #pragma unroll
                     for (int ts = 0; ts < TS; ts++)
 #pragma unroll
@@ -470,75 +448,73 @@ fp32_compact_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ ga
         }
     }
 
-    if constexpr (!EF) {
-        // ---- partial image: [tau][channel item of class (hy, hx)][my M + mx]
-        __syncthreads();
-        float4 *sum4 = reinterpret_cast<float4 *>(R);
-        float *sum1 = reinterpret_cast<float *>(R);
-        for (int pass = TS - 1; pass >= 0; pass--) {             // TS == 2: the second sample's sums first, through R
-            if (warp < kFW) {
-                const uint32_t tw0 = taddr + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + (warp >> 2) * (S::SL * S::CW);
-                for (int k = 0; k < S::SL; k++) {
-                    const int task = warp + k * kFW;
-                    if (task >= S::TASKS) break;
-                    const int h = S::cls(task, k), blk = (task / Q) % (N / S::CB), ts = task / (Q * (N / S::CB));
-                    if (ts != pass) continue;
-                    const int p = lane / S::CB, col = blk * S::CB + lane % S::CB;
-                    const int hx = col % Q, mx = col / Q;
-                    const size_t item = static_cast<size_t>(tau) * (n_chan * Q * Q) + ci * Q * Q + h * Q + hx;
-                    const int slot = (task % (Q * (N / S::CB))) * 8;   // the pair of tasks of two samples share it
+    // ---- partial image: [tau][channel item of class (hy, hx)][my M + mx]
+    __syncthreads();
+    float4 *sum4 = reinterpret_cast<float4 *>(R);
+    float *sum1 = reinterpret_cast<float *>(R);
+    for (int pass = TS - 1; pass >= 0; pass--) {             // TS == 2: the second sample's sums first, through R
+        if (warp < kFW) {
+            const uint32_t tw0 = taddr + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + (warp >> 2) * (S::SL * S::CW);
+            for (int k = 0; k < S::SL; k++) {
+                const int task = warp + k * kFW;
+                if (task >= S::TASKS) break;
+                const int h = S::cls(task, k), blk = (task / Q) % (N / S::CB), ts = task / (Q * (N / S::CB));
+                if (ts != pass) continue;
+                const int p = lane / S::CB, col = blk * S::CB + lane % S::CB;
+                const int hx = col % Q, mx = col / Q;
+                const size_t item = static_cast<size_t>(tau) * (n_chan * Q * Q) + ci * Q * Q + h * Q + hx;
+                const int slot = (task % (Q * (N / S::CB))) * 8;   // the pair of tasks of two samples share it
 #pragma unroll
-                    for (int k1 = 0; k1 < 8; k1++) {
-                        if constexpr (P == 2) {
-                            uint32_t s[16];
-                            tc::tmem_ld16_issue(tw0 + k * S::CW + 16 * k1, s);
-                            tc::tmem_wait_ld();
-                            tc::reg_fence16(s);
-                            float4 *dst = reinterpret_cast<float4 *>(partial) + item * (M * M) + mx;
+                for (int k1 = 0; k1 < 8; k1++) {
+                    if constexpr (P == 2) {
+                        uint32_t s[16];
+                        tc::tmem_ld16_issue(tw0 + k * S::CW + 16 * k1, s);
+                        tc::tmem_wait_ld();
+                        tc::reg_fence16(s);
+                        float4 *dst = reinterpret_cast<float4 *>(partial) + item * (M * M) + mx;
 #pragma unroll
-                            for (int j = 0; j < KH; j++) {
-                                const float a = __uint_as_float(s[4 * j]), b = __uint_as_float(s[4 * j + 1]);
-                                const float re = __uint_as_float(s[4 * j + 2]), im = __uint_as_float(s[4 * j + 3]);
-                                float4 f = p ? make_float4(b, a, re, -im) : make_float4(a, b, re, im);
-                                float4 *sl = sum4 + ((slot + k1) * KH + j) * 32 + lane;
-                                if (TS == 2 && pass == 1) {
-                                    *sl = f;
-                                    continue;
-                                }
-                                if (TS == 2) {
-                                    const float4 o = *sl;
-                                    f = make_float4(f.x + o.x, f.y + o.y, f.z + o.z, f.w + o.w);
-                                }
-                                dst[(k1 + 8 * (j + p * KH)) * M] = f;
+                        for (int j = 0; j < KH; j++) {
+                            const float a = __uint_as_float(s[4 * j]), b = __uint_as_float(s[4 * j + 1]);
+                            const float re = __uint_as_float(s[4 * j + 2]), im = __uint_as_float(s[4 * j + 3]);
+                            float4 f = p ? make_float4(b, a, re, -im) : make_float4(a, b, re, im);
+                            float4 *sl = sum4 + ((slot + k1) * KH + j) * 32 + lane;
+                            if (TS == 2 && pass == 1) {
+                                *sl = f;
+                                continue;
                             }
-                        } else {
-                            uint32_t s[8];
-                            tc::tmem_ld8_issue(tw0 + k * S::CW + 8 * k1, s);
-                            tc::tmem_wait_ld();
-                            tc::reg_fence8(s);
-                            float *dst = partial + item * (M * M) + mx;
-#pragma unroll
-                            for (int j = 0; j < KO; j++) {
-                                float f = __uint_as_float(s[j]);
-                                float *sl = sum1 + ((slot + k1) * KO + j) * 32 + lane;
-                                if (TS == 2 && pass == 1) {
-                                    *sl = f;
-                                    continue;
-                                }
-                                if (TS == 2) f += *sl;
-                                dst[(k1 + 8 * j) * M] = f;
+                            if (TS == 2) {
+                                const float4 o = *sl;
+                                f = make_float4(f.x + o.x, f.y + o.y, f.z + o.z, f.w + o.w);
                             }
+                            dst[(k1 + 8 * (j + p * KH)) * M] = f;
+                        }
+                    } else {
+                        uint32_t s[8];
+                        tc::tmem_ld8_issue(tw0 + k * S::CW + 8 * k1, s);
+                        tc::tmem_wait_ld();
+                        tc::reg_fence8(s);
+                        float *dst = partial + item * (M * M) + mx;
+#pragma unroll
+                        for (int j = 0; j < KO; j++) {
+                            float f = __uint_as_float(s[j]);
+                            float *sl = sum1 + ((slot + k1) * KO + j) * 32 + lane;
+                            if (TS == 2 && pass == 1) {
+                                *sl = f;
+                                continue;
+                            }
+                            if (TS == 2) f += *sl;
+                            dst[(k1 + 8 * j) * M] = f;
                         }
                     }
                 }
             }
-            if (TS == 2) __syncthreads();
         }
-        tc::fence_before_sync();
-        __syncthreads();
-        tc::fence_after_sync();
-        if (warp == 0) tc::tmem_dealloc(taddr, S::COLS);
+        if (TS == 2) __syncthreads();
     }
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    if (warp == 0) tc::tmem_dealloc(taddr, S::COLS);
 }
 
 template <int V>
@@ -556,15 +532,15 @@ int compact_dispatch(const GroupCfg &g, int P, F &&f)
     return P == 2 ? with_p(IC<2>{}) : with_p(IC<1>{});
 }
 
-template <int M, int Q, int P, int TS, bool AK, bool EF>
+template <int M, int Q, int P, int TS, bool AK>
 int launch_compact_t(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int n_tau,
-                     cudaStream_t stream, float2 *ef_out, long long ef_stride)
+                     cudaStream_t stream)
 {
     const CompactSmem L = compact_smem(P, TS, g.N, g.crows, plan->A, plan->K, plan->nker, g.ctaps, g.cstage ? g.cwords : 0);
-    fp32_compact_kernel<M, Q, P, TS, AK, EF><<<static_cast<unsigned>(g.n_chan * n_tau), kCThreads, L.total, stream>>>(
+    fp32_compact_kernel<M, Q, P, TS, AK><<<static_cast<unsigned>(g.n_chan * n_tau), kCThreads, L.total, stream>>>(
         v, gains, plan->d_kernel, plan->K, g.d_chans, g.d_ltab, g.d_lidx, g.d_lchan, plan->A, plan->C, T, g.n_chan, n_tau,
-        g.crows, (g.cstage ? 1 : 0) | (g.ctaps ? 2 : 0), g.d_partial, plan->d_dfreq, !EF && plan->delays ? plan->d_dtab : nullptr, g.d_twN,
-        ef_out, g.d_ef_off, ef_stride, plan->d_status, plan->wait_budget);
+        g.crows, (g.cstage ? 1 : 0) | (g.ctaps ? 2 : 0), g.d_partial, plan->d_dfreq, plan->delays ? plan->d_dtab : nullptr, plan->d_status,
+        plan->wait_budget);
     return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
 }
 
@@ -676,14 +652,8 @@ int prepare_compact(const epic_plan_s *plan, const GroupCfg &g)
     const size_t need = compact_smem_bytes(g.N, plan->P, g.crows, plan->A, plan->K, plan->nker, g.ctaps, g.cstage ? g.cwords : 0);
     return compact_dispatch(g, plan->P, [&](auto m_, auto q_, auto p_, auto ts_) {
         constexpr int M = decltype(m_)::value, Q = decltype(q_)::value, P = decltype(p_)::value, TS = decltype(ts_)::value;
-        auto both = [&](auto ak) {
-            constexpr bool AK = decltype(ak)::value != 0;
-            const int rc = raise_dyn_smem_cap(reinterpret_cast<const void *>(fp32_compact_kernel<M, Q, P, TS, AK, false>), need);
-            return rc != EPIC_OK
-                       ? rc
-                       : raise_dyn_smem_cap(reinterpret_cast<const void *>(fp32_compact_kernel<M, Q, P, TS, AK, true>), need);
-        };
-        return plan->nker > 1 ? both(IC<1>{}) : both(IC<0>{});
+        return plan->nker > 1 ? raise_dyn_smem_cap(reinterpret_cast<const void *>(fp32_compact_kernel<M, Q, P, TS, true>), need)
+                              : raise_dyn_smem_cap(reinterpret_cast<const void *>(fp32_compact_kernel<M, Q, P, TS, false>), need);
     });
 }
 
@@ -694,19 +664,8 @@ int launch_compact(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const
     *n_tau_out = n_tau;
     return compact_dispatch(g, plan->P, [&](auto m_, auto q_, auto p_, auto ts_) {
         constexpr int M = decltype(m_)::value, Q = decltype(q_)::value, P = decltype(p_)::value, TS = decltype(ts_)::value;
-        return plan->nker > 1 ? launch_compact_t<M, Q, P, TS, true, false>(plan, g, v, gains, T, n_tau, stream, nullptr, 0)
-                              : launch_compact_t<M, Q, P, TS, false, false>(plan, g, v, gains, T, n_tau, stream, nullptr, 0);
-    });
-}
-
-int launch_compact_efield(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T,
-                          float2 *out, long long stride, cudaStream_t stream)
-{
-    const int n_tau = choose_tau(plan, g, T);
-    return compact_dispatch(g, plan->P, [&](auto m_, auto q_, auto p_, auto ts_) {
-        constexpr int M = decltype(m_)::value, Q = decltype(q_)::value, P = decltype(p_)::value, TS = decltype(ts_)::value;
-        return plan->nker > 1 ? launch_compact_t<M, Q, P, TS, true, true>(plan, g, v, gains, T, n_tau, stream, out, stride)
-                              : launch_compact_t<M, Q, P, TS, false, true>(plan, g, v, gains, T, n_tau, stream, out, stride);
+        return plan->nker > 1 ? launch_compact_t<M, Q, P, TS, true>(plan, g, v, gains, T, n_tau, stream)
+                              : launch_compact_t<M, Q, P, TS, false>(plan, g, v, gains, T, n_tau, stream);
     });
 }
 

@@ -823,9 +823,15 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                            static_cast<size_t>(smem_optin);
                 };
                 // the planes must fit; then the antennas' kernels, then the lists (else through L1)
-                g.compact = fits(false, 0);
+                auto ef_fits = [&](bool taps, int words) {
+                    return epic::efield_smem_bytes(g.N, n_pol, g.crows, n_ant, p->K, p->nker, taps, words) + 64 <=
+                           static_cast<size_t>(smem_optin);
+                };
+                g.compact = fits(false, 0) && ef_fits(false, 0);
                 g.ctaps = p->nker > 1 && fits(true, 0);
                 g.cstage = fits(g.ctaps, g.cwords) && !(diag & EPIC_DIAG_GATHER_GLOBAL);
+                g.etaps = p->nker > 1 && ef_fits(true, 0);
+                g.estage = ef_fits(g.etaps, g.cwords) && !(diag & EPIC_DIAG_GATHER_GLOBAL);
             }
             if (g.compact) {
                 g.R1 = 1;
@@ -1042,6 +1048,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
         if (rc != EPIC_OK) break;
         if (!g.tensor) rc = epic::prepare_fp32(p, g);
         if (rc == EPIC_OK && g.compact) rc = epic::prepare_compact(p, g);
+        if (rc == EPIC_OK && g.compact) rc = epic::prepare_efield(p, g);
         if (rc == EPIC_OK && g.wide) rc = epic::prepare_wide(p, g);
         if (rc == EPIC_OK && g.alias) rc = epic::prepare_alias(p);
     }
