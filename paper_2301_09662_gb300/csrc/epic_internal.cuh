@@ -77,6 +77,7 @@ struct GroupCfg {
     bool ctaps = false;                // and, with a kernel per antenna, the kernels
     bool estage = false, etaps = false;   // the same for its E-field form (fp32_efield.cu)
     int crows = 0, cwords = 0;         // most occupied rows, most list words of a channel
+    int erows = 0;                     // the E-field form's rows between its transforms
     uint16_t *d_ltab = nullptr;        // device: gather lists (build_compact_lists)
     int2 *d_lidx = nullptr;            // device: [n_chan][gridding warps] (first batch, batches)
     int4 *d_lchan = nullptr;           // device: [n_chan][2] (block start, words, rows, columns), (origin x, y, 0, 0)
@@ -249,7 +250,8 @@ int build_compact_lists(const std::vector<short2> &cells, int A, int K, int P, c
                         std::vector<uint16_t> &tab, std::vector<int2> &idx, std::vector<int4> &chan);
 size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words);
 int prepare_compact(const epic_plan_s *plan, const GroupCfg &g);
-size_t efield_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words);
+size_t efield_smem_bytes(int N, int P, int rows, int rrows, int A, int K, int nker, bool taps, int words);
+int efield_rows(int N, const std::vector<int4> &lchan);   // most rows of R where every channel is placed on a quarter
 int prepare_efield(const epic_plan_s *plan, const GroupCfg &g);
 int launch_compact(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
                    cudaStream_t stream);

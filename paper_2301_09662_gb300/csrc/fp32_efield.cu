@@ -7,10 +7,14 @@
 // holds a column of both, so a warp writes 32 consecutive pixels of each, and
 // without time sums to keep the 32-point classes leave room for it.  The
 // imaging kernel's lanes hold one polarisation and 16 columns a warp: 0.404 ms
-// for 50 spectra of 64 channels of 128 x 128 (840 MB written), 0.340 ms here.  (With
+// for 50 spectra of 64 channels of 128 x 128 (840 MB written), 0.311 ms here.  (With
 // products this form was the slower one: 3.44 ms against 3.10 for 1000 spectra.)
 //
-// The corner-based array's transform takes the factor w_N^{x0 lx + y0 ly} back.
+// An origin (x0, y0) other than 0 leaves a factor w_N^{x0 lx + y0 ly} on the
+// transform.  The array is placed from the origin's quarter of the grid on
+// (efield_place), so that the factor is a power of i and rounds nothing: 1.28e-7
+// of the fields' norm in that case, 1.35e-7 with factors from a table (0.319 ms).
+// An aperture that is too far off the grid's centre for that takes the table's.
 #include <algorithm>
 #include <type_traits>
 
@@ -29,18 +33,37 @@ constexpr uint16_t kNoCell = 0xFFFFu;      // (bit 15 of a cell offset: odd row,
 // Rows of R: whole blocks of eight (pair_load), the last ones zeros.
 __host__ __device__ inline int efield_pad(int rows) { return (rows + 7) & ~7; }
 
+// Where the transforms see a channel's occupied cells (rows x cols from (x0, y0)): moved by (dx, dy)
+// from the corner, with origins kx N/4 and ky N/4; quarter 0: from the corner, with origin (x0, y0).
+struct EfieldPlace {
+    int dx, dy, kx, ky, quarter;
+};
+__host__ __device__ inline EfieldPlace efield_place(int N, int rows, int cols, int x0, int y0)
+{
+    auto axis = [N](int at, int n, int &d, int &k) {
+        k = at >= N / 4 && at - N / 4 + n <= 64;
+        d = at - k * (N / 4);
+        return d + n <= 64;
+    };
+    EfieldPlace p{};
+    p.quarter = axis(x0, cols, p.dx, p.kx) && axis(y0, rows, p.dy, p.ky);
+    if (!p.quarter) p.dx = p.dy = 0;
+    return p;
+}
+
 // Byte offsets of the shared-memory regions.
 struct EfieldSmem {
     unsigned R, es, gp, taps, tab, total;
 };
-// pairs: signal pairs per iteration; taps: the kernels of every antenna are staged (nker > 1)
-__host__ __device__ inline EfieldSmem efield_smem(int P, int pairs, int N, int rows, int A, int K, int nker, bool taps,
-                                                    int words)
+// pairs: signal pairs per iteration; rows: most rows of G, rrows: of R; taps: the kernels of every
+// antenna are staged (nker > 1)
+__host__ __device__ inline EfieldSmem efield_smem(int P, int pairs, int N, int rows, int rrows, int A, int K, int nker,
+                                                    bool taps, int words)
 {
     auto up = [](unsigned b) { return (b + 15u) & ~15u; };
     EfieldSmem s;
     s.R = static_cast<unsigned>(pairs * rows * kES) * 16u;
-    s.es = s.R + static_cast<unsigned>(pairs * efield_pad(rows)) * (N + 1) * 16u;
+    s.es = s.R + static_cast<unsigned>(pairs * efield_pad(rrows)) * (N + 1) * 16u;
     s.gp = s.es + 2u * pairs * A * 16u;
     s.taps = s.gp + up(static_cast<unsigned>(A * P) * 8u);
     s.tab = s.taps + (nker > 1 ? (taps ? up(static_cast<unsigned>(nker * K * K) * 8u) : 0u)
@@ -61,13 +84,14 @@ struct EfieldShape {
 };
 constexpr int kEThreads = 384;
 
-// staged: bit 0 the gather lists, bit 1 the antennas' kernels (AK) are in shared memory
+// staged: bit 0 the gather lists, bit 1 the antennas' kernels (AK) are in shared memory; rmax and
+// rrows: most rows of G and of R
 template <int Q, int P, int PAIRS, bool AK>
 __global__ void __launch_bounds__(kEThreads, 1)
 efield_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gains, const float2 *__restrict__ kern,
                     int K, const int *__restrict__ chans, const uint16_t *__restrict__ ltab,
                     const int2 *__restrict__ lidx, const int4 *__restrict__ lchan, int A, int C, int T, int n_chan,
-                    int n_tau, int rmax, int staged, const float2 *__restrict__ twN, float2 *__restrict__ ef_out,
+                    int n_tau, int rmax, int rrows, int staged, const float2 *__restrict__ twN, float2 *__restrict__ ef_out,
                     const long long *__restrict__ ef_off, long long ef_stride, int *__restrict__ status,
                     long long wait_budget)
 {
@@ -77,15 +101,15 @@ efield_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gains, c
     // G holds a sample (gridding warps arrive); G has been read, R has been read (transform warps)
     __shared__ __align__(8) uint64_t bar_full, bar_free, bar_read;
     const int AP = A * P, KK = K * K, TPN = K * (K + 1);
-    const EfieldSmem L = efield_smem(P, PAIRS, N, rmax, A, K, AK ? A : 1, (staged & 2) != 0, 0);
+    const EfieldSmem L = efield_smem(P, PAIRS, N, rmax, rrows, A, K, AK ? A : 1, (staged & 2) != 0, 0);
     float4 *G = reinterpret_cast<float4 *>(smem_c);              // [PAIRS][rmax][65]: (re a, re b, im a, im b)
-    float4 *R = reinterpret_cast<float4 *>(smem_c + L.R);        // [PAIRS][padded rmax][N + 1]
+    float4 *R = reinterpret_cast<float4 *>(smem_c + L.R);        // [PAIRS][padded rrows][N + 1]
     float4 *es = reinterpret_cast<float4 *>(smem_c + L.es);      // [2][PAIRS][A]
     float2 *gp = reinterpret_cast<float2 *>(smem_c + L.gp);      // [A P]
     float4 *tw2 = reinterpret_cast<float4 *>(smem_c + L.taps);   // [K (K + 1) + 1][8 copies] (one kernel)
     uint16_t *stab = reinterpret_cast<uint16_t *>(smem_c + L.tab);
     const float2 *tapw = staged & 2 ? reinterpret_cast<const float2 *>(smem_c + L.taps) : kern;   // [A][K K] (AK)
-    const int gplane = rmax * kES, rplane = efield_pad(rmax) * RS;
+    const int gplane = rmax * kES, rplane = efield_pad(rrows) * RS;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ci = blockIdx.x % n_chan, tau = blockIdx.x / n_chan;
@@ -94,6 +118,9 @@ efield_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gains, c
     const int t1 = static_cast<int>(static_cast<long long>(T) * (tau + 1) / n_tau);
     const int4 ch = lchan[2 * ci];                               // (block start, block words, rows, columns)
     const int rows = ch.z, cols = ch.w;
+    const int4 org = lchan[2 * ci + 1];                          // (x0, y0, -, -)
+    EfieldPlace pl = efield_place(N, rows, cols, org.x, org.y);
+    if (pl.dy + rows > rrows) pl = EfieldPlace{};                // no room for the moved rows
 
     if (tid == 0) {
         tc::mbar_init(&bar_full, S::GW);
@@ -101,11 +128,12 @@ efield_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gains, c
         tc::mbar_init(&bar_read, S::FW);
         tc::fence_mbar_init();
     }
-    // ---- set-up: a zero G (the cells no list names stay zero), zeros past R's rows, gains, taps, lists
+    // ---- set-up: a zero G (the cells no list names stay zero), zeros before and past R's rows, gains, taps, lists
     const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
     for (int i = tid; i < PAIRS * gplane; i += kEThreads) G[i] = zero4;
-    const int rpad = (efield_pad(rows) - rows) * RS;
-    for (int i = tid; i < PAIRS * rpad; i += kEThreads) R[(i / rpad) * rplane + rows * RS + i % rpad] = zero4;
+    const int ry = pl.dy, rpad = (efield_pad(ry + rows) - rows) * RS;
+    for (int i = tid; i < PAIRS * rpad; i += kEThreads)
+        R[(i / rpad) * rplane + (i % rpad < ry * RS ? 0 : rows * RS) + i % rpad] = zero4;
     for (int i = tid; i < AP; i += kEThreads)
         gp[i] = gains ? gains[static_cast<size_t>(c) * AP + i] : make_float2(1.f, 0.f);
     if constexpr (AK) {
@@ -143,7 +171,7 @@ efield_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gains, c
     };
     if (warp < S::FW) {
         // ================ transforms
-        const int rb = (rows + 31) >> 5, nbx = (cols + 7) >> 3, nby = (rows + 7) >> 3;
+        const int rb = (rows + 31) >> 5, nbx = (pl.dx + cols + 7) >> 3, nby = (ry + rows + 7) >> 3;
         const int n_row = PAIRS * Q * rb;
         const int last_k = (S::TASKS - 1 - warp) / S::FW;        // the warp's last column task (TASKS - 1 < warp: none)
         uint32_t ph = 0;
@@ -158,7 +186,7 @@ efield_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gains, c
                 pair_load<Q, 1>(xr, xi, G + pr * gplane + (ok ? y : 0) * kES, nbx, h);
                 if (task + S::FW >= n_row) arrive(bar_free);     // this warp has read G
                 pair_turn<Q>(xr, xi, nbx, h);
-                float4 *dst = R + pr * rplane + y * RS + h;
+                float4 *dst = R + pr * rplane + (ry + y) * RS + h;
                 if (!r_free) {
                     wait(bar_read, ph ^ 1u);                     // the columns of the sample before have been read
                     r_free = true;
@@ -184,8 +212,7 @@ efield_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gains, c
                 pair_load<Q, RS>(xr, xi, R + pr * rplane + col, nby, h);
                 if (k == last_k) arrive(bar_read);
                 pair_turn<Q>(xr, xi, nby, h);
-                // F(l) of the corner-based array times w_N^{x0 lx + y0 ly}, on the shifted layout
-                const int4 org = lchan[2 * ci + 1];
+                // F(l) of the placed array times the origin's factor, on the shifted layout
                 const long long NN = static_cast<long long>(N) * N;
                 const int ta = P == 2 ? t + pr : t + 2 * pr;
                 float2 *dst = ef_out + static_cast<long long>(ta) * ef_stride + ef_off[ci] +
@@ -193,10 +220,14 @@ efield_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gains, c
                 float2 *dst_b = dst + (P == 2 ? NN : ef_stride);   // Y, or the next sample
                 const bool ok_a = ta < t1, ok_b = P == 2 ? ok_a : ta + 1 < t1;
                 pair_fft32(xr, xi, [&](int k1, auto &r, auto &i) {
+                    // i^{kx lx + ky ly}, the same for the four k2 (8 Q is a multiple of 4)
+                    const int e = pl.kx * col + pl.ky * (Q * k1 + h);
+                    const float s = e & 2 ? -1.f : 1.f;
+                    float2 w = e & 1 ? make_float2(0.f, s) : make_float2(s, 0.f);
 #pragma unroll
                     for (int k2 = 0; k2 < 4; k2++) {
                         const int ly = Q * (k1 + 8 * k2) + h;
-                        const float2 w = __ldg(twN + (org.x * col + org.y * ly) % N);
+                        if (!pl.quarter) w = __ldg(twN + (org.x * col + org.y * ly) % N);
                         pair_mul(r[k2], i[k2], make_float2(w.x, w.x), make_float2(w.y, w.y), make_float2(-w.y, -w.y));
                         const long long o = static_cast<long long>(ly >= N / 2 ? ly - N / 2 : ly + N / 2) * N;
                         if (ok_a) dst[o] = make_float2(r[k2].x, i[k2].x);
@@ -325,7 +356,7 @@ efield_kernel(const uint8_t *__restrict__ v, const float2 *__restrict__ gains, c
 #pragma unroll
                     for (int pr = 0; pr < PAIRS; pr++)
 #pragma unroll
-                        for (int u = 0; u < 2; u++) G[pr * gplane + (off & 0x7FFFu) + u] = acc[pr][u];
+                        for (int u = 0; u < 2; u++) G[pr * gplane + pl.dx + (off & 0x7FFFu) + u] = acc[pr][u];
                 }
                 bt = nbt;
                 d = dn;
@@ -377,23 +408,31 @@ template <int Q, int P, int PAIRS, bool AK>
 int launch_efield_t(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int n_tau,
                     float2 *out, long long stride, cudaStream_t stream)
 {
-    const EfieldSmem L = efield_smem(P, PAIRS, g.N, g.crows, plan->A, plan->K, plan->nker, g.etaps, g.estage ? g.cwords : 0);
+    const EfieldSmem L = efield_smem(P, PAIRS, g.N, g.crows, g.erows, plan->A, plan->K, plan->nker, g.etaps, g.estage ? g.cwords : 0);
     efield_kernel<Q, P, PAIRS, AK><<<static_cast<unsigned>(g.n_chan * n_tau), kEThreads, L.total, stream>>>(
         v, gains, plan->d_kernel, plan->K, g.d_chans, g.d_ltab, g.d_lidx, g.d_lchan, plan->A, plan->C, T, g.n_chan, n_tau,
-        g.crows, (g.estage ? 1 : 0) | (g.etaps ? 2 : 0), g.d_twN, out, g.d_ef_off, stride, plan->d_status, plan->wait_budget);
+        g.crows, g.erows, (g.estage ? 1 : 0) | (g.etaps ? 2 : 0), g.d_twN, out, g.d_ef_off, stride, plan->d_status, plan->wait_budget);
     return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
 }
 
 }  // namespace
 
-size_t efield_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words)
+size_t efield_smem_bytes(int N, int P, int rows, int rrows, int A, int K, int nker, bool taps, int words)
 {
-    return efield_smem(P, efield_pairs(N, P), N, rows, A, K, nker, taps, words).total;
+    return efield_smem(P, efield_pairs(N, P), N, rows, rrows, A, K, nker, taps, words).total;
+}
+
+int efield_rows(int N, const std::vector<int4> &lchan)
+{
+    int most = 0;
+    for (size_t i = 0; i < lchan.size(); i += 2)
+        most = std::max(most, lchan[i].z + efield_place(N, lchan[i].z, lchan[i].w, lchan[i + 1].x, lchan[i + 1].y).dy);
+    return most;
 }
 
 int prepare_efield(const epic_plan_s *plan, const GroupCfg &g)
 {
-    const size_t need = efield_smem_bytes(g.N, plan->P, g.crows, plan->A, plan->K, plan->nker, g.etaps, g.estage ? g.cwords : 0);
+    const size_t need = efield_smem_bytes(g.N, plan->P, g.crows, g.erows, plan->A, plan->K, plan->nker, g.etaps, g.estage ? g.cwords : 0);
     return efield_dispatch(g, plan->P, [&](auto q_, auto p_, auto pr_) {
         constexpr int Q = decltype(q_)::value, P = decltype(p_)::value, PAIRS = decltype(pr_)::value;
         return plan->nker > 1 ? raise_dyn_smem_cap(reinterpret_cast<const void *>(efield_kernel<Q, P, PAIRS, true>), need)

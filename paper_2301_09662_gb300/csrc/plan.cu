@@ -824,9 +824,11 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 };
                 // the planes must fit; then the antennas' kernels, then the lists (else through L1)
                 auto ef_fits = [&](bool taps, int words) {
-                    return epic::efield_smem_bytes(g.N, n_pol, g.crows, n_ant, p->K, p->nker, taps, words) + 64 <=
+                    return epic::efield_smem_bytes(g.N, n_pol, g.crows, g.erows, n_ant, p->K, p->nker, taps, words) + 64 <=
                            static_cast<size_t>(smem_optin);
                 };
+                g.erows = epic::efield_rows(g.N, lchan);
+                if (!ef_fits(false, 0)) g.erows = g.crows;
                 g.compact = fits(false, 0) && ef_fits(false, 0);
                 g.ctaps = p->nker > 1 && fits(true, 0);
                 g.cstage = fits(g.ctaps, g.cwords) && !(diag & EPIC_DIAG_GATHER_GLOBAL);

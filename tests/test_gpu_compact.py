@@ -52,3 +52,26 @@ def test_efield_keeps_the_origin_phase(N, P, T):
     p.close()
     ref = oracle.workload_efield(wl)
     assert np.max(np.abs(got - ref)) / np.max(np.abs(ref)) < TOL
+
+
+@pytest.mark.parametrize("N,left,right", [
+    (128, 31, 30),     # from the quarter on, 62 cells + the kernel's
+    (128, 36, 23),     # begins before the quarter and ends past cell 64: the factor from the table
+    (96, 30, 30),      # the same at side 96, from cell 18 - 1
+    (64, 20, 26),      # begins before the quarter, fits from the corner
+])
+def test_efield_placements(N, left, right):
+    wl = synth.random_small(A=36, P=2, C=2, T=2, N=N, K=3, seed=left)
+    cell = synth.C0 / wl.freq_hz[0] * wl.du
+    rng = np.random.default_rng(N + left)
+    for axis in (0, 1):
+        x = rng.uniform(-8, 8, 36)
+        x[0], x[1] = -left, right
+        x[2:] -= x.sum() / 34
+        wl.ant_xy[:, axis] = x * cell
+    p = epic.Plan.from_workload(wl)
+    v, g = torch_inputs(wl)
+    got = p.image_efield(v, g).cpu().numpy().astype(np.complex128)
+    p.close()
+    ref = oracle.workload_efield(wl)
+    assert np.max(np.abs(got - ref)) / np.max(np.abs(ref)) < TOL
