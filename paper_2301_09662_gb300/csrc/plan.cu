@@ -901,15 +901,19 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                     const int most = static_cast<int>(std::max<size_t>(1, kBudget / (per * g.wtb)));
                     const int n_grp = (g.n_chan + most - 1) / most;
                     g.wcb = (g.n_chan + n_grp - 1) / n_grp;
-                    g.wide = true;
-                    g.wforce = cap_tb > 0;
+                    // no room for the workspace: the paths below need less or none (the fold path's
+                    // own batches, per-class gridding)
+                    g.wide = dev_upload(&g.d_wws, static_cast<const float2 *>(nullptr),
+                                        per / sizeof(float2) * g.wcb * g.wtb) == EPIC_OK;
+                    if (!g.wide) cudaGetLastError();
+                }
+                if (g.wide) {
+                    g.wforce = ((diag >> 16) & 255u) > 0;
                     g.wgains = epic::wide_rows_smem_bytes(n_ant, p->K, true) + 64 <= static_cast<size_t>(smem_optin);
                     g.tau_cap = std::max(g.tau_cap, epic::wide_pick_tau(g, max_spectra, p->sm_count));
                     rc = dev_upload(&g.d_wtab, wtab.data(), wtab.size());
                     if (rc == EPIC_OK) rc = dev_upload(&g.d_widx, widx.data(), widx.size());
                     if (rc == EPIC_OK) rc = dev_upload(&g.d_wchan, wchan.data(), wchan.size());
-                    if (rc == EPIC_OK)
-                        rc = dev_upload(&g.d_wws, static_cast<const float2 *>(nullptr), per / sizeof(float2) * g.wcb * g.wtb);
                 }
             }
             // large sides with one shared kernel of more than one tap: grid once per (channel,

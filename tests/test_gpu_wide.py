@@ -68,3 +68,17 @@ def test_delays_against_the_per_class_kernel(N):
         out.append(p.image(v, g, delays=d).cpu().numpy().astype(np.complex128))
         p.close()
     assert peak_rel_err(out[0], out[1], wl.grid_n, 2).max() < TOL
+
+
+def test_no_room_for_the_workspace():
+    """1.5 GiB of device memory left, the workspace wants 4: the plan is made and images per class."""
+    import torch
+    wl = _case(256, 60, 3, 5, 100, 90)
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (3 << 29), dtype=torch.uint8, device="cuda")
+    p = epic.Plan.from_workload(wl, max_spectra=16384)
+    got, _ = run_gpu(wl, plan=p)
+    p.close()
+    del hold
+    torch.cuda.empty_cache()
+    assert peak_rel_err(got, oracle.workload_image(wl), wl.grid_n, 2).max() < TOL
