@@ -125,20 +125,13 @@ def fp32_flops_per_spectrum(A, K, N):
 
 
 def kernel_source_hash(form):
-    """Hash of the device code of the imaging kernel a form runs at grid side
-    128: the FP32 register kernel (fp32_reg64.cu up to its large-side part, and
-    the transform headers) or the tensor pair kernel (tc_pair128.cu and the
-    tensor helpers)."""
+    """Hash of the source of the imaging kernel a form runs on the LWA-like
+    workload: the compact FP32 kernel (fp32_compact.cu and its transforms) or
+    the tensor pair kernel (tc_pair128.cu and the tensor helpers)."""
     csrc = os.path.join(ROOT, "paper_2301_09662_gb300", "csrc")
-    if form == "fp32":
-        src = open(os.path.join(csrc, "fp32_reg64.cu")).read()
-        start = src.index("// Register transforms of the folded side M")
-        end = src.index("// Large grid sides: the folded grids", start)
-        h = hashlib.sha256(src[start:end].encode())
-        files = ("fft64.cuh", "dft_small.cuh")
-    else:
-        h = hashlib.sha256()
-        files = ("tc_pair128.cu", "tc_common.cuh", "tc_ptx.cuh", "dft_small.cuh")
+    h = hashlib.sha256()
+    files = (("fp32_compact.cu", "fft_class.cuh", "fft64.cuh", "fft48.cuh", "dft_small.cuh", "tc_ptx.cuh")
+             if form == "fp32" else ("tc_pair128.cu", "tc_common.cuh", "tc_ptx.cuh", "dft_small.cuh"))
     for f in files:
         with open(os.path.join(csrc, f), "rb") as fh:
             h.update(fh.read())
@@ -414,8 +407,8 @@ def time_variants(wl, v, g, out, flush, args, stream):
              "fp32_antenna_kernels": dict(flags=epic.EPIC_ANTENNA_KERNELS),
              "fp32_series_stokes": dict(flags=epic.EPIC_STOKES),
              "fp32_efield": dict()}
-    notes = {"fp32": "plain FP32 form: gather gridding, register 64-point FFTs on packed FP32 pairs, products "
-                     "summed in registers (literal gridding)",
+    notes = {"fp32": "plain FP32 form: gather gridding of the occupied cells, register 64-point FFTs on packed FP32 "
+                     "pairs, products summed in tensor memory (literal gridding)",
              "kernel_taper": "FP32; image-domain |W^|^2 taper with point gridding (exact for one shared kernel)",
              "tc_split_fp16": "row and column DFTs on tcgen05, FP16 hi+lo operands (3 MMAs per k-block), "
                               "FP32 accumulate in TMEM; at grid side 128 two pixel classes per CTA share one "
@@ -433,7 +426,7 @@ def time_variants(wl, v, g, out, flush, args, stream):
                                    f"{SERIES_SPI} spectra ({wl.T // SERIES_SPI if wl.T % SERIES_SPI == 0 else 0} "
                                    f"images per integration)",
              "fp32_efield": "epic_image_efield: the complex E-field image of every sample, channel and "
-                            "polarisation (FP32 register kernel, no products), written to HBM"}
+                            "polarisation (FP32 pair kernel, no products), written to HBM"}
     import copy
 
     from paper_2301_09662_gb300 import synth
