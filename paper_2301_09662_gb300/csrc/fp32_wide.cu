@@ -611,14 +611,16 @@ int wide_pick_tau(const GroupCfg &g, int T, int sms)
     return g.N == 512 ? n : std::max(n, fp32_pick_tau(g.n_items, T, sms));
 }
 // Whether an integration of T spectra is worth the two launches: for the smallest the per-class
-// kernel's single launch is shorter.  Its work goes as the classes times gridding and transform; one
+// kernel's single launch is shorter.  Its time goes as the classes times transform and gridding, a
+// footprint cell weighing three times the arithmetic's share (lists and shared-memory reads).  One
 // GB300, us wide / per class: side 256, 300 antennas, 5 x 5, 2 channels x 16 spectra 40 / 34, 4 x 16
-// 46 / 50; 2048 antennas, 7 x 7, 1 x 8 45 / 63; side 512, 64 antennas, 3 x 3, 1 x 8 50 / 30, 2 x 16
-// 68 / 62, 4 x 16 102 / 110; 300 antennas, 5 x 5, 2 x 16 77 / 83.
+// 46 / 50; 2048 antennas, 7 x 7, 1 x 8 45 / 63; side 512, 2048 antennas, 7 x 7, 1 x 2 59 / 65, 1 x 4
+// 60 / 107; 1000 antennas, 7 x 7, 1 x 4 54 / 47, 1 x 8 58 / 72; 300 antennas, 5 x 5, 1 x 16 60 / 54,
+// 2 x 16 77 / 83; 64 antennas, 3 x 3, 2 x 16 109 / 97, 4 x 12 106 / 105.
 bool wide_pays(const epic_plan_s *plan, const GroupCfg &g, int T)
 {
-    const double work = static_cast<double>(g.n_items) * T * (static_cast<double>(plan->A) * plan->K * plan->K + 16384.0);
-    return g.wforce || work >= (g.N == 512 ? 4e7 : 1.4e7);
+    const double work = static_cast<double>(g.n_items) * T * (3.0 * plan->A * plan->K * plan->K + 16384.0);
+    return g.wforce || work >= (g.N == 512 ? 5.5e7 : 3e7);
 }
 static int wide_tau(const GroupCfg &g, int T, int sms) { return std::max(1, std::min(wide_pick_tau(g, T, sms), g.tau_cap)); }
 
