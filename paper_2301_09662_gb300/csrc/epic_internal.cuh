@@ -47,7 +47,8 @@ struct GroupCfg {
     long long *d_out_off = nullptr;    // device: output offset (complex elements) per group channel
     float2 *d_wpow = nullptr;          // device: |W^(l)|^2 on the shifted [N][N] layout, as FP32 pairs (hi, lo)
     double2 *d_tw64 = nullptr;         // per-antenna kernels: exp(+2 pi i k / N) in FP64
-    double2 *d_Y = nullptr;            // per-antenna kernels: [n_chan][3][2K-1][N] partial auto images
+    float4 *d_twp = nullptr;           // per-antenna kernels: (cos, -sin) of 2 pi k / N as FP32 pairs
+    float4 *d_Y = nullptr;             // per-antenna kernels: [n_chan][4][K][N] half-transformed auto grids, FP32 pairs
     float2 *d_twN = nullptr;           // device: exp(+2 pi i k / N), k < N
     int n_items = 0;                   // n_chan * Q
     int tau_cap = 1;                   // time chunks the partial buffer holds

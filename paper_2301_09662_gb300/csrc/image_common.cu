@@ -191,14 +191,15 @@ __device__ __forceinline__ void pair_msub(float2 &s, float2 a, float2 b)
 // image (auto_sum_kernel), not in every block.  Whole calls: 25 Stokes images of
 // 64 channels of 128 x 128 5.21 -> 3.66 ms, 64 channels of 512 x 512 with 2048
 // antennas 21.75 -> 20.40 ms.
-template <int N, int M, int P>
-__global__ void __launch_bounds__(kThreads)
+// AK: an auto image from the per-antenna auto-correlation grids (Yauto) instead of A_pq |W^|^2
+template <int N, int M, int P, bool AK>
+__global__ void __launch_bounds__(kThreads, 4)
 epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R1, int R2,
                 const int *__restrict__ chans, const long long *__restrict__ out_off,
                 const float2 *__restrict__ wpow, const double *__restrict__ apq_tab, const int *__restrict__ autoint,
                 int auto_n, size_t auto_stride,
                 const float2 *__restrict__ gains, int A, int C, int T, unsigned flags, float2 *__restrict__ out,
-                long long out_stride, const double2 *__restrict__ Yauto, const double2 *__restrict__ tw64, int K)
+                long long out_stride, const float4 *__restrict__ Yauto, const float4 *__restrict__ twp, int K)
 {
     constexpr int NPF = P == 2 ? 4 : 1;          // sums and products per pixel
     constexpr int up = N < M ? M / N : 1, Q1 = N < M ? 1 : N / M, Q = Q1 * Q1, NN = N * N;
@@ -210,16 +211,15 @@ epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R
     const int ci = blockIdx.y;
     const int c = chans[ci];
     const bool autosub = !(flags & EPIC_NO_AUTOSUB);
-    const bool ant_kernels = Yauto != nullptr;   // auto image from the per-antenna auto-correlation grid
 
     __shared__ double red[kThreads / 32][4];
     __shared__ double apq[4];   // XX, YY, Re XY, Im XY (YX = conj XY)
-    if (autosub && !ant_kernels && !apq_tab)
+    if (autosub && !AK && !apq_tab)
         auto_reduce<P>(autoint + static_cast<size_t>(img) * auto_n * auto_stride, auto_n, auto_stride, gains, A, c, red, apq);
     float2 aq[NPF];
 #pragma unroll
     for (int k = 0; k < NPF; k++)
-        aq[k] = autosub && !ant_kernels ? to_pair(apq_tab ? apq_tab[(static_cast<size_t>(img) * C + c) * 4 + k] : apq[k])
+        aq[k] = autosub && !AK ? to_pair(apq_tab ? apq_tab[(static_cast<size_t>(img) * C + c) * 4 + k] : apq[k])
                                         : make_float2(0.f, 0.f);
 
     const double scale = ((flags & EPIC_MEAN) && T > 0) ? 1.0 / T : 1.0;
@@ -231,6 +231,8 @@ epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R
         const int item = ci * Q + hy * Q1 + hx;
         const int px = up * (R1 == 1 ? mx : R2 * (mx % 8) + mx / 8), py = up * (R1 == 1 ? my : R2 * (my % 8) + my / 8);
         const size_t pos = static_cast<size_t>(py) * M + px;
+        float2 w = make_float2(0.f, 0.f);
+        if constexpr (!AK) w = __ldg(wpow + pix);
         // time chunks added in time order as compensated FP32 (hi, lo) pairs: TwoSum keeps
         // hi + lo equal to the exact running sum up to the roundings of lo, far below FP32
         float2 s[NPF];
@@ -251,31 +253,29 @@ epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R
                 s[0].y += two_sum(s[0].x, __ldg(src));
             }
         }
-        if (ant_kernels) {
+        if constexpr (AK) {
             if (autosub) {
-                // auto_pq(l) = sum_{rho_y} Y_pq(rho_y, l_x) exp(+2 pi i rho_y l_y / N)
-                const int R = 2 * K - 1;
-                const int lyv = i - N / 2;
-                double ax = 0, ay = 0, axr = 0, axi = 0;
-                for (int ry = 0; ry < R; ry++) {
-                    const int m = (((ry - (K - 1)) * lyv) % N + N) % N;
-                    const double2 tw = tw64[m];
-                    const double2 y0 = Yauto[(static_cast<size_t>(ci) * 3 * R + ry) * N + j];
-                    ax += y0.x * tw.x - y0.y * tw.y;
-                    if (P == 2) {
-                        const double2 y1 = Yauto[(static_cast<size_t>(ci) * 3 * R + R + ry) * N + j];
-                        const double2 y2 = Yauto[(static_cast<size_t>(ci) * 3 * R + 2 * R + ry) * N + j];
-                        ay += y1.x * tw.x - y1.y * tw.y;
-                        axr += y2.x * tw.x - y2.y * tw.y;
-                        axi += y2.x * tw.y + y2.y * tw.x;
+                // the auto image sum_{rho_y >= 0} Re(Y(rho_y, l_x) exp(+2 pi i rho_y l_y / N)), in pairs
+                const float4 *y = Yauto + static_cast<size_t>(ci) * 4 * K * N + j;   // [4][K][N]
+#pragma unroll
+                for (int k = 0; k < NPF; k++) {
+                    const float4 y0 = __ldg(y + static_cast<size_t>(k) * K * N);
+                    s[k].y += two_sum(s[k].x, -y0.x) - y0.y;
+                }
+                int m = 0;
+                for (int ry = 1; ry < K; ry++) {
+                    m += ly;
+                    if (m >= N) m -= N;
+                    const float4 tw = __ldg(twp + m);            // (cos, -sin)
+#pragma unroll
+                    for (int k = 0; k < NPF; k++) {
+                        const float4 yk = __ldg(y + (static_cast<size_t>(k) * K + ry) * N);
+                        pair_msub(s[k], make_float2(yk.x, yk.y), make_float2(tw.x, tw.y));
+                        pair_msub(s[k], make_float2(yk.z, yk.w), make_float2(tw.z, tw.w));
                     }
                 }
-                const double au[4] = {ax, ay, axr, axi};
-#pragma unroll
-                for (int k = 0; k < NPF; k++) s[k] = to_pair((static_cast<double>(s[k].x) + static_cast<double>(s[k].y)) - au[k]);
             }
         } else {
-            const float2 w = __ldg(wpow + pix);
             if (flags & EPIC_KERNEL_TAPER) {
                 // point-gridded sums: subtract the bare autos, then apply |W^(l)|^2
 #pragma unroll
@@ -325,64 +325,94 @@ epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R
 // sum_a A_a,pq |W^_a(l)|^2 = sum_rho X_pq(rho) exp(+2 pi i rho.l / N) with the
 // auto-correlation grid X_pq(rho) = sum_a A_a,pq B_aa(rho),
 // B_aa = W_a (x) W_a^* on the (2K-1)^2 offsets rho (Sec. 2.2's "auto-correlation
-// grids from individual antenna voltages").  One block per (channel, product):
-// X in FP64, then the l_x half of the separable transform,
-// Y(rho_y, l_x) = sum_rho_x X(rho_x, rho_y) exp(+2 pi i rho_x l_x / N), for the
-// epilogue to finish along l_y.
+// grids from individual antenna voltages").  The real and imaginary parts of A_XY
+// make grids of their own, so all four grids are Hermitian, their images real and
+// rows rho_y < 0 the conjugates of the others: K rows are enough.  One block per
+// (channel, grid): X in FP64, each antenna's weight once, then the l_x half of the
+// separable transform, Y(rho_y, l_x) = sum_rho_x X(rho_x, rho_y) exp(+2 pi i rho_x
+// l_x / N), doubled for rho_y > 0 and stored as FP32 pairs for the epilogue to
+// finish along l_y.  Bound by the FP64 pipe (2 operations a clock and SM), as the
+// epilogue was when it summed the 2K - 1 rows of complex grids in FP64: 250 spectra
+// of 64 channels of 128 x 128, 256 antennas, 5 x 5 kernels, whole call: 1.575 -> 0.988 ms
+// (the two kernels 0.68 -> 0.10).
+constexpr int kRhoTile = 512;                    // antennas whose weights are held at once
+
 __global__ void __launch_bounds__(kThreads)
 auto_rho_kernel(const int *__restrict__ autoint, const float2 *__restrict__ gains,
                 const double2 *__restrict__ bauto, const int *__restrict__ chans, const double2 *__restrict__ tw64,
-                int A, int P, int K, int N, double2 *__restrict__ Y)
+                int A, int P, int K, int N, int parts, float4 *__restrict__ Y)
 {
-    extern __shared__ double2 X[];     // [R][R]
-    const int R = 2 * K - 1, RR = R * R;
-    const int ci = blockIdx.x, pq = blockIdx.y;
+    extern __shared__ double2 X[];               // [parts][K][R]
+    __shared__ double wt[kRhoTile];
+    const int R = 2 * K - 1, RR = R * R, KR = K * R;
+    const int ci = blockIdx.x, pq = blockIdx.y;  // XX, YY, Re XY, Im XY
     const int c = chans[ci];
-    for (int rho = threadIdx.x; rho < RR; rho += blockDim.x) {
+    for (int base = 0; base < parts * KR; base += kThreads) {   // (parts > 1: once)
+        const int idx = base + threadIdx.x, rho = idx % KR, part = idx / KR;
         double xr = 0, xi = 0;
-        for (int a = 0; a < A; a++) {
-            const int *ia = autoint + (static_cast<size_t>(c) * A + a) * 4;
-            double ar, ai;
-            double gxr = 1, gxi = 0, gyr = 1, gyi = 0;
-            if (gains) {
-                const float2 gx = gains[(static_cast<size_t>(c) * A + a) * P];
-                gxr = gx.x;
-                gxi = gx.y;
-                if (P == 2) {
-                    const float2 gy = gains[(static_cast<size_t>(c) * A + a) * P + 1];
-                    gyr = gy.x;
-                    gyi = gy.y;
+        for (int a0 = 0; a0 < A; a0 += kRhoTile) {
+            const int na = min(kRhoTile, A - a0);
+            __syncthreads();
+            for (int i = threadIdx.x; i < na; i += kThreads) {
+                const size_t ca = static_cast<size_t>(c) * A + a0 + i;
+                const int *ia = autoint + ca * 4;
+                double gxr = 1, gxi = 0, gyr = 1, gyi = 0;
+                if (gains) {
+                    const float2 gx = gains[ca * P];
+                    gxr = gx.x;
+                    gxi = gx.y;
+                    if (P == 2) {
+                        const float2 gy = gains[ca * P + 1];
+                        gyr = gy.x;
+                        gyi = gy.y;
+                    }
+                }
+                const double pr = gxr * gyr + gxi * gyi, pi = gxi * gyr - gxr * gyi;
+                wt[i] = pq == 0   ? (gxr * gxr + gxi * gxi) * ia[0]
+                        : pq == 1 ? (gyr * gyr + gyi * gyi) * ia[1]
+                        : pq == 2 ? pr * ia[2] - pi * ia[3]
+                                  : pr * ia[3] + pi * ia[2];
+            }
+            __syncthreads();
+            if (idx < parts * KR) {
+                const double2 *b = bauto + static_cast<size_t>(a0) * RR + (K - 1) * R + rho;   // rows rho_y >= 0
+#pragma unroll 8
+                for (int i = part; i < na; i += parts) {
+                    const double2 v = __ldg(b + static_cast<size_t>(i) * RR);
+                    xr = fma(wt[i], v.x, xr);
+                    xi = fma(wt[i], v.y, xi);
                 }
             }
-            if (pq == 0) {
-                ar = (gxr * gxr + gxi * gxi) * ia[0];
-                ai = 0;
-            } else if (pq == 1) {
-                ar = (gyr * gyr + gyi * gyi) * ia[1];
-                ai = 0;
-            } else {
-                const double pr = gxr * gyr + gxi * gyi, pi = gxi * gyr - gxr * gyi;
-                ar = pr * ia[2] - pi * ia[3];
-                ai = pr * ia[3] + pi * ia[2];
-            }
-            const double2 b = bauto[static_cast<size_t>(a) * RR + rho];
-            xr += ar * b.x - ai * b.y;
-            xi += ar * b.y + ai * b.x;
         }
-        X[rho] = make_double2(xr, xi);
+        if (idx < parts * KR) X[idx] = make_double2(xr, xi);
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < R * N; e += blockDim.x) {
-        const int ry = e / N, j = e % N;
-        const int lx = j - N / 2;
-        double yr = 0, yi = 0;
-        for (int rx = 0; rx < R; rx++) {
-            const int m = (((rx - (K - 1)) * lx) % N + N) % N;
-            const double2 tw = tw64[m], x = X[ry * R + rx];
-            yr += x.x * tw.x - x.y * tw.y;
-            yi += x.x * tw.y + x.y * tw.x;
+    if (parts > 1) {
+        for (int rho = threadIdx.x; rho < KR; rho += kThreads) {
+            double2 x = X[rho];
+            for (int p = 1; p < parts; p++) {
+                x.x += X[p * KR + rho].x;
+                x.y += X[p * KR + rho].y;
+            }
+            X[rho] = x;
         }
-        Y[(static_cast<size_t>(ci) * 3 * R + static_cast<size_t>(pq) * R + ry) * N + j] = make_double2(yr, yi);
+        __syncthreads();
+    }
+    for (int e = threadIdx.x; e < K * N; e += kThreads) {
+        const int ry = e / N, j = e % N;
+        const int lx = j < N / 2 ? j + N / 2 : j - N / 2;       // (j - N / 2) mod N
+        double yr = 0, yi = 0;
+        int m = ((N - lx) * (K - 1)) % N;                        // rho_x l_x mod N from rho_x = -(K - 1) on
+        for (int rx = 0; rx < R; rx++) {
+            const double2 tw = __ldg(tw64 + m), x = X[ry * R + rx];
+            yr = fma(-x.y, tw.y, fma(x.x, tw.x, yr));
+            yi = fma(x.y, tw.x, fma(x.x, tw.y, yi));
+            m += lx;
+            if (m >= N) m -= N;
+        }
+        const double f = ry ? 2.0 : 1.0;
+        const float2 re = to_pair(f * yr), im = to_pair(f * yi);
+        Y[((static_cast<size_t>(ci) * 4 + pq) * K + ry) * N + j] = make_float4(re.x, re.y, im.x, im.y);
     }
 }
 
@@ -427,11 +457,12 @@ int launch_epi(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T,
         constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
         const dim3 grid(static_cast<unsigned>(epi_tiles(N, g.n_chan * n_img, plan->sm_count)), static_cast<unsigned>(g.n_chan),
                         static_cast<unsigned>(n_img));
-        epilogue_kernel<N, M, P><<<grid, kThreads, 0, stream>>>(
+        const auto kfn = plan->nker > 1 ? epilogue_kernel<N, M, P, true> : epilogue_kernel<N, M, P, false>;
+        kfn<<<grid, kThreads, 0, stream>>>(
             g.d_partial, n_tau, g.n_items, g.R1, g.R2, g.d_chans, g.d_out_off, g.d_wpow,
             auto_in_epilogue(plan) ? nullptr : plan->d_apq, plan->d_autoint, auto_n, static_cast<size_t>(plan->C) * plan->A * 4,
             gains, plan->A, plan->C, T, plan->flags, out, static_cast<long long>(plan->out_floats / 2),
-            plan->nker > 1 ? g.d_Y : nullptr, g.d_tw64, plan->K);
+            g.d_Y, g.d_twp, plan->K);
         return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
     });
 }
@@ -481,7 +512,7 @@ int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, cud
     return epi_dispatch(r.N, r.M, r.P, [&](auto n_, auto m_, auto p_) {
         constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
         const dim3 grid(static_cast<unsigned>(epi_tiles(N, r.C, 148)), static_cast<unsigned>(r.C));
-        epilogue_kernel<N, M, P><<<grid, kThreads, 0, stream>>>(r.partial, r.n_tau, r.n_items, 8, M / 8, r.chans, r.out_off,
+        epilogue_kernel<N, M, P, false><<<grid, kThreads, 0, stream>>>(r.partial, r.n_tau, r.n_items, 8, M / 8, r.chans, r.out_off,
                                                                 r.wpow, nullptr, r.autoint, 1, 0, gains, r.A, r.C, r.T, r.flags,
                                                                 out, 0, nullptr, nullptr, 0);
         return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
@@ -530,10 +561,10 @@ int launch_delay_prep(epic_plan_s *plan, int T, cudaStream_t stream)
 
 int launch_auto_rho(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, cudaStream_t stream)
 {
-    const int R = 2 * plan->K - 1;
-    const dim3 grid(static_cast<unsigned>(g.n_chan), static_cast<unsigned>(plan->P == 2 ? 3 : 1));
-    auto_rho_kernel<<<grid, kThreads, sizeof(double2) * R * R, stream>>>(
-        plan->d_autoint, gains, plan->d_bauto, g.d_chans, g.d_tw64, plan->A, plan->P, plan->K, g.N, g.d_Y);
+    const int KR = plan->K * (2 * plan->K - 1), parts = std::max(1, std::min(8, kThreads / KR));
+    const dim3 grid(static_cast<unsigned>(g.n_chan), static_cast<unsigned>(plan->P == 2 ? 4 : 1));
+    auto_rho_kernel<<<grid, kThreads, sizeof(double2) * parts * KR, stream>>>(
+        plan->d_autoint, gains, plan->d_bauto, g.d_chans, g.d_tw64, plan->A, plan->P, plan->K, g.N, parts, g.d_Y);
     return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
 }
 

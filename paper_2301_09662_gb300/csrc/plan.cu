@@ -103,6 +103,7 @@ void free_plan(epic_plan_s *p)
         cudaFree(g.d_gidx);
         cudaFree(g.d_gchan);
         cudaFree(g.d_tw64);
+        cudaFree(g.d_twp);
         cudaFree(g.d_Y);
         cudaFree(g.d_ptab);
         cudaFree(g.d_pchan);
@@ -998,14 +999,18 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
         if (rc == EPIC_OK) rc = dev_upload(&g.d_twN, tw.data(), tw.size());
         if (rc == EPIC_OK && ant_kernels) {
             std::vector<double2> tw64(g.N);
+            std::vector<float4> twp(g.N);
             for (int k = 0; k < g.N; k++) {
-                const double ang = 2.0 * M_PI * k / g.N;
-                tw64[k] = make_double2(std::cos(ang), std::sin(ang));
+                const double ang = 2.0 * M_PI * k / g.N, co = std::cos(ang), si = std::sin(ang);
+                tw64[k] = make_double2(co, si);
+                const float ch = static_cast<float>(co), sh = static_cast<float>(-si);
+                twp[k] = make_float4(ch, static_cast<float>(co - ch), sh, static_cast<float>(-si - sh));
             }
             rc = dev_upload(&g.d_tw64, tw64.data(), tw64.size());
+            if (rc == EPIC_OK) rc = dev_upload(&g.d_twp, twp.data(), twp.size());
             if (rc == EPIC_OK)
-                rc = dev_upload(&g.d_Y, static_cast<const double2 *>(nullptr),
-                                static_cast<size_t>(g.n_chan) * 3 * (2 * K - 1) * g.N);
+                rc = dev_upload(&g.d_Y, static_cast<const float4 *>(nullptr),
+                                static_cast<size_t>(g.n_chan) * 4 * K * g.N);
         }
         if (rc == EPIC_OK)
             rc = dev_upload(&g.d_partial, static_cast<const float *>(nullptr),
