@@ -754,14 +754,30 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
     }
     if (rc == EPIC_OK && cudaMemset(p->d_status, 0, sizeof(int)) != cudaSuccess) rc = EPIC_ERR_CUDA;
 
-    // channel groups by grid side
-    std::map<int, std::vector<int>> by_n;
-    for (int c = 0; c < n_chan; c++) by_n[grid_n[c]].push_back(c);
+    // channel groups by grid side; at sides 256 and 512 those whose footprints span at most 128 x 128
+    // cells apart from wider ones, so that the wide kernels serve them whatever the others are (a
+    // 350 m array over 46.8 to 53.2 MHz: 256 channels x 500 spectra of 512 x 512 423 -> 173 ms)
+    std::map<std::pair<int, int>, std::vector<int>> by_n;
+    for (int c = 0; c < n_chan; c++) {
+        int narrow = 0;
+        if (!tensor && n_pol == 2 && !ant_kernels && (grid_n[c] == 256 || grid_n[c] == 512)) {
+            int x0 = 1 << 20, x1 = 0, y0 = 1 << 20, y1 = 0;
+            for (int a = 0; a < n_ant; a++) {
+                const short2 k = cells[static_cast<size_t>(c) * n_ant + a];
+                x0 = std::min<int>(x0, k.x);
+                x1 = std::max<int>(x1, k.x);
+                y0 = std::min<int>(y0, k.y);
+                y1 = std::max<int>(y1, k.y);
+            }
+            narrow = x1 - x0 + p->K <= 128 && y1 - y0 + p->K <= 128;
+        }
+        by_n[{grid_n[c], narrow}].push_back(c);
+    }
     const int npf = n_pol == 2 ? 4 : 1;
     for (auto &kv : by_n) {
         if (rc != EPIC_OK) break;
         GroupCfg g;
-        g.N = kv.first;
+        g.N = kv.first.first;
         g.Q1 = fold_for(g.N);
         g.M = g.N / g.Q1;
         if (tensor && g.N == 32) {
@@ -939,6 +955,10 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                     if (rc == EPIC_OK)
                         rc = dev_upload(&g.d_gf, static_cast<const float2 *>(nullptr), per_sample / sizeof(float2) * g.alias_tb);
                     g.alias = rc == EPIC_OK;
+                    if (rc == EPIC_ERR_NOMEM && !tensor) {   // no room: per class
+                        cudaGetLastError();
+                        rc = EPIC_OK;
+                    }
                 }
             }
             if (rc == EPIC_OK && g.tensor && !g.tc_regular && !g.alias) rc = EPIC_ERR_UNSUPPORTED;
@@ -1474,12 +1494,25 @@ int epic_stage_times(epic_plan_t plan, float *ms, int max_stages)
 {
     if (!plan || !ms || max_stages < 0) return EPIC_ERR_ARG;
     if (!plan->profiling || plan->n_recorded == 0) return EPIC_ERR_ARG;
-    const int n = plan->n_recorded < max_stages ? plan->n_recorded : max_stages;
     for (int i = 0; i < plan->n_recorded; i++)
         if (cudaEventSynchronize(plan->events[2 * i + 1]) != cudaSuccess) return EPIC_ERR_CUDA;
-    for (int i = 0; i < n; i++)
-        if (cudaEventElapsedTime(&ms[i], plan->events[2 * i], plan->events[2 * i + 1]) != cudaSuccess)
-            return EPIC_ERR_CUDA;
+    // the groups of one side (two at most, one after the other) are one stage: from the first start to
+    // the last end
+    const int lead = plan->n_recorded - 2 * static_cast<int>(plan->groups.size());   // the auto sums
+    int n = 0;
+    for (int i = 0; i < plan->n_recorded && n < max_stages; i++) {
+        const size_t gi = static_cast<size_t>(std::max(0, i - lead) / 2);
+        if (i >= lead && gi > 0 && plan->groups[gi].N == plan->groups[gi - 1].N) continue;   // counted already
+        const bool two = i >= lead && gi + 1 < plan->groups.size() && plan->groups[gi + 1].N == plan->groups[gi].N;
+        float most = 0.f;
+        for (int u = i; u <= (two ? i + 2 : i); u += 2)
+            for (int w = i; w <= (two ? i + 2 : i); w += 2) {
+                float t;
+                if (cudaEventElapsedTime(&t, plan->events[2 * u], plan->events[2 * w + 1]) != cudaSuccess) return EPIC_ERR_CUDA;
+                most = std::max(most, t);
+            }
+        ms[n++] = most;
+    }
     return n;
 }
 

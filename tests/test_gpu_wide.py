@@ -82,3 +82,17 @@ def test_no_room_for_the_workspace():
     del hold
     torch.cuda.empty_cache()
     assert peak_rel_err(got, oracle.workload_image(wl), wl.grid_n, 2).max() < TOL
+
+
+@pytest.mark.parametrize("flags", [0, epic.EPIC_DIAG_ALIAS_BATCH(3)])
+def test_channels_on_both_sides_of_the_range(flags):
+    """Two of three channels span at most 128 cells: a group each, one stage of the side."""
+    wl = _case(512, 40, 7, 5, 120, 110, C=3)
+    wl.freq_hz = wl.freq_hz[0] * np.array([1.0, 1.2, 0.9])
+    p = epic.Plan.from_workload(wl, flags=flags | (WIDE if not flags else 0))
+    p.set_profiling()
+    got, _ = run_gpu(wl, plan=p)
+    times = p.stage_times()
+    p.close()
+    assert peak_rel_err(got, oracle.workload_image(wl), wl.grid_n, 2).max() < TOL
+    assert sorted(times) == ["autopower", "epilogue[N=512]", "image[N=512]"] and min(times.values()) > 0
