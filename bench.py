@@ -50,19 +50,19 @@ L2_FLUSH_BYTES = 256 << 20
 # with the hash of the kernel source it was taken on; ignored (null) once the
 # source changes.  Filled in from the committed profiles/ summaries.
 NCU_TRAFFIC = {
-    ("lwa", "tc_split_fp16"): (197.21e6, "e16cc173ad5d718a"),     # profiles/tc_pair128_kernel_lwa.md
-    ("lwa", "fp32"): (144.11e6, "e8796ed7dfd2eaa3"),              # profiles/fp32_reg64_kernel_lwa.md
+    ("lwa", "tc_split_fp16"): (197.09e6, "3059080590207818"),     # profiles/tc_pair128_kernel_lwa.md
+    ("lwa", "fp32"): (207.89e6, "56cb6a9d84deedc1"),              # profiles/fp32_compact_kernel_lwa.md
 }
 # What the same capture shows about the kernel's limits (same keys and hashes).
 NCU_LIMITER = {
-    ("lwa", "tc_split_fp16"): ({"tensor_pipe_active_pct": 60.0, "issue_active_pct": 49.7, "warps_active_pct": 18.7,
-                               "smem_conflict_wavefront_share": 0.42,
-                               "top_stalls": "short_scoreboard 1.18, wait 1.04, long_scoreboard 0.62"},
-                              "e16cc173ad5d718a"),
-    ("lwa", "fp32"): ({"fma_pipe_active_pct": 41.9, "issue_active_pct": 45.2, "warps_active_pct": 12.5,
-                      "registers_per_thread": 228, "smem_conflict_wavefront_share": 0.20,
-                      "top_stalls": "wait 1.10, short_scoreboard 0.75, not_selected 0.44"},
-                     "e8796ed7dfd2eaa3"),
+    ("lwa", "tc_split_fp16"): ({"tensor_pipe_active_pct": 46.8, "issue_active_pct": 51.4, "warps_active_pct": 18.7,
+                               "smem_conflict_wavefront_share": 0.37,
+                               "top_stalls": "short_scoreboard 1.04, wait 1.04, not_selected 0.66"},
+                              "3059080590207818"),
+    ("lwa", "fp32"): ({"fma_pipe_active_pct": 55.1, "issue_active_pct": 54.7, "warps_active_pct": 18.7,
+                      "registers_per_thread": 162, "smem_conflict_wavefront_share": 0.15,
+                      "top_stalls": "wait 0.95, long_scoreboard 0.84, barrier 0.68"},
+                     "56cb6a9d84deedc1"),
 }
 
 

@@ -119,14 +119,16 @@ enum {
  * but an explicit flag turns one on.
  */
 #define EPIC_DIAG_NO_GRAPH       (1u << 8)   /* launch each kernel directly instead of replaying a CUDA graph */
-#define EPIC_DIAG_GATHER_GLOBAL  (1u << 9)   /* FP32 register kernel: read the gather table through L1 instead
+#define EPIC_DIAG_GATHER_GLOBAL  (1u << 9)   /* FP32 kernels: read the gather lists through L1 instead
                                                 of staging it in shared memory (bitwise the same result) */
-#define EPIC_DIAG_NO_ALIAS       (1u << 10)  /* 512 grid sides: grid per pixel class instead of folding */
+#define EPIC_DIAG_NO_ALIAS       (1u << 10)  /* 256 and 512 grid sides: grid per pixel class (neither wide
+                                                kernels nor folding) */
 #define EPIC_DIAG_WITHHOLD_MMA   (1u << 11)  /* fault injection: the tensor kernel issues no MMA, its bounded
                                                 wait (budget ~1 ms) runs out and epic_status reports
                                                 EPIC_ERR_TIMEOUT; the context stays usable */
-#define EPIC_DIAG_ALIAS_BATCH(n) ((((unsigned)(n)) & 255u) << 16)   /* fold path: at most n (1..255) samples
-                                                                        per time batch */
+#define EPIC_DIAG_ALIAS_BATCH(n) ((((unsigned)(n)) & 255u) << 16)   /* fold path and wide kernels: at most
+                                                                        n (1..255) samples per time batch;
+                                                                        small calls take them too */
 #define EPIC_DIAG_NO_PAIR        (1u << 12)  /* tensor form without the gather-gridding pair kernel (two
                                                 classes from one gridding at sides 128 and 96, its one
                                                 class at 64): sides 128 and 64 run the two-stage kernel
@@ -160,10 +162,13 @@ enum {
  * adjacent folded cells, the antennas whose footprints cover it: 4 bytes per
  * entry, about A * K * (K + 1) / 2 entries plus padding; 43 KB per channel at
  * A = 256, K = 5), staged in shared memory by the kernel when they fit.
- * Channels with a 512 grid side and one shared kernel wider than one tap are
- * imaged by gridding each (channel, sample) once and folding the 64 pixel
- * classes from it: their workspace adds the folded class grids of one time
- * batch, up to 4 GiB (C * 64 * n_pol * 32 KB per spectrum, batched).  Returns
+ * FP32 channels with a 256 or 512 grid side, both polarisations, one shared
+ * kernel and footprints within 128 x 128 cells add a workspace of transformed
+ * rows of up to 4 GiB (N * 16 bytes per occupied row and spectrum, batched);
+ * other channels with a 512 grid side and one shared kernel wider than one tap
+ * add the folded class grids of one time batch, up to 4 GiB (C * 64 * n_pol *
+ * 32 KB per spectrum, batched).  FP32 plans without room for either grid per
+ * pixel class, more slowly.  Returns
  * EPIC_ERR_OUT_OF_GRID when some antenna footprint k_a +- (K-1)/2 leaves
  * [0, N_c) in some channel; EPIC_ERR_UNSUPPORTED for a grid side, precision or
  * size this build does not provide.
