@@ -165,6 +165,7 @@ gain_solve_cluster_kernel(const uint8_t *__restrict__ v, const short2 *__restric
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
+    cl.barrier_arrive();                             // met before the first store to another CTA's shared memory
     const int rank = static_cast<int>(cl.block_rank()), CL = static_cast<int>(cl.num_blocks());
     extern __shared__ float2 sm[];
     const int AP = A * P;
@@ -184,7 +185,9 @@ gain_solve_cluster_kernel(const uint8_t *__restrict__ v, const short2 *__restric
     const int i0 = static_cast<int>(static_cast<long long>(AP) * rank / CL);
     const int i1 = static_cast<int>(static_cast<long long>(AP) * (rank + 1) / CL);
 
-    // the lattice phases of the CTA's slice, to every CTA of the cluster
+    // the lattice phases of the CTA's slice, to every CTA of the cluster; another CTA's shared memory may be
+    // accessed only once that CTA runs
+    cl.barrier_wait();
     for (int i = i0 + tid; i < i1; i += kCalThreads) {
         const short2 k = cells[static_cast<size_t>(c) * A + i / P];
         double turns = (static_cast<double>(k.x) * lx + static_cast<double>(k.y) * ly) / N;
