@@ -211,9 +211,9 @@ int launch_epilogue(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, i
 int launch_auto_rho(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, cudaStream_t stream);
 // delay table of the current call (plan->delays, [T][A] seconds) into plan->d_dtab
 int launch_delay_prep(epic_plan_s *plan, int T, cudaStream_t stream);
-// image series: per-image auto sums and one epilogue image per time chunk
+// image series: per-image auto sums, and an epilogue image per n_tau time chunks
 int launch_autopower_series(epic_plan_s *plan, const uint8_t *v, const float2 *gains, int spi, int n_img, cudaStream_t stream);
-int launch_epilogue_series(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int spi, int n_img,
+int launch_epilogue_series(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int spi, int n_img, int n_tau,
                            float2 *out, cudaStream_t stream);
 // imaging kernel of one group (FP32 or tensor form as the plan says)
 int launch_imaging(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
@@ -297,6 +297,7 @@ struct RawImage {
 };
 int fp32_pick_tau(int n_items, int T, int sms);
 int compact_pick_tau(int n_chan, int n_items, int T, int sms);
+int series_chunks(int n_chan, int n_img, int spi, int tau_cap, int sms);   // compact kernel: time chunks per image
 // time chunks of one launch: forced (image series), else autotuned for this T, else the cost model
 int choose_tau(const epic_plan_s *plan, const GroupCfg &g, int T);
 // large grid sides (GroupCfg::alias)

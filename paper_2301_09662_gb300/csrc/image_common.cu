@@ -544,10 +544,10 @@ int launch_autopower_series(epic_plan_s *plan, const uint8_t *v, const float2 *g
     return rc != EPIC_OK ? rc : launch_auto_sum(plan, gains, 1, n_img, stream);
 }
 
-int launch_epilogue_series(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int spi, int n_img,
+int launch_epilogue_series(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int spi, int n_img, int n_tau,
                            float2 *out, cudaStream_t stream)
 {
-    return launch_epi(plan, g, gains, spi, 1, n_img, 1, out, stream);
+    return launch_epi(plan, g, gains, spi, n_tau, n_img, 1, out, stream);
 }
 
 int launch_delay_prep(epic_plan_s *plan, int T, cudaStream_t stream)

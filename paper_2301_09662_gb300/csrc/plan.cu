@@ -1293,12 +1293,13 @@ int epic_image_series_ex(epic_plan_t plan, const uint8_t *ci4, const float *gain
         // the batch's delays, time-indexed from the batch's first spectrum like its voltages
         plan->delays = delays_s ? delays_s + static_cast<size_t>(i0) * spi * plan->A : nullptr;
         if (rc == EPIC_OK && plan->delays) rc = epic::launch_delay_prep(plan, spi * b, s);
-        plan->force_tau = b;   // one time chunk per image
         for (const auto &g : plan->groups) {
             if (rc != EPIC_OK) break;
             int n_tau = 0;
+            const int per = g.compact ? epic::series_chunks(g.n_chan, b, spi, g.tau_cap, plan->sm_count) : 1;
+            plan->force_tau = b * per;   // chunks of one image each, per of them to an image
             rc = epic::launch_imaging(plan, g, vb, g2, spi * b, &n_tau, s);
-            if (rc == EPIC_OK) rc = epic::launch_epilogue_series(plan, g, g2, spi, b, ob, s);
+            if (rc == EPIC_OK) rc = epic::launch_epilogue_series(plan, g, g2, spi, b, per, ob, s);
         }
         plan->force_tau = 0;
         plan->delays = nullptr;

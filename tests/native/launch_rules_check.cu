@@ -1,0 +1,46 @@
+// Host-side check of the rules that choose a call's launch shape (no GPU needed): a rule leaves no SM
+// idle that the work could use, and stays within the buffers the plan has.
+// Usage: launch_rules_check   (exit status 0 when every check holds)
+#include <algorithm>
+#include <cstdio>
+
+#include "epic_internal.cuh"
+
+static long g_bad = 0;
+#define CHECK(cond, ...)                  \
+    do {                                  \
+        if (!(cond)) {                    \
+            if (g_bad < 20) {             \
+                std::printf(__VA_ARGS__); \
+                std::printf("\n");        \
+            }                             \
+            g_bad++;                      \
+        }                                 \
+    } while (0)
+
+// Image series in the compact kernel: one CTA per channel and time chunk, so a batch of few images
+// splits each, within the partial images of the plan.
+static void series()
+{
+    for (int sms : {148, 152})
+        for (int chan : {1, 3, 12, 32, 64, 200})
+            for (int img : {1, 2, 3, 10, 25})
+                for (int spi : {1, 8, 40, 100, 1000})
+                    for (int cap : {img, 2 * img + 1, 64}) {
+                        const int n = epic::series_chunks(chan, img, spi, cap, sms);
+                        CHECK(n >= 1 && n * img <= std::max(cap, img) && n <= spi, "%d chunks of %d x %d spectra, cap %d", n, img,
+                              spi, cap);
+                        // the batch's time, in samples on the busiest SM (4 for set-up and partial image)
+                        auto cost = [&](int k) { return ((chan * img * k + sms - 1) / sms) * ((spi + k - 1) / k + 4.0); };
+                        for (int k = 1; k * img <= cap && k <= spi; k++)
+                            CHECK(cost(n) <= cost(k) + 1e-9, "%d channels, %d x %d spectra: %d chunks cost %g, %d cost %g", chan,
+                                  img, spi, n, cost(n), k, cost(k));
+                    }
+}
+
+int main()
+{
+    series();
+    if (g_bad) std::printf("%ld checks failed\n", g_bad);
+    return g_bad ? 1 : 0;
+}

@@ -109,3 +109,21 @@ def test_stokes_output():
         peak = max(np.abs(xx).max(), np.abs(yy).max())
         assert np.max(np.abs(a.real - stokes)) / peak < 2 * FP32_TOL
         assert np.all(a.imag == 0)
+
+
+@pytest.mark.parametrize("N,P,spi,n_img", [(128, 2, 50, 1), (96, 1, 33, 3), (64, 2, 21, 2), (128, 1, 7, 5)])
+def test_few_images_in_several_time_chunks(N, P, spi, n_img):
+    """A batch of few images leaves SMs idle at one time chunk each (a CTA per channel), so an image
+    is summed from several, odd lengths among them; delays too.  FP32 sums of at most 50 spectra."""
+    import torch
+    wl = synth.random_small(A=40, P=P, C=2, T=spi * n_img, N=N, K=3, seed=spi)
+    p = epic.Plan.from_workload(wl)
+    v, g = torch_inputs(wl)
+    d = synth.geometric_delays(wl.ant_xy, wl.T)
+    got = p.image_series(v, spi, g, delays=torch.from_numpy(d).cuda())
+    assert p.status() == epic.EPIC_OK
+    got = got.cpu().numpy().astype(np.complex128)
+    p.close()
+    for i in range(n_img):
+        ref = oracle.workload_image(_block(wl, i * spi, (i + 1) * spi), delays=d[i * spi:(i + 1) * spi])
+        assert peak_rel_err(got[i], ref, wl.grid_n, P).max() < FP32_TOL
