@@ -74,6 +74,7 @@ struct GroupCfg {
     bool gstage = false;               // blocks staged in shared memory
     // FP32 plans whose aperture occupies at most 64 x 64 cells: the compact kernel (fp32_compact.cu)
     bool compact = false;
+    bool cimage = false;               // its images too (compact_pays), else only its E-field images
     bool cstage = false;               // its gather lists are staged in shared memory
     bool ctaps = false;                // and, with a kernel per antenna, the kernels
     bool estage = false, etaps = false;   // the same for its E-field form (fp32_efield.cu)
@@ -249,6 +250,7 @@ int build_gather_table(const std::vector<short2> &cells, int A, int K, int M, in
 // FP32 kernel for apertures of at most 64 x 64 cells, grid sides 64, 96, 128 (fp32_compact.cu)
 int build_compact_lists(const std::vector<short2> &cells, int A, int K, int P, const std::vector<int> &chans,
                         std::vector<uint16_t> &tab, std::vector<int2> &idx, std::vector<int4> &chan);
+bool compact_pays(int N, int P, int A, int K, int rows, int cols);
 size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words);
 int prepare_compact(const epic_plan_s *plan, const GroupCfg &g);
 size_t efield_smem_bytes(int N, int P, int rows, int rrows, int A, int K, int nker, bool taps, int words);
@@ -297,7 +299,7 @@ struct RawImage {
 };
 int fp32_pick_tau(int n_items, int T, int sms);
 int compact_pick_tau(int n_chan, int n_items, int T, int sms);
-int series_chunks(int n_chan, int n_img, int spi, int tau_cap, int sms);   // compact kernel: time chunks per image
+int series_chunks(int items, int n_img, int spi, int tau_cap, int sms);   // compact groups: time chunks per image
 // time chunks of one launch: forced (image series), else autotuned for this T, else the cost model
 int choose_tau(const epic_plan_s *plan, const GroupCfg &g, int T);
 // large grid sides (GroupCfg::alias)

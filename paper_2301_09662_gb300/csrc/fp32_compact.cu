@@ -38,6 +38,7 @@
 // gains, taps and gather lists (read through L1 where they do not fit).
 // Side 64 takes two samples at a time, so that its transforms fill the 8 warps.
 #include <algorithm>
+#include <cmath>
 #include <type_traits>
 
 #include "epic_internal.cuh"
@@ -640,6 +641,21 @@ int build_compact_lists(const std::vector<short2> &cells, int A, int K, int P, c
     }
     if (tab.empty()) tab.push_back(0);
     return EPIC_OK;
+}
+
+// Whether images of a side are faster here than in the per-class kernel.  At side 64 there is one
+// class, so nothing is gridded twice there: its gather uses all warps between the transforms, this
+// kernel's four warps run beside them, but with a single polarisation only half of the transform warps
+// have work.  What decides is the gather, as footprint cells a row (batches get longer, not more, where
+// footprints overlap).  One GB300, us per class / compact, 300 spectra of 32 channels: one polarisation,
+// footprints over 56 x 56 cells, 64 antennas 5 x 5 (29 cells a row) 129 / 153, 64 of 7 x 7 (56) 143 / 150;
+// over 15 x 15, 64 of 3 x 3 (38) 129 / 145, 32 of 5 x 5 (50) 141 / 144, 64 of 5 x 5 (100) 162 / 146; two
+// polarisations over 14 x 14, 16 antennas 1 x 1 (1) 166 / 172, 32 of 3 x 3 (19) 187 / 177; over 56 x 56,
+// 16 of 1 x 1 (0.3) 166 / 183.
+bool compact_pays(int N, int P, int A, int K, int rows, int cols)
+{
+    const double per_row = static_cast<double>(A) * K * K / std::sqrt(static_cast<double>(rows) * cols);
+    return N != 64 || per_row > (P == 2 ? 5.0 : 60.0);
 }
 
 size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words)

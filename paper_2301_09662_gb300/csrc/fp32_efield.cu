@@ -443,7 +443,7 @@ int prepare_efield(const epic_plan_s *plan, const GroupCfg &g)
 int launch_compact_efield(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T,
                           float2 *out, long long stride, cudaStream_t stream)
 {
-    const int n_tau = choose_tau(plan, g, T);
+    const int n_tau = g.cimage ? choose_tau(plan, g, T) : compact_pick_tau(g.n_chan, g.n_items, T, plan->sm_count);
     return efield_dispatch(g, plan->P, [&](auto q_, auto p_, auto pr_) {
         constexpr int Q = decltype(q_)::value, P = decltype(p_)::value, PAIRS = decltype(pr_)::value;
         return plan->nker > 1 ? launch_efield_t<Q, P, PAIRS, true>(plan, g, v, gains, T, n_tau, out, stride, stream)

@@ -350,20 +350,21 @@ int compact_pick_tau(int n_chan, int n_items, int T, int sms)
 }
 
 // A series' image has one time chunk per channel and class in the per-class kernels.  In the compact
-// kernel that is a quarter of the CTAs, so where a batch of n_img images leaves SMs idle each image is
-// split further, within the tau_cap partial images there are.  32 channels of 128 x 128, 256 antennas,
-// one image of 1000 spectra: 3.59 ms per class, 7.40 compact with one chunk, 1.77 split; 12
-// channels, 64 antennas, three images of 100: 304, 737, 246 us.
-int series_chunks(int n_chan, int n_img, int spi, int tau_cap, int sms)
+// kernel that is a quarter of the CTAs (items: its channels), so where a batch of n_img images leaves
+// SMs idle each image is split further, within the tau_cap partial images there are.  32 channels of
+// 128 x 128, 256 antennas, one image of 1000 spectra: 3.59 ms per class, 7.40 compact with one chunk,
+// 1.77 split; 12 channels, 64 antennas, three images of 100: 304, 737, 246 us; the same at side 64, one
+// polarisation (per class with a CTA a channel): 170 -> 66 us.
+int series_chunks(int items, int n_img, int spi, int tau_cap, int sms)
 {
-    return pick_tau(n_chan * n_img, spi, sms, 1, 4.0, std::max(1, tau_cap / n_img));
+    return pick_tau(items * n_img, spi, sms, 1, 4.0, std::max(1, tau_cap / n_img));
 }
 
 int choose_tau(const epic_plan_s *plan, const GroupCfg &g, int T)
 {
     int n = plan->force_tau > 0                       ? plan->force_tau
             : (g.tuned_tau > 0 && g.tuned_T == T) ? g.tuned_tau
-            : g.compact                             ? compact_pick_tau(g.n_chan, g.n_items, T, plan->sm_count)
+            : g.cimage                              ? compact_pick_tau(g.n_chan, g.n_items, T, plan->sm_count)
                                                   : fp32_pick_tau(g.launch_items, T, plan->sm_count);
     return std::max(1, std::min(n, g.tau_cap));
 }
@@ -416,7 +417,7 @@ int launch_imaging(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const
     if (g.alias && plan->force_tau == 0) return launch_alias(plan, g, v, gains, T, n_tau, s);
     if (g.tensor && !g.tc_regular) return EPIC_ERR_UNSUPPORTED;   // e.g. an image series: no fold path there
     if (g.tensor) return g.pair ? launch_tc_pair(plan, g, v, gains, T, n_tau, s) : launch_tc_dual(plan, g, v, gains, T, n_tau, s);
-    if (g.compact) return launch_compact(plan, g, v, gains, T, n_tau, s);
+    if (g.cimage) return launch_compact(plan, g, v, gains, T, n_tau, s);
     if (g.reg64) return launch_reg64(plan, g, v, gains, T, n_tau, s);
     switch (g.M * 4 + plan->P) {
     case 32 * 4 + 2: return launch_group<32, 2>(plan, g, v, gains, T, n_tau, s);

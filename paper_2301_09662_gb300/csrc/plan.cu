@@ -852,6 +852,10 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 g.etaps = p->nker > 1 && ef_fits(true, 0);
                 g.estage = ef_fits(g.etaps, g.cwords) && !(diag & EPIC_DIAG_GATHER_GLOBAL);
             }
+            // images per class where that is faster (and possible)
+            int ccols = 0;
+            for (size_t i = 0; i < lchan.size(); i += 2) ccols = std::max(ccols, lchan[i].w);
+            g.cimage = g.compact && (!g.reg64 || epic::compact_pays(g.N, n_pol, n_ant, p->K, g.crows, ccols));
             if (g.compact) {
                 g.R1 = 1;
                 g.R2 = g.M;
@@ -860,7 +864,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 if (rc == EPIC_OK) rc = dev_upload(&g.d_lchan, lchan.data(), lchan.size());
             }
         }
-        if (g.reg64 && !g.compact) {
+        if (g.reg64 && !g.cimage) {
             g.R1 = 1;
             g.R2 = g.M;
             std::vector<uint32_t> desc;
@@ -1005,9 +1009,9 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 }
             }
         }
-        g.launch_items = g.pair ? g.n_chan * (g.Q1 == 2 ? 2 : 1) : g.compact ? g.n_chan : g.n_items;
+        g.launch_items = g.pair ? g.n_chan * (g.Q1 == 2 ? 2 : 1) : g.cimage ? g.n_chan : g.n_items;
         if (g.pair) g.tau_cap = std::max(g.tau_cap, epic::fp32_pick_tau(g.launch_items, max_spectra, p->sm_count));
-        if (g.compact) g.tau_cap = std::max(g.tau_cap, epic::compact_pick_tau(g.n_chan, g.n_items, max_spectra, p->sm_count));
+        if (g.cimage) g.tau_cap = std::max(g.tau_cap, epic::compact_pick_tau(g.n_chan, g.n_items, max_spectra, p->sm_count));
         if (rc == EPIC_OK) rc = dev_upload(&g.d_chans, g.chans.data(), g.chans.size());
         if (rc == EPIC_OK) rc = dev_upload(&g.d_out_off, offs.data(), offs.size());
         if (rc == EPIC_OK) {
@@ -1078,7 +1082,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
     for (const auto &g : p->groups) {
         if (rc != EPIC_OK) break;
         if (!g.tensor) rc = epic::prepare_fp32(p, g);
-        if (rc == EPIC_OK && g.compact) rc = epic::prepare_compact(p, g);
+        if (rc == EPIC_OK && g.cimage) rc = epic::prepare_compact(p, g);
         if (rc == EPIC_OK && g.compact) rc = epic::prepare_efield(p, g);
         if (rc == EPIC_OK && g.wide) rc = epic::prepare_wide(p, g);
         if (rc == EPIC_OK && g.alias) rc = epic::prepare_alias(p);
@@ -1202,7 +1206,7 @@ int epic_autotune(epic_plan_t plan, int n_spectra, void *stream)
         auto add = [&](int n) {
             if (n >= 1 && n <= cap && std::find(cand.begin(), cand.end(), n) == cand.end()) cand.push_back(n);
         };
-        const int c0 = g.compact ? epic::compact_pick_tau(g.n_chan, g.n_items, n_spectra, plan->sm_count)
+        const int c0 = g.cimage ? epic::compact_pick_tau(g.n_chan, g.n_items, n_spectra, plan->sm_count)
                                  : epic::fp32_pick_tau(g.launch_items, n_spectra, plan->sm_count);
         for (int d = -2; d <= 2; d++) add(c0 + d);
         for (int waves = 1; waves <= 4; waves++)
@@ -1296,7 +1300,7 @@ int epic_image_series_ex(epic_plan_t plan, const uint8_t *ci4, const float *gain
         for (const auto &g : plan->groups) {
             if (rc != EPIC_OK) break;
             int n_tau = 0;
-            const int per = g.compact ? epic::series_chunks(g.n_chan, b, spi, g.tau_cap, plan->sm_count) : 1;
+            const int per = g.compact ? epic::series_chunks(g.cimage ? g.n_chan : g.n_items, b, spi, g.tau_cap, plan->sm_count) : 1;
             plan->force_tau = b * per;   // chunks of one image each, per of them to an image
             rc = epic::launch_imaging(plan, g, vb, g2, spi * b, &n_tau, s);
             if (rc == EPIC_OK) rc = epic::launch_epilogue_series(plan, g, g2, spi, b, per, ob, s);

@@ -38,8 +38,24 @@ static void series()
                     }
 }
 
+// Side 64: images per class where the gather is small (the measured pairs beside the rule).
+static void side64()
+{
+    const struct {
+        int P, A, K, span;
+        bool compact;
+    } at[] = {{1, 64, 5, 56, false}, {1, 64, 7, 56, false}, {1, 64, 3, 15, false}, {1, 32, 5, 15, false}, {1, 64, 5, 16, true},
+              {1, 256, 3, 15, true},  {2, 16, 1, 14, false}, {2, 16, 1, 56, false}, {2, 32, 3, 15, true},  {2, 256, 5, 40, true}};
+    for (const auto &c : at) {
+        CHECK(epic::compact_pays(64, c.P, c.A, c.K, c.span, c.span) == c.compact, "side 64, P %d, %d antennas, K %d, %d cells", c.P,
+              c.A, c.K, c.span);
+        for (int N : {96, 128}) CHECK(epic::compact_pays(N, c.P, c.A, c.K, c.span, c.span), "side %d", N);
+    }
+}
+
 int main()
 {
+    side64();
     series();
     if (g_bad) std::printf("%ld checks failed\n", g_bad);
     return g_bad ? 1 : 0;

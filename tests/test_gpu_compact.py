@@ -35,6 +35,9 @@ def _span(wl, span, K):
     (64, 2, 24, 7, 3, 40),      # two samples at a time, the last one absent
     (64, 1, 23, 8, 1, 33),
     (64, 2, 40, 3, 5, 60),      # planes of two samples do not fit: the per-class kernel
+    (64, 1, 104, 9, 5, 40),     # 65 footprint cells a row: compact with a single polarisation
+    (64, 1, 92, 9, 5, 40),      # 57.5: the per-class kernel
+    (64, 2, 16, 5, 1, 20),      # few footprint cells: the per-class kernel
 ])
 def test_edges(N, P, A, T, K, span):
     wl = _span(synth.random_small(A=A, P=P, C=3, T=T, N=N, K=K, seed=A + N + T, full_range=True), span, K)
