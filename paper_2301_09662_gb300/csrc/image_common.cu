@@ -437,12 +437,6 @@ int epi_dispatch(int N, int M, int P, F &&f)
     return EPIC_ERR_UNSUPPORTED;
 }
 
-// Pixel tiles: four pixels a thread, one where that would leave SMs idle.
-int epi_tiles(int N, int images, int sms)
-{
-    const int one = (N * N + kThreads - 1) / kThreads, four = (one + 3) / 4;
-    return four * images >= 4 * sms ? four : one;
-}
 
 // A_pq summed by the epilogue's own blocks (small arrays: the sums are shorter than a launch) or by
 // auto_sum_kernel.  16 antennas, 4 channels of 32 x 32, 64 spectra, whole
@@ -500,6 +494,16 @@ __global__ void delay_prep_kernel(const double *__restrict__ delays, int n, doub
 
 }  // namespace
 
+// Pixel tiles: four pixels a thread, one where that would leave SMs without a block.  One GB300, whole
+// calls of 16 spectra, us with four / one: two polarisations, 16 antennas, 128 x 128, 4 channels (64 /
+// 256 blocks) 32 / 29, 16 channels (256 / 1024) 39 / 49, 32 channels 57 / 82; one polarisation, 100
+// antennas, 64 x 64, 32 channels (128 / 512) 27 / 24, 64 channels 33 / 33; two of 512 x 512 (512 / 2048) 41 / 49.
+int epi_tiles(int N, int images, int sms)
+{
+    const int one = (N * N + kThreads - 1) / kThreads, four = (one + 3) / 4;
+    return four * images >= sms ? four : one;
+}
+
 int launch_autopower_raw(const RawImage &r, const uint8_t *v, int sm_count, cudaStream_t stream)
 {
     if (r.T == 0) return EPIC_OK;
@@ -507,11 +511,11 @@ int launch_autopower_raw(const RawImage &r, const uint8_t *v, int sm_count, cuda
     return launch_auto(v, r.T, r.C, r.A, r.P, chunks, 0, r.autoint, stream);
 }
 
-int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, cudaStream_t stream)
+int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, int sm_count, cudaStream_t stream)
 {
     return epi_dispatch(r.N, r.M, r.P, [&](auto n_, auto m_, auto p_) {
         constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
-        const dim3 grid(static_cast<unsigned>(epi_tiles(N, r.C, 148)), static_cast<unsigned>(r.C));
+        const dim3 grid(static_cast<unsigned>(epi_tiles(N, r.C, sm_count)), static_cast<unsigned>(r.C));
         epilogue_kernel<N, M, P, false><<<grid, kThreads, 0, stream>>>(r.partial, r.n_tau, r.n_items, 8, M / 8, r.chans, r.out_off,
                                                                 r.wpow, nullptr, r.autoint, 1, 0, gains, r.A, r.C, r.T, r.flags,
                                                                 out, 0, nullptr, nullptr, 0);

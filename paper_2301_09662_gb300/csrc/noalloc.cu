@@ -180,5 +180,5 @@ extern "C" int epic_image_static(const double *ant_xy_m, int n_ant, int n_pol, c
     }
     rc = launch_fp32_raw(r, ci4, gains, stream);
     if (rc != EPIC_OK) return rc;
-    return launch_epilogue_raw(r, gains, reinterpret_cast<float2 *>(out_c64), stream);
+    return launch_epilogue_raw(r, gains, reinterpret_cast<float2 *>(out_c64), sms, stream);
 }

@@ -53,8 +53,20 @@ static void side64()
     }
 }
 
+// Epilogue: one pixel a thread only where four would leave SMs without a block (measured pairs).
+static void tiles()
+{
+    const struct {
+        int N, images, want;
+    } at[] = {{32, 4, 4}, {128, 4, 64}, {128, 16, 16}, {128, 32, 16}, {64, 32, 16}, {64, 64, 4}, {64, 150, 4}, {512, 1, 256}, {128, 8, 64}};
+    for (const auto &c : at)
+        CHECK(epic::epi_tiles(c.N, c.images, 152) == c.want, "side %d, %d images: %d tiles", c.N, c.images,
+              epic::epi_tiles(c.N, c.images, 152));
+}
+
 int main()
 {
+    tiles();
     side64();
     series();
     if (g_bad) std::printf("%ld checks failed\n", g_bad);
