@@ -188,7 +188,10 @@ __device__ __forceinline__ void pair_msub(float2 &s, float2 a, float2 b)
 // runs in FP32 pairs (~48 bits): GB300's FP64 pipe does ~2 operations a clock
 // and SM, and five FP64 operations and eight conversions a value made it, not
 // the memory, the limit; A_pq itself is summed in FP64, once per channel and
-// image (auto_sum_kernel), not in every block.  Whole calls: 25 Stokes images of
+// image (auto_sum_kernel), not in every block (apq_tab null: the plan-free entry point's blocks sum
+// autoint themselves).  Also for small arrays, whose sums are shorter than a launch: 16 antennas, 32 x 32,
+// 4 channels of 64 spectra 18.4 us with the blocks' own sums, 16.4 so; 64 channels of 128 x 128, 16 spectra
+// 88 and 78.  Whole calls: 25 Stokes images of
 // 64 channels of 128 x 128 5.21 -> 3.66 ms, 64 channels of 512 x 512 with 2048
 // antennas 21.75 -> 20.40 ms.
 // AK: an auto image from the per-antenna auto-correlation grids (Yauto) instead of A_pq |W^|^2
@@ -438,14 +441,9 @@ int epi_dispatch(int N, int M, int P, F &&f)
 }
 
 
-// A_pq summed by the epilogue's own blocks (small arrays: the sums are shorter than a launch) or by
-// auto_sum_kernel.  16 antennas, 4 channels of 32 x 32, 64 spectra, whole
-// call: 26.4 us with the extra kernel, 18.6 us without it and with one pixel a thread.
-bool auto_in_epilogue(const epic_plan_s *plan) { return plan->A <= 64; }
-
-// n_img images of n_tau time chunks each, their auto sums in auto_n chunks each
-int launch_epi(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T, int n_tau, int n_img, int auto_n,
-               float2 *out, cudaStream_t stream)
+// n_img images of n_tau time chunks each
+int launch_epi(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T, int n_tau, int n_img, float2 *out,
+               cudaStream_t stream)
 {
     return epi_dispatch(g.N, g.M, plan->P, [&](auto n_, auto m_, auto p_) {
         constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
@@ -454,8 +452,7 @@ int launch_epi(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T,
         const auto kfn = plan->nker > 1 ? epilogue_kernel<N, M, P, true> : epilogue_kernel<N, M, P, false>;
         kfn<<<grid, kThreads, 0, stream>>>(
             g.d_partial, n_tau, g.n_items, g.R1, g.R2, g.d_chans, g.d_out_off, g.d_wpow,
-            auto_in_epilogue(plan) ? nullptr : plan->d_apq, plan->d_autoint, auto_n, static_cast<size_t>(plan->C) * plan->A * 4,
-            gains, plan->A, plan->C, T, plan->flags, out, static_cast<long long>(plan->out_floats / 2),
+            plan->d_apq, nullptr, 0, 0, gains, plan->A, plan->C, T, plan->flags, out, static_cast<long long>(plan->out_floats / 2),
             g.d_Y, g.d_twp, plan->K);
         return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
     });
@@ -527,13 +524,12 @@ int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, int
 // each, few enough that summing them (auto_sum_kernel, one block a channel) stays short.
 int auto_chunks(const epic_plan_s *plan, int T)
 {
-    return std::max(1, std::min({(8 * plan->sm_count + plan->C - 1) / plan->C, T / 4, plan->A <= 64 ? 8 : 32}));
+    return std::max(1, std::min({(8 * plan->sm_count + plan->C - 1) / plan->C, T / 4, 32}));
 }
 
 // A_pq of n_img images from the auto sums of chunks chunks each
 static int launch_auto_sum(epic_plan_s *plan, const float2 *gains, int chunks, int n_img, cudaStream_t stream)
 {
-    if (auto_in_epilogue(plan)) return EPIC_OK;
     const dim3 grid(static_cast<unsigned>(plan->C), static_cast<unsigned>(n_img));
     const size_t stride = static_cast<size_t>(plan->C) * plan->A * 4;
     if (plan->P == 2) auto_sum_kernel<2><<<grid, kThreads, 0, stream>>>(plan->d_autoint, chunks, stride, gains, plan->A, plan->C, plan->d_apq);
@@ -551,7 +547,7 @@ int launch_autopower_series(epic_plan_s *plan, const uint8_t *v, const float2 *g
 int launch_epilogue_series(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int spi, int n_img, int n_tau,
                            float2 *out, cudaStream_t stream)
 {
-    return launch_epi(plan, g, gains, spi, n_tau, n_img, 1, out, stream);
+    return launch_epi(plan, g, gains, spi, n_tau, n_img, out, stream);
 }
 
 int launch_delay_prep(epic_plan_s *plan, int T, cudaStream_t stream)
@@ -587,7 +583,7 @@ int launch_autopower(epic_plan_s *plan, const uint8_t *v, const float2 *gains, i
 int launch_epilogue(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T, int n_tau, float2 *out,
                     cudaStream_t stream)
 {
-    return launch_epi(plan, g, gains, T, n_tau, 1, auto_chunks(plan, T), out, stream);
+    return launch_epi(plan, g, gains, T, n_tau, 1, out, stream);
 }
 
 }  // namespace epic

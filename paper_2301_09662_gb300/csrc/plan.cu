@@ -1053,7 +1053,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
     if (rc == EPIC_OK)
         rc = dev_upload(&p->d_autoint, static_cast<const int *>(nullptr),
                         static_cast<size_t>(std::max(p->series_cap, epic::auto_chunks(p, max_spectra))) * n_chan * n_ant * 4);
-    if (rc == EPIC_OK && !ant_kernels)
+    if (rc == EPIC_OK && p->nker == 1)
         rc = dev_upload(&p->d_apq, static_cast<const double *>(nullptr), static_cast<size_t>(p->series_cap) * n_chan * 4);
     if (rc == EPIC_OK && tensor) {
         // both 64-point DFT stages on the tensor cores (tc_dual64.cu)

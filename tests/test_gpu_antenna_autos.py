@@ -30,3 +30,16 @@ def test_auto_image_edges(A, P, N, K):
     got, p = run_gpu(wl, flags=epic.EPIC_ANTENNA_KERNELS)
     p.close()
     assert peak_rel_err(got, oracle.workload_image(wl), wl.grid_n, P).max() < 1e-5
+
+
+def test_one_antenna():
+    """Its kernel is the plan's one kernel, and its image its auto image: nothing is left of it."""
+    wl = copy.copy(synth.random_small(A=1, P=2, C=2, T=3, N=64, K=3, seed=1, full_range=True))
+    wl.kernel = synth.antenna_kernels(1, 3, np.random.default_rng(3))
+    got, p = run_gpu(wl, flags=epic.EPIC_ANTENNA_KERNELS)
+    p.close()
+    whole, p = run_gpu(wl, flags=epic.EPIC_ANTENNA_KERNELS | epic.EPIC_NO_AUTOSUB)
+    p.close()
+    ref = oracle.workload_image(wl, flags=epic.EPIC_NO_AUTOSUB)
+    assert peak_rel_err(whole, ref, wl.grid_n, 2).max() < 1e-5
+    assert np.abs(got).max() < 1e-5 * np.abs(ref).max()
