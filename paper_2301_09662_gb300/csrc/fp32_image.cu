@@ -430,11 +430,25 @@ int launch_imaging(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const
     }
 }
 
+// Whether the auto sums of a plan with one group of side 32 run beside its imaging.  That kernel's CTAs
+// share SMs, so where they come to one wave of long chunks (n_tau chunks of T spectra) blocks of the auto
+// sums placed among them can leave two on an SM and none on another for the whole call, and which are
+// placed first varies in a row of calls.  Two polarisations, ms one after the other / beside each other:
+// 256 antennas, 152 channels x 500 spectra (chunks of 500) 4.12 / 4.11 .. 5.00; 16 antennas, 8 channels x
+// 1000 (of 53) 0.271 / 0.263 .. 0.306, 16 channels x 200 (of 23) 0.127 / 0.121; 4 channels x 64, one
+// polarisation (of 2) 0.0205 / 0.0164.
+bool fork_pays(int n_items, int n_tau, int T, int sms)
+{
+    return static_cast<long long>(n_items) * n_tau > sms || (T + n_tau - 1) / n_tau < 48;
+}
+
 // Launch every kernel of one integration.  With fork, the auto-power kernel
 // runs on `stream` while each grid side's imaging kernel runs on its own side
 // stream; each epilogue waits for its imaging kernel and for the auto-power,
 // and `stream` joins all branches at the end (the shape captured into the
-// plan's CUDA graph).
+// plan's CUDA graph).  A group of side 32 alone starts its imaging first, so
+// that its CTAs spread over empty SMs (256 antennas, 16 channels x 200 spectra, waited for:
+// 257 us after the auto sums' blocks, 215 before them, 225 without the fork).
 int image_fp32(epic_plan_s *plan, const uint8_t *v, const float2 *gains, int T, float2 *out, cudaStream_t stream,
                bool fork)
 {
@@ -443,33 +457,38 @@ int image_fp32(epic_plan_s *plan, const uint8_t *v, const float2 *gains, int T, 
                                                                                                 : EPIC_ERR_CUDA;
     }
     const bool autosub = !(plan->flags & EPIC_NO_AUTOSUB);
-    fork = fork && !plan->side.empty();
+    const bool side32 = plan->groups.size() == 1 && plan->groups[0].M == 32;
+    fork = fork && !plan->side.empty() &&
+           !(side32 && !fork_pays(plan->groups[0].n_items, choose_tau(plan, plan->groups[0], T), T, plan->sm_count));
     int rc = EPIC_OK;
-    int stage = 0;
+    const int lead = autosub ? 1 : 0;    // stages: the auto sums, then imaging and epilogue of each group
     prof_begin(plan);
     if (plan->delays && (rc = launch_delay_prep(plan, T, stream)) != EPIC_OK) return rc;
     if (fork && cudaEventRecord(plan->ev_fork, stream) != cudaSuccess) return EPIC_ERR_CUDA;
-    if (autosub) {
-        prof_mark(plan, stream, stage, true);
-        rc = launch_autopower(plan, v, gains, T, stream);
-        prof_mark(plan, stream, stage++, false);
-        if (rc != EPIC_OK) return rc;
-        if (fork && cudaEventRecord(plan->ev_auto, stream) != cudaSuccess) return EPIC_ERR_CUDA;
-    }
+    auto autos = [&]() -> int {
+        prof_mark(plan, stream, 0, true);
+        const int r = launch_autopower(plan, v, gains, T, stream);
+        prof_mark(plan, stream, 0, false);
+        if (r != EPIC_OK) return r;
+        return fork && cudaEventRecord(plan->ev_auto, stream) != cudaSuccess ? EPIC_ERR_CUDA : EPIC_OK;
+    };
+    if (autosub && !side32 && (rc = autos()) != EPIC_OK) return rc;
     for (size_t gi = 0; gi < plan->groups.size(); gi++) {
         const GroupCfg &g = plan->groups[gi];
+        const int stage = lead + 2 * static_cast<int>(gi);
         cudaStream_t s = fork ? plan->side[gi] : stream;
         if (fork && cudaStreamWaitEvent(s, plan->ev_fork, 0) != cudaSuccess) return EPIC_ERR_CUDA;
         int n_tau = 1;
         prof_mark(plan, s, stage, true);
         rc = launch_imaging(plan, g, v, gains, T, &n_tau, s);
-        prof_mark(plan, s, stage++, false);
+        prof_mark(plan, s, stage, false);
         if (rc != EPIC_OK) return rc;
+        if (autosub && side32 && (rc = autos()) != EPIC_OK) return rc;
         if (fork && autosub && cudaStreamWaitEvent(s, plan->ev_auto, 0) != cudaSuccess) return EPIC_ERR_CUDA;
-        prof_mark(plan, s, stage, true);
+        prof_mark(plan, s, stage + 1, true);
         if (autosub && plan->nker > 1) rc = launch_auto_rho(plan, g, gains, s);
         if (rc == EPIC_OK) rc = launch_epilogue(plan, g, gains, T, n_tau, out, s);
-        prof_mark(plan, s, stage++, false);
+        prof_mark(plan, s, stage + 1, false);
         if (rc != EPIC_OK) return rc;
         if (fork) {
             if (cudaEventRecord(plan->ev_join[gi], s) != cudaSuccess) return EPIC_ERR_CUDA;

@@ -64,8 +64,17 @@ static void tiles()
               epic::epi_tiles(c.N, c.images, 152));
 }
 
+// Side 32 alone: no fork beside one wave of long chunks (measured pairs).
+static void fork32()
+{
+    CHECK(!epic::fork_pays(152, 1, 500, 152) && !epic::fork_pays(8, 19, 1000, 152), "one wave of long chunks");
+    CHECK(epic::fork_pays(4, 32, 64, 152) && epic::fork_pays(64, 7, 200, 152) && epic::fork_pays(16, 9, 200, 152),
+          "short chunks, several waves");
+}
+
 int main()
 {
+    fork32();
     tiles();
     side64();
     series();
