@@ -74,6 +74,7 @@ struct GroupCfg {
     bool gstage = false;               // blocks staged in shared memory
     // FP32 plans whose aperture occupies at most 64 x 64 cells: the compact kernel (fp32_compact.cu)
     bool compact = false;
+    bool eclass = false;               // has the per-class tables too, for small E-field calls (efield_per_class)
     bool cimage = false;               // its images too (compact_pays), else only its E-field images
     bool cstage = false;               // its gather lists are staged in shared memory
     bool ctaps = false;                // and, with a kernel per antenna, the kernels
@@ -255,6 +256,7 @@ size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool t
 int prepare_compact(const epic_plan_s *plan, const GroupCfg &g);
 size_t efield_smem_bytes(int N, int P, int rows, int rrows, int A, int K, int nker, bool taps, int words);
 int efield_rows(int N, const std::vector<int4> &lchan);   // most rows of R where every channel is placed on a quarter
+bool efield_per_class(int N, int P, int n_items, int T, int sms);   // an E-field call so small that the per-class kernel is faster
 int prepare_efield(const epic_plan_s *plan, const GroupCfg &g);
 int launch_compact(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
                    cudaStream_t stream);

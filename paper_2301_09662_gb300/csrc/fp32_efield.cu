@@ -430,6 +430,19 @@ int efield_rows(int N, const std::vector<int4> &lchan)
     return most;
 }
 
+// A CTA here transforms all classes of a sample one after the other
+// where the per-class kernel has a CTA for each.  Where those find room on the SMs at
+// once (a CTA takes one sample, or two of one polarisation) the call is its latency.  One GB300, us per
+// class / here: side 128, two polarisations, 4 channels x 8 spectra (128 CTAs) 12.3 / 18.4, 4 x 12 (192) 15.4
+// / 18.5, 8 x 8 with 1000 antennas (256) 35 / 39, 4 x 20 (320) 22.5 / 18.5, 64 x 2 (512) 28.7 / 20.5; one, 4
+// x 8 (64) 10.3 / 16.4, 16 x 8 (256) 16.4 / 18.5, 64 x 2 (256 in one sample's classes) 20.7 / 18.5; side
+// 96, two, 4 x 12 14.4 / 15.4, 4 x 20 19.5 / 16.0.  At side 64 this kernel is not the slower one.
+bool efield_per_class(int N, int P, int n_items, int T, int sms)
+{
+    const long long ctas = static_cast<long long>(n_items) * (P == 1 ? (T + 1) / 2 : T);
+    return (N == 96 || N == 128) && n_items <= sms && 4 * ctas <= 7LL * sms;
+}
+
 int prepare_efield(const epic_plan_s *plan, const GroupCfg &g)
 {
     const size_t need = efield_smem_bytes(g.N, plan->P, g.crows, g.erows, plan->A, plan->K, plan->nker, g.etaps, g.estage ? g.cwords : 0);

@@ -470,7 +470,7 @@ int launch_reg64_t(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const
     auto kfn = fp32_reg64_kernel<M, P, TS, DL, GS, EF>;
     const size_t smem = reg64_smem<M, P, TS>(plan->A, plan->K, plan->nker) +
                         (GS ? sizeof(uint32_t) * static_cast<size_t>(g.gwords) : 0);
-    int n_tau = choose_tau(plan, g, T);
+    int n_tau = EF && g.cimage ? fp32_pick_tau(g.n_items, T, plan->sm_count) : choose_tau(plan, g, T);
     if (n_tau > g.tau_cap) n_tau = g.tau_cap;
     *n_tau_out = n_tau;
     const dim3 grid(static_cast<unsigned>(g.n_items * n_tau));

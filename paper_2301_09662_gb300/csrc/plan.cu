@@ -855,6 +855,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
             // images per class where that is faster (and possible)
             int ccols = 0;
             for (size_t i = 0; i < lchan.size(); i += 2) ccols = std::max(ccols, lchan[i].w);
+            g.eclass = g.compact && g.reg64 && epic::efield_per_class(g.N, n_pol, g.n_items, 1, p->sm_count);
             g.cimage = g.compact && (!g.reg64 || epic::compact_pays(g.N, n_pol, n_ant, p->K, g.crows, ccols));
             if (g.compact) {
                 g.R1 = 1;
@@ -864,7 +865,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 if (rc == EPIC_OK) rc = dev_upload(&g.d_lchan, lchan.data(), lchan.size());
             }
         }
-        if (g.reg64 && !g.cimage) {
+        if (g.reg64 && (!g.cimage || g.eclass)) {
             g.R1 = 1;
             g.R2 = g.M;
             std::vector<uint32_t> desc;
@@ -1327,8 +1328,9 @@ int epic_image_efield(epic_plan_t plan, const uint8_t *ci4, const float *gains, 
     const auto *g2 = reinterpret_cast<const float2 *>(gains);
     plan->delays = nullptr;
     for (const auto &g : plan->groups) {
-        const int rc = g.compact ? epic::launch_compact_efield(plan, g, ci4, g2, n_spectra, o, plan->ef_stride, s)
-                                 : epic::launch_reg64_efield(plan, g, ci4, g2, n_spectra, o, plan->ef_stride, s);
+        const bool classes = !g.compact || (g.eclass && epic::efield_per_class(g.N, plan->P, g.n_items, n_spectra, plan->sm_count));
+        const int rc = classes ? epic::launch_reg64_efield(plan, g, ci4, g2, n_spectra, o, plan->ef_stride, s)
+                               : epic::launch_compact_efield(plan, g, ci4, g2, n_spectra, o, plan->ef_stride, s);
         if (rc != EPIC_OK) return rc;
     }
     return EPIC_OK;

@@ -72,8 +72,23 @@ static void fork32()
           "short chunks, several waves");
 }
 
+// E-field calls: per class while its CTAs fit on the SMs at once (measured pairs).
+static void efield()
+{
+    const struct {
+        int N, P, items, T;
+        bool classes;
+    } at[] = {{128, 2, 16, 8, true}, {128, 2, 16, 12, true}, {128, 2, 32, 8, true}, {128, 2, 16, 20, false}, {128, 2, 256, 1, false},
+              {128, 1, 16, 8, true}, {128, 1, 64, 8, true},  {128, 1, 256, 2, false}, {96, 2, 16, 12, true}, {96, 2, 16, 20, false},
+              {64, 2, 4, 1, false}};
+    for (const auto &c : at)
+        CHECK(epic::efield_per_class(c.N, c.P, c.items, c.T, 152) == c.classes, "side %d, P %d, %d classes x %d spectra", c.N, c.P,
+              c.items, c.T);
+}
+
 int main()
 {
+    efield();
     fork32();
     tiles();
     side64();
