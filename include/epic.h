@@ -164,8 +164,9 @@ enum {
  * A = 256, K = 5), staged in shared memory by the kernel when they fit.
  * FP32 channels with a 256 or 512 grid side, both polarisations, one shared
  * kernel and footprints within 128 x 128 cells add a workspace of transformed
- * rows of up to 4 GiB (N * 16 bytes per occupied row and spectrum, batched);
- * other channels with a 512 grid side and one shared kernel wider than one tap
+ * rows of up to 4 GiB (N * 16 bytes per occupied row and spectrum, batched)
+ * and take up to 2 GiB of partial images (C * N * N * 16 bytes each) where the
+ * other kernels take fewer; other channels with a 512 grid side and one shared kernel wider than one tap
  * add the folded class grids of one time batch, up to 4 GiB (C * 64 * n_pol *
  * 32 KB per spectrum, batched).  FP32 plans without room for either grid per
  * pixel class, more slowly.  Returns

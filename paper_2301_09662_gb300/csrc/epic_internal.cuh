@@ -268,7 +268,15 @@ int build_wide_lists(const std::vector<short2> &cells, int A, int K, const std::
 size_t wide_rows_smem_bytes(int A, int K, bool gains);
 bool wide_pays(const epic_plan_s *plan, const GroupCfg &g, int T);
 int wide_stages(int rpad, size_t smem_optin);
-int wide_pick_tau(const GroupCfg &g, int T, int sms);
+struct WideSplit {
+    int batches, n_sub, rounds;        // time batches, chunks of a batch, sets of partial images
+    double cost;
+};
+struct WideLayout {
+    int cb, tb, slots;                 // channels and spectra of a batch, partial images
+};
+WideSplit wide_split(int N, int n_items, int cb, int tb, int slots, int T, int sms);
+WideLayout wide_layout(int N, int n_chan, int rpad, int max_spectra, int cap_tb, int tau_class, int sms);
 int prepare_wide(const epic_plan_s *plan, const GroupCfg &g);
 int launch_wide(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
                 cudaStream_t stream);

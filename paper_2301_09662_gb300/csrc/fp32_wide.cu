@@ -603,13 +603,62 @@ int wide_stages(int rpad, size_t smem_optin)
     return s >= 2 ? s : 0;
 }
 
-// Time chunks of one integration: enough column blocks for whole waves of SMs; at side 256 no fewer
-// than the per-class kernel would take, so FP32 sums run over no more samples than there.
-int wide_pick_tau(const GroupCfg &g, int T, int sms)
+// How an integration of T spectra in groups of cb channels runs: batches of at most tb spectra, each in
+// n_sub chunks side by side, batch b adding to the partial images of round b mod rounds (n_sub rounds
+// slots in all, every one of them written).  The fewest samples on the busiest SM, a chunk costing two
+// more, one that continues earlier sums three, and a batch's launches four.  At side 256 no slot sums more spectra than a chunk of
+// the per-class kernel (at side 512 the fold path adds all of them into one).
+WideSplit wide_split(int N, int n_items, int cb, int tb, int slots, int T, int sms)
 {
-    const int Q = g.N / 64, n = fp32_pick_tau(std::min(g.wcb, g.n_chan) * 2 * Q, T, sms);
-    return g.N == 512 ? n : std::max(n, fp32_pick_tau(g.n_items, T, sms));
+    const int blocks = cb * 2 * (N / 64), need = std::max(1, (T + tb - 1) / tb);
+    const int n_min = N == 512 ? 1 : std::max(1, std::min(slots, fp32_pick_tau(n_items, T, sms)));
+    WideSplit best{need, 1, 1, 1e300};
+    for (int n = 1; n <= slots; n++) {
+        const int rounds = need == 1 ? 1 : (n_min + n - 1) / n;
+        if (rounds * n < n_min || rounds * n > slots) continue;
+        WideSplit s{rounds * ((need + rounds - 1) / rounds), n, rounds, 0};
+        const int nb = (T + s.batches - 1) / s.batches;
+        if (n > 1 && n > nb) break;
+        const long long waves = (static_cast<long long>(blocks) * n + sms - 1) / sms;
+        s.cost = s.batches * (waves * ((nb + n - 1) / n + (s.batches > rounds ? 3.0 : 2.0)) + 4.0);
+        if (s.cost < best.cost - 1e-9) best = s;
+    }
+    return best;
 }
+
+// Channels and spectra of a batch and the partial images of a plan: the workspace holds cb x tb channel
+// samples within 4 GiB, the partial images stay within 2 GiB (or the tau_class of the per-class kernel).
+// Few channels at a time leave SMs idle, many make short batches, so the cheapest split over the whole
+// call decides.  16 channels, 300 antennas, side 512, 5000 spectra: in batches of 2500 of one channel with
+// one chunk each 488 ms, in 19 chunks 72.9 (fold path 143); side 256, 9000 spectra 412, 46.0 (per class 58).
+WideLayout wide_layout(int N, int n_chan, int rpad, int max_spectra, int cap_tb, int tau_class, int sms)
+{
+    constexpr size_t kWork = size_t(4) << 30, kSums = size_t(2) << 30;
+    const size_t per = static_cast<size_t>(N) * 2 * rpad * sizeof(float2);
+    const size_t slot = static_cast<size_t>(n_chan) * N * N * sizeof(float4);
+    const int room = static_cast<int>(std::max<size_t>(1, kWork / per));   // channel samples
+    const int n_items = n_chan * (N / 64) * (N / 64);
+    const int slots = std::max(tau_class, static_cast<int>(std::max<size_t>(1, std::min<size_t>(kMaxTau, kSums / slot))));
+    WideLayout best{1, 1, tau_class};
+    double best_cost = 1e300;
+    int last = 0;
+    for (int groups = 1; groups <= n_chan; groups++) {
+        const int cb = (n_chan + groups - 1) / groups;
+        if (cb == last || cb > room) continue;
+        last = cb;
+        int tb = std::min(max_spectra, room / cb);
+        if (cap_tb > 0) tb = std::min(tb, cap_tb);
+        const WideSplit s = wide_split(N, n_items, cb, tb, slots, max_spectra, sms);
+        double cost = s.cost * (n_chan / cb);
+        if (n_chan % cb) cost += wide_split(N, n_items, n_chan % cb, tb, slots, max_spectra, sms).cost;
+        if (cost < best_cost - 1e-9) {
+            best_cost = cost;
+            best = WideLayout{cb, tb, std::max(tau_class, s.n_sub * s.rounds)};
+        }
+    }
+    return best;
+}
+
 // Whether an integration of T spectra is worth the two launches: for the smallest the per-class
 // kernel's single launch is shorter.  Its time goes as the classes times transform and gridding, a
 // footprint cell weighing three times the arithmetic's share (lists and shared-memory reads).  One
@@ -622,8 +671,6 @@ bool wide_pays(const epic_plan_s *plan, const GroupCfg &g, int T)
     const double work = static_cast<double>(g.n_items) * T * (3.0 * plan->A * plan->K * plan->K + 16384.0);
     return g.wforce || work >= (g.N == 512 ? 5.5e7 : 3e7);
 }
-static int wide_tau(const GroupCfg &g, int T, int sms) { return std::max(1, std::min(wide_pick_tau(g, T, sms), g.tau_cap)); }
-
 int prepare_wide(const epic_plan_s *plan, const GroupCfg &g)
 {
     const size_t rows = wide_rows_smem(plan->A, plan->K, g.wgains), cols = wide_cols_smem(g.wrpad, g.wstages);
@@ -640,25 +687,22 @@ static int launch_wide_t(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v,
                          cudaStream_t stream)
 {
     const size_t sm_rows = wide_rows_smem(plan->A, plan->K, g.wgains), sm_cols = wide_cols_smem(g.wrpad, g.wstages);
-    const int batches = (T + g.wtb - 1) / g.wtb;
-    // one batch: time chunks side by side, a slot each; more: one chunk a batch, past the last slot
-    // the sums go on in it
-    const int n_sub = batches == 1 ? wide_tau(g, T, plan->sm_count) : 1;
-    *n_tau = batches == 1 ? n_sub : std::min(batches, g.tau_cap);
+    const WideSplit split = wide_split(g.N, g.n_items, std::min(g.wcb, g.n_chan), g.wtb, g.tau_cap, T, plan->sm_count);
+    *n_tau = split.n_sub * split.rounds;
     const size_t slot = static_cast<size_t>(g.n_items) * 64 * 64;
     for (int c0 = 0; c0 < g.n_chan; c0 += g.wcb) {
         const int nc = std::min(g.wcb, g.n_chan - c0);
-        for (int b = 0; b < batches; b++) {
-            const int tb0 = static_cast<int>(static_cast<long long>(T) * b / batches);
-            const int nb = static_cast<int>(static_cast<long long>(T) * (b + 1) / batches) - tb0;
-            const int s = std::min(b, g.tau_cap - 1);
+        for (int b = 0; b < split.batches; b++) {
+            const int tb0 = static_cast<int>(static_cast<long long>(T) * b / split.batches);
+            const int nb = static_cast<int>(static_cast<long long>(T) * (b + 1) / split.batches) - tb0;
+            const int s = b % split.rounds * split.n_sub;
             const int chunks = fp32_pick_tau(nc * g.wbands, nb, plan->sm_count);
             wide_rows_kernel<Q><<<static_cast<unsigned>(nc * g.wbands * chunks), kRowsThreads, sm_rows, stream>>>(
                 v, gains, plan->d_kernel, plan->K, g.d_chans, g.d_wtab, g.d_widx, g.d_wchan, plan->A, plan->C, c0, g.wbands,
                 tb0, nb, chunks, g.wrpad, g.wgains ? 1 : 0, plan->d_dfreq, plan->delays ? plan->d_dtab : nullptr, g.d_wws);
-            wide_cols_kernel<Q><<<static_cast<unsigned>(nc * 2 * Q * n_sub), kColThreads, sm_cols, stream>>>(
-                g.d_wws, nb, nc, n_sub, c0, g.wrpad, g.wstages, b > s ? 1 : 0, reinterpret_cast<float4 *>(g.d_partial) + slot * s,
-                slot, plan->d_status, plan->wait_budget);
+            wide_cols_kernel<Q><<<static_cast<unsigned>(nc * 2 * Q * split.n_sub), kColThreads, sm_cols, stream>>>(
+                g.d_wws, nb, nc, split.n_sub, c0, g.wrpad, g.wstages, b >= split.rounds ? 1 : 0,
+                reinterpret_cast<float4 *>(g.d_partial) + slot * s, slot, plan->d_status, plan->wait_budget);
             if (cudaGetLastError() != cudaSuccess) return EPIC_ERR_CUDA;
         }
     }

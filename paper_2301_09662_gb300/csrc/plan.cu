@@ -914,28 +914,24 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                     g.wstages = epic::wide_stages(g.wrpad, static_cast<size_t>(smem_optin));
                 }
                 if (wrc == EPIC_OK && g.wstages > 0) {
-                    // channels per group and samples per batch within the workspace; whole integrations first
-                    const size_t per = static_cast<size_t>(g.N) * 2 * g.wrpad * sizeof(float2);
-                    constexpr size_t kBudget = size_t(4) << 30;
-                    g.wtb = static_cast<int>(std::max<size_t>(1, std::min<size_t>(max_spectra, kBudget / per)));
                     const int cap_tb = static_cast<int>((diag >> 16) & 255u);   // as for the fold path
-                    if (cap_tb > 0) g.wtb = std::min(g.wtb, cap_tb);
-                    const int most = static_cast<int>(std::max<size_t>(1, kBudget / (per * g.wtb)));
-                    const int n_grp = (g.n_chan + most - 1) / most;
-                    g.wcb = (g.n_chan + n_grp - 1) / n_grp;
+                    const epic::WideLayout lay =
+                        epic::wide_layout(g.N, g.n_chan, g.wrpad, max_spectra, cap_tb, g.tau_cap, p->sm_count);
+                    const size_t per = static_cast<size_t>(g.N) * 2 * g.wrpad * lay.cb * lay.tb;
                     // no room for the workspace: the paths below need less or none (the fold path's
                     // own batches, per-class gridding)
-                    g.wide = dev_upload(&g.d_wws, static_cast<const float2 *>(nullptr),
-                                        per / sizeof(float2) * g.wcb * g.wtb) == EPIC_OK;
+                    g.wide = dev_upload(&g.d_wws, static_cast<const float2 *>(nullptr), per) == EPIC_OK;
                     if (!g.wide) cudaGetLastError();
-                }
-                if (g.wide) {
-                    g.wforce = ((diag >> 16) & 255u) > 0;
-                    g.wgains = epic::wide_rows_smem_bytes(n_ant, p->K, true) + 64 <= static_cast<size_t>(smem_optin);
-                    g.tau_cap = std::max(g.tau_cap, epic::wide_pick_tau(g, max_spectra, p->sm_count));
-                    rc = dev_upload(&g.d_wtab, wtab.data(), wtab.size());
-                    if (rc == EPIC_OK) rc = dev_upload(&g.d_widx, widx.data(), widx.size());
-                    if (rc == EPIC_OK) rc = dev_upload(&g.d_wchan, wchan.data(), wchan.size());
+                    if (g.wide) {
+                        g.wcb = lay.cb;
+                        g.wtb = lay.tb;
+                        g.tau_cap = lay.slots;
+                        g.wforce = cap_tb > 0;
+                        g.wgains = epic::wide_rows_smem_bytes(n_ant, p->K, true) + 64 <= static_cast<size_t>(smem_optin);
+                        rc = dev_upload(&g.d_wtab, wtab.data(), wtab.size());
+                        if (rc == EPIC_OK) rc = dev_upload(&g.d_widx, widx.data(), widx.size());
+                        if (rc == EPIC_OK) rc = dev_upload(&g.d_wchan, wchan.data(), wchan.size());
+                    }
                 }
             }
             // large sides with one shared kernel of more than one tap: grid once per (channel,

@@ -86,8 +86,67 @@ static void efield()
               c.items, c.T);
 }
 
+// Wide kernels: buffers within their budgets, no FP32 sum longer than the per-class kernel's (side 256), and
+// long calls as well spread over the SMs as short ones.
+static void wide()
+{
+    const int sms = 152;
+    for (int N : {256, 512})
+        for (int chan : {1, 2, 16, 63, 64, 256, 1000})
+            for (int rpad : {32, 128})
+                for (int most : {1, 7, 100, 500, 1000, 5000, 9000, 20000}) {
+                    const int Q = N / 64, items = chan * Q * Q, tau = epic::fp32_pick_tau(items, most, sms);
+                    const epic::WideLayout w = epic::wide_layout(N, chan, rpad, most, 0, tau, sms);
+                    const double work = static_cast<double>(w.cb) * w.tb * N * 2 * rpad * 8;
+                    CHECK(w.cb >= 1 && w.cb <= chan && w.tb >= 1 && work <= 4.0 * (1ull << 30), "workspace: %d x %d", w.cb, w.tb);
+                    const double slot = static_cast<double>(chan) * N * N * 16;
+                    CHECK(w.slots <= tau || w.slots * slot <= 2.0 * (1ull << 30), "%d partial images of %g bytes", w.slots, slot);
+                    for (int T : {1, 2, 50, most / 2, most - 1, most}) {
+                        if (T < 1 || T > most) continue;
+                        const epic::WideSplit s = epic::wide_split(N, items, w.cb, w.tb, w.slots, T, sms);
+                        const int nb = (T + s.batches - 1) / s.batches, n = (nb + s.n_sub - 1) / s.n_sub;
+                        CHECK(s.batches % s.rounds == 0 && s.n_sub * s.rounds <= w.slots && nb <= w.tb, "side %d, %d channels, %d of %d: "
+                              "%d batches, %d x %d of %d slots", N, chan, T, most, s.batches, s.n_sub, s.rounds, w.slots);
+                        const int per_class = std::min(tau, epic::fp32_pick_tau(items, T, sms)), per_slot = s.batches / s.rounds;
+                        if (N == 256)
+                            CHECK(per_slot * n <= (T + per_class - 1) / per_class + 2 * per_slot, "side %d, %d channels, %d spectra: sums of %d",
+                                  N, chan, T, per_slot * n);
+                        // samples of column work on the busiest SM against an even spread
+                        if (T != most || T < 500) continue;
+                        double busy = 0;
+                        for (int c0 = 0; c0 < chan; c0 += w.cb) {
+                            const long long blocks = static_cast<long long>(std::min(w.cb, chan - c0)) * 2 * Q * s.n_sub;
+                            busy += static_cast<double>(s.batches) * ((blocks + sms - 1) / sms) * n;
+                        }
+                        const double even = std::max(1.0 * T * chan * 2 * Q / sms, T / 64.0);
+                        CHECK(busy <= 1.25 * even, "side %d, %d channels, %d rows, %d spectra: %g samples, %g if even", N, chan, rpad, T, busy,
+                              even);
+                    }
+                }
+}
+
+// The shapes by which test_gpu_wide.py continues sums in a partial image and images channels in two groups
+static void wide_test_shapes()
+{
+    const struct {
+        int N, C, T, most, cap, rpad;
+        bool more;      // batches beyond the first set of partial images
+        int groups;
+    } at[] = {{512, 2, 7, 7, 1, 112, true, 1}, {512, 2, 7, 7, 3, 112, true, 1},   {256, 2, 16, 16, 1, 128, true, 1},
+              {256, 2, 8, 8, 3, 128, false, 1}, {512, 63, 2, 100, 200, 128, false, 2}, {512, 9, 5, 5, 2, 80, true, 1}};
+    for (const auto &c : at) {
+        const int items = c.C * (c.N / 64) * (c.N / 64);
+        const epic::WideLayout w = epic::wide_layout(c.N, c.C, c.rpad, c.most, c.cap, epic::fp32_pick_tau(items, c.most, 152), 152);
+        const epic::WideSplit s = epic::wide_split(c.N, items, w.cb, w.tb, w.slots, c.T, 152);
+        CHECK((s.batches > s.rounds) == c.more && (c.C + w.cb - 1) / w.cb == c.groups, "side %d, %d x %d: %d batches, %d rounds, %d channels",
+              c.N, c.C, c.T, s.batches, s.rounds, w.cb);
+    }
+}
+
 int main()
 {
+    wide();
+    wide_test_shapes();
     efield();
     fork32();
     tiles();

@@ -32,10 +32,12 @@ def _case(N, A, T, K, span_x, span_y, C=2):
     (512, 44, 2, 5, 63, 65, 0),                            # one row in the second band
     (512, 36, 7, 3, 66, 33, 0),                            # one band, folded columns only
     (512, 40, 4, 5, 100, 120, epic.EPIC_KERNEL_TAPER),     # one tap
-    (512, 40, 7, 5, 90, 100, epic.EPIC_DIAG_ALIAS_BATCH(3)),  # three time batches into one partial image
+    (512, 40, 7, 5, 90, 100, epic.EPIC_DIAG_ALIAS_BATCH(3)),  # three time batches into the same partial images
+    (512, 40, 7, 5, 90, 100, epic.EPIC_DIAG_ALIAS_BATCH(1)),  # seven into one
     (256, 60, 9, 5, 128, 127, 0),
     (256, 30, 1, 3, 17, 16, epic.EPIC_STOKES),             # one sample, one block of 16 rows
-    (256, 34, 8, 7, 60, 128, epic.EPIC_DIAG_ALIAS_BATCH(3)),
+    (256, 34, 8, 7, 60, 128, epic.EPIC_DIAG_ALIAS_BATCH(3)),   # batches into a partial image each
+    (256, 34, 16, 7, 60, 128, epic.EPIC_DIAG_ALIAS_BATCH(1)),  # sixteen into four in turn
 ])
 def test_edges(N, A, T, K, sx, sy, flags):
     wl = _case(N, A, T, K, sx, sy)
@@ -82,6 +84,19 @@ def test_no_room_for_the_workspace():
     del hold
     torch.cuda.empty_cache()
     assert peak_rel_err(got, oracle.workload_image(wl), wl.grid_n, 2).max() < TOL
+
+
+def test_two_channel_groups():
+    """63 channels x 100 spectra take two turns of the workspace, the second of one channel fewer."""
+    wl = _case(512, 24, 2, 3, 126, 120, C=63)
+    p = epic.Plan.from_workload(wl, flags=WIDE, max_spectra=100)
+    got, _ = run_gpu(wl, plan=p)
+    p.close()
+    ch = [0, 31, 32, 62]
+    got = [oracle.split_channels(got, wl.grid_n, 2)[c] for c in ch]
+    ref = oracle.split_channels(oracle.workload_image(wl, channels=ch), wl.grid_n[ch], 2)
+    for a, b in zip(got, ref):
+        assert np.max(np.abs(a - b)) / np.max(np.abs(b[:2])) < TOL
 
 
 @pytest.mark.parametrize("flags", [0, epic.EPIC_DIAG_ALIAS_BATCH(3)])
