@@ -918,19 +918,31 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                     const epic::WideLayout lay =
                         epic::wide_layout(g.N, g.n_chan, g.wrpad, max_spectra, cap_tb, g.tau_cap, p->sm_count);
                     const size_t per = static_cast<size_t>(g.N) * 2 * g.wrpad * lay.cb * lay.tb;
-                    // no room for the workspace: the paths below need less or none (the fold path's
-                    // own batches, per-class gridding)
-                    g.wide = dev_upload(&g.d_wws, static_cast<const float2 *>(nullptr), per) == EPIC_OK;
-                    if (!g.wide) cudaGetLastError();
+                    g.wide = dev_upload(&g.d_wws, static_cast<const float2 *>(nullptr), per) == EPIC_OK &&
+                             dev_upload(&g.d_partial, static_cast<const float *>(nullptr),
+                                        static_cast<size_t>(lay.slots) * g.n_items * g.M * g.M * npf) == EPIC_OK &&
+                             dev_upload(&g.d_wtab, wtab.data(), wtab.size()) == EPIC_OK &&
+                             dev_upload(&g.d_widx, widx.data(), widx.size()) == EPIC_OK &&
+                             dev_upload(&g.d_wchan, wchan.data(), wchan.size()) == EPIC_OK;
                     if (g.wide) {
                         g.wcb = lay.cb;
                         g.wtb = lay.tb;
                         g.tau_cap = lay.slots;
                         g.wforce = cap_tb > 0;
                         g.wgains = epic::wide_rows_smem_bytes(n_ant, p->K, true) + 64 <= static_cast<size_t>(smem_optin);
-                        rc = dev_upload(&g.d_wtab, wtab.data(), wtab.size());
-                        if (rc == EPIC_OK) rc = dev_upload(&g.d_widx, widx.data(), widx.size());
-                        if (rc == EPIC_OK) rc = dev_upload(&g.d_wchan, wchan.data(), wchan.size());
+                    } else {
+                        // no room: the paths below need less or none (the fold path's own batches, per-class
+                        // gridding)
+                        cudaGetLastError();
+                        auto drop = [](auto *&q) {
+                            cudaFree(q);
+                            q = nullptr;
+                        };
+                        drop(g.d_wws);
+                        drop(g.d_partial);
+                        drop(g.d_wtab);
+                        drop(g.d_widx);
+                        drop(g.d_wchan);
                     }
                 }
             }
@@ -1033,7 +1045,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 rc = dev_upload(&g.d_Y, static_cast<const float4 *>(nullptr),
                                 static_cast<size_t>(g.n_chan) * 4 * K * g.N);
         }
-        if (rc == EPIC_OK)
+        if (rc == EPIC_OK && !g.d_partial)
             rc = dev_upload(&g.d_partial, static_cast<const float *>(nullptr),
                             static_cast<size_t>(g.tau_cap) * g.n_items * g.M * g.M * npf);
         p->groups.push_back(g);

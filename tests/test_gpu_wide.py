@@ -99,6 +99,33 @@ def test_two_channel_groups():
         assert np.max(np.abs(a - b)) / np.max(np.abs(b[:2])) < TOL
 
 
+def test_no_room_for_the_partial_images():
+    """44 MiB left: the workspace (16) fits, with its nine partial images (36) it does not, and the
+    plan images per class with two (8)."""
+    import torch
+    wl = _case(512, 40, 64, 3, 30, 28, C=1)
+    v, g = torch_inputs(wl)
+    out = torch.empty(4 * 512 * 512, dtype=torch.complex64, device="cuda")
+    for flags in (WIDE, epic.EPIC_DIAG_NO_ALIAS):        # loads both paths' kernels
+        p = epic.Plan.from_workload(wl, flags=flags)
+        p.image(v, g, out=out)
+        torch.cuda.synchronize()
+        p.close()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (44 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        p = epic.Plan.from_workload(wl)
+        p.image(v, g, out=out)
+        torch.cuda.synchronize()
+        assert p.status() == epic.EPIC_OK
+        p.close()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    got = out.cpu().numpy().astype(np.complex128)
+    assert peak_rel_err(got, oracle.workload_image(wl), wl.grid_n, 2).max() < TOL
+
+
 @pytest.mark.parametrize("flags", [0, epic.EPIC_DIAG_ALIAS_BATCH(3)])
 def test_channels_on_both_sides_of_the_range(flags):
     """Two of three channels span at most 128 cells: a group each, one stage of the side."""
