@@ -364,7 +364,8 @@ void epic_destroy(epic_plan_t plan);
  * epic_stage_times waits for the last such call and writes the device time in
  * milliseconds of each launch, in launch order: [0] the auto-power kernel
  * (absent with EPIC_NO_AUTOSUB), then for each grid side in ascending order
- * the imaging kernel and its epilogue.  Returns the number of values written
+ * the imaging kernel and its epilogue (of a side's channels in two groups, the
+ * time that either group's ran).  Returns the number of values written
  * (at most max_stages), or a negative EPIC_ERR_* code (EPIC_ERR_ARG if
  * profiling is off or no call was recorded).
  */

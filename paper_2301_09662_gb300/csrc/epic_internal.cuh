@@ -191,6 +191,7 @@ struct epic_plan_s {
 namespace epic {
 
 // Stage timing helpers: no-ops unless profiling is on.
+float stage_union(float s0, float e0, float s1, float e1);   // time covered by two intervals
 void prof_begin(epic_plan_s *plan);
 void prof_mark(epic_plan_s *plan, cudaStream_t stream, int stage, bool start);
 

@@ -520,6 +520,12 @@ int build_gather_table(const std::vector<short2> &cells, int A, int K, int M, in
     return EPIC_OK;
 }
 
+// Time covered by the intervals (s0, e0) and (s1, e1)
+float stage_union(float s0, float e0, float s1, float e1)
+{
+    return (e0 - s0) + (e1 - s1) - std::max(0.f, std::min(e0, e1) - std::max(s0, s1));
+}
+
 void prof_begin(epic_plan_s *plan)
 {
     if (plan->profiling) plan->n_recorded = 0;
@@ -1511,22 +1517,19 @@ int epic_stage_times(epic_plan_t plan, float *ms, int max_stages)
     if (!plan->profiling || plan->n_recorded == 0) return EPIC_ERR_ARG;
     for (int i = 0; i < plan->n_recorded; i++)
         if (cudaEventSynchronize(plan->events[2 * i + 1]) != cudaSuccess) return EPIC_ERR_CUDA;
-    // the groups of one side (two at most, one after the other) are one stage: from the first start to
-    // the last end
+    // the groups of one side (two at most, in branches of their own) are one stage: the time that
+    // either of them ran
     const int lead = plan->n_recorded - 2 * static_cast<int>(plan->groups.size());   // the auto sums
     int n = 0;
     for (int i = 0; i < plan->n_recorded && n < max_stages; i++) {
         const size_t gi = static_cast<size_t>(std::max(0, i - lead) / 2);
         if (i >= lead && gi > 0 && plan->groups[gi].N == plan->groups[gi - 1].N) continue;   // counted already
         const bool two = i >= lead && gi + 1 < plan->groups.size() && plan->groups[gi + 1].N == plan->groups[gi].N;
-        float most = 0.f;
-        for (int u = i; u <= (two ? i + 2 : i); u += 2)
-            for (int w = i; w <= (two ? i + 2 : i); w += 2) {
-                float t;
-                if (cudaEventElapsedTime(&t, plan->events[2 * u], plan->events[2 * w + 1]) != cudaSuccess) return EPIC_ERR_CUDA;
-                most = std::max(most, t);
-            }
-        ms[n++] = most;
+        float at[4] = {0.f, 0.f, 0.f, 0.f};   // starts and ends from this one's start
+        for (int k = 1; k < (two ? 4 : 2); k++)
+            if (cudaEventElapsedTime(&at[k], plan->events[2 * i], plan->events[2 * i + (k < 2 ? k : k + 2)]) != cudaSuccess)
+                return EPIC_ERR_CUDA;
+        ms[n++] = two ? epic::stage_union(at[0], at[1], at[2], at[3]) : at[1];
     }
     return n;
 }

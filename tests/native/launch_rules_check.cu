@@ -143,8 +143,16 @@ static void wide_test_shapes()
     }
 }
 
+// A stage of two groups: the time either ran, not the span between them
+static void stage_time()
+{
+    CHECK(epic::stage_union(0, 2, 10, 13) == 5 && epic::stage_union(0, 2, -7, -4) == 5, "apart");
+    CHECK(epic::stage_union(0, 4, 3, 9) == 9 && epic::stage_union(0, 9, 2, 5) == 9 && epic::stage_union(0, 3, -2, 1) == 5, "overlapping");
+}
+
 int main()
 {
+    stage_time();
     wide();
     wide_test_shapes();
     efield();
