@@ -313,6 +313,7 @@ int compact_pick_tau(int n_chan, int n_items, int T, int sms);
 bool fork_pays(int n_items, int n_tau, int T, int sms);   // side 32: auto sums beside the imaging
 int series_chunks(int items, int n_img, int spi, int tau_cap, int sms);   // compact groups: time chunks per image
 // time chunks of one launch: forced (image series), else autotuned for this T, else the cost model
+bool tunable(const epic_plan_s *plan, const GroupCfg &g, int T);   // epic_autotune has something to measure
 int choose_tau(const epic_plan_s *plan, const GroupCfg &g, int T);
 // large grid sides (GroupCfg::alias)
 size_t fold64_smem_bytes(int P);

@@ -409,6 +409,9 @@ int prepare_fp32(const epic_plan_s *plan, const GroupCfg &g)
     }
 }
 
+// Whether a call of T spectra has time chunks to tune: the fold path and the wide kernels have their own
+bool tunable(const epic_plan_s *plan, const GroupCfg &g, int T) { return !(g.alias || (g.wide && wide_pays(plan, g, T))); }
+
 int launch_imaging(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
                    cudaStream_t s)
 {

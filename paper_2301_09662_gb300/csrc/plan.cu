@@ -1215,7 +1215,7 @@ int epic_autotune(epic_plan_t plan, int n_spectra, void *stream)
     if (rc == EPIC_OK && autosub) rc = epic::launch_autopower(plan, v, nullptr, n_spectra, s);
     for (auto &g : plan->groups) {
         if (rc != EPIC_OK) break;
-        if (g.alias || g.wide) continue;     // time chunks set by the plan: nothing to tune
+        if (!epic::tunable(plan, g, n_spectra)) continue;
         const int cap = std::max(1, std::min(g.tau_cap, n_spectra));
         std::vector<int> cand;
         auto add = [&](int n) {

@@ -150,8 +150,26 @@ static void stage_time()
     CHECK(epic::stage_union(0, 4, 3, 9) == 9 && epic::stage_union(0, 9, 2, 5) == 9 && epic::stage_union(0, 3, -2, 1) == 5, "overlapping");
 }
 
+// A wide group's small calls go to the per-class kernel, whose time chunks are tuned like any other's
+static void tuning()
+{
+    epic_plan_s plan;
+    plan.A = 300;
+    plan.K = 5;
+    epic::GroupCfg g;
+    g.N = 256;
+    g.n_items = 2 * 16;
+    CHECK(epic::tunable(&plan, g, 16), "per-class group");
+    g.wide = true;
+    CHECK(epic::tunable(&plan, g, 16) && !epic::tunable(&plan, g, 100), "wide group, small and ordinary call");
+    g.wide = false;
+    g.alias = true;
+    CHECK(!epic::tunable(&plan, g, 16), "fold path");
+}
+
 int main()
 {
+    tuning();
     stage_time();
     wide();
     wide_test_shapes();
