@@ -313,9 +313,11 @@ wide_cols_kernel(const float2 *__restrict__ ws, int nb, int nc, int n_sub, int c
     };
 
     // sample q's tile into its buffer, one bulk copy a polarisation (warp 0)
+    int fetched = 0;
     auto fetch = [&](int q) {
         const int s = q % stages, use = q / stages;
         if (use > 0) wait(empty[s], (use - 1) & 1);
+        if (!dead) fetched = q + 1;
         if (lane == 0 && !dead) {
             tc::mbar_expect_tx(&full[s], 2 * bytes);
             const float2 *src = ws + ((static_cast<size_t>(cb) * nb + b0 + q) * Q + hx) * 2 * 64 * rpad + static_cast<size_t>(m0) * rpad;
@@ -441,6 +443,8 @@ wide_cols_kernel(const float2 *__restrict__ ws, int nb, int nc, int n_sub, int c
             }
         }
     }
+    if (tid == 0 && dead)                // copies still in flight land before the block's memory is another's
+        for (int q = max(0, fetched - stages); q < fetched; q++) tc::mbar_wait(&full[q % stages], (q / stages) & 1, wait_budget);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
