@@ -45,7 +45,8 @@ struct GroupCfg {
     std::vector<int> chans;            // plan channel indices in this group
     int *d_chans = nullptr;            // device copy of chans
     long long *d_out_off = nullptr;    // device: output offset (complex elements) per group channel
-    float2 *d_wpow = nullptr;          // device: |W^(l)|^2 on the shifted [N][N] layout, as FP32 pairs (hi, lo)
+    float2 *d_wpow = nullptr;          // device: |W^(l)|^2 / wscale on the shifted [N][N] layout, as FP32 pairs (hi, lo)
+    double wscale = 1;                 // a power of two
     double2 *d_tw64 = nullptr;         // per-antenna kernels: exp(+2 pi i k / N) in FP64
     float4 *d_twp = nullptr;           // per-antenna kernels: (cos, -sin) of 2 pi k / N as FP32 pairs
     float4 *d_Y = nullptr;             // per-antenna kernels: [n_chan][4][K][N] half-transformed auto grids, FP32 pairs
@@ -302,7 +303,8 @@ struct RawImage {
     const float2 *kernel = nullptr;    // [K*K]
     const int *chans = nullptr;        // [C] identity channel list
     const long long *out_off = nullptr;  // [C]
-    const float2 *wpow = nullptr;      // [N][N], FP32 pairs
+    const float2 *wpow = nullptr;      // [N][N], FP32 pairs, divided by wscale
+    double wscale = 1;
     const float2 *twN = nullptr;       // [N]
     float *partial = nullptr;          // [n_tau][n_items][M*M][NPF]
     int *autoint = nullptr;            // [C][A][4]
@@ -332,7 +334,7 @@ int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, int
 // host tables shared by the plan and the static-scratch entry point
 int host_cell_map(const double *ant_xy_m, int n_ant, const double *freq_hz, int n_chan, const int *grid_n,
                   double du, int K, std::vector<short2> &cells);
-void host_kernel_power(const float *kern, int K, int N, std::vector<float2> &out);
+double host_kernel_power(const float *kern, int K, int N, bool taper, std::vector<float2> &out);   // returns the table's scale
 // raise a kernel's dynamic shared-memory cap to the device limit (less its static shared memory);
 // EPIC_ERR_UNSUPPORTED if `need` does not fit
 int raise_dyn_smem_cap(const void *kfn, size_t need);

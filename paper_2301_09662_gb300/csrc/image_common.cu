@@ -153,11 +153,11 @@ auto_sum_kernel(const int *__restrict__ autoint, int n_chunks, size_t chunk_stri
     if (threadIdx.x < 4) apq_out[(static_cast<size_t>(blockIdx.y) * C + blockIdx.x) * 4 + threadIdx.x] = apq[threadIdx.x];
 }
 
-// A number as an unevaluated FP32 pair (hi, lo), about 48 bits.
+// A number as an unevaluated FP32 pair (hi, lo), about 48 bits (infinity as itself).
 __device__ __forceinline__ float2 to_pair(double x)
 {
     const float hi = static_cast<float>(x);
-    return make_float2(hi, static_cast<float>(x - static_cast<double>(hi)));
+    return make_float2(hi, isinf(hi) ? 0.f : static_cast<float>(x - static_cast<double>(hi)));
 }
 // h + x exactly as (sum, error): the error is returned (Knuth's TwoSum)
 __device__ __forceinline__ float two_sum(float &h, float x)
@@ -194,17 +194,20 @@ __device__ __forceinline__ void pair_msub(float2 &s, float2 a, float2 b)
 // 88 and 78.  Whole calls: 25 Stokes images of
 // 64 channels of 128 x 128 5.21 -> 3.66 ms, 64 channels of 512 x 512 with 2048
 // antennas 21.75 -> 20.40 ms.
-// AK: an auto image from the per-antenna auto-correlation grids (Yauto) instead of A_pq |W^|^2
-template <int N, int M, int P, bool AK>
+// MODE: kShared; kAntennas: an auto image from the per-antenna auto-correlation grids (Yauto) instead of
+// A_pq |W^|^2; kTaper64: a taper whose |W^|^2 leaves FP32's exponents, applied in FP64
+enum { kShared, kAntennas, kTaper64 };
+template <int N, int M, int P, int MODE>
 __global__ void __launch_bounds__(kThreads, 4)
 epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R1, int R2,
                 const int *__restrict__ chans, const long long *__restrict__ out_off,
-                const float2 *__restrict__ wpow, const double *__restrict__ apq_tab, const int *__restrict__ autoint,
+                const float2 *__restrict__ wpow, double wscale, const double *__restrict__ apq_tab, const int *__restrict__ autoint,
                 int auto_n, size_t auto_stride,
                 const float2 *__restrict__ gains, int A, int C, int T, unsigned flags, float2 *__restrict__ out,
                 long long out_stride, const float4 *__restrict__ Yauto, const float4 *__restrict__ twp, int K)
 {
     constexpr int NPF = P == 2 ? 4 : 1;          // sums and products per pixel
+    constexpr bool AK = MODE == kAntennas;
     constexpr int up = N < M ? M / N : 1, Q1 = N < M ? 1 : N / M, Q = Q1 * Q1, NN = N * N;
     // blockIdx.z = image: it sums time chunks [z n_tau, (z + 1) n_tau) and uses
     // the auto sums and output block of index z (one image unless a series)
@@ -219,11 +222,20 @@ epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R
     __shared__ double apq[4];   // XX, YY, Re XY, Im XY (YX = conj XY)
     if (autosub && !AK && !apq_tab)
         auto_reduce<P>(autoint + static_cast<size_t>(img) * auto_n * auto_stride, auto_n, auto_stride, gains, A, c, red, apq);
+    // |W^|^2's scale, a power of two, goes into A_pq (not with the taper, where A_pq has the sums' own);
+    // by one thread each, since the FP64 pipe does ~2 operations a clock
+    constexpr bool taper64 = MODE == kTaper64;
+    const bool taper = taper64 || (flags & EPIC_KERNEL_TAPER) != 0;
+    __shared__ float2 aqs[4];
+    if (!AK && threadIdx.x < NPF) {
+        double a = 0;
+        if (autosub) a = apq_tab ? apq_tab[(static_cast<size_t>(img) * C + c) * 4 + threadIdx.x] : apq[threadIdx.x];
+        aqs[threadIdx.x] = to_pair(taper ? a : a * wscale);
+    }
+    if (!AK) __syncthreads();
     float2 aq[NPF];
 #pragma unroll
-    for (int k = 0; k < NPF; k++)
-        aq[k] = autosub && !AK ? to_pair(apq_tab ? apq_tab[(static_cast<size_t>(img) * C + c) * 4 + k] : apq[k])
-                                        : make_float2(0.f, 0.f);
+    for (int k = 0; k < NPF; k++) aq[k] = AK ? make_float2(0.f, 0.f) : aqs[k];
 
     const double scale = ((flags & EPIC_MEAN) && T > 0) ? 1.0 / T : 1.0;
     float2 *oc = out + out_off[ci];
@@ -279,12 +291,17 @@ epilogue_kernel(const float *__restrict__ partial, int n_tau, int n_items, int R
                 }
             }
         } else {
-            if (flags & EPIC_KERNEL_TAPER) {
+            if (taper) {
                 // point-gridded sums: subtract the bare autos, then apply |W^(l)|^2
 #pragma unroll
                 for (int k = 0; k < NPF; k++) {
                     float2 d = s[k];
                     d.y += two_sum(d.x, -aq[k].x) - aq[k].y;
+                    if constexpr (taper64) {
+                        const double x = static_cast<double>(d.x) + static_cast<double>(d.y);
+                        s[k] = to_pair(x * (static_cast<double>(w.x) + static_cast<double>(w.y)) * wscale);
+                        continue;
+                    }
                     const float p = __fmul_rn(d.x, w.x);
                     s[k] = make_float2(p, fmaf(d.x, w.y, fmaf(d.y, w.x, fmaf(d.x, w.x, -p))));
                 }
@@ -449,9 +466,11 @@ int launch_epi(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T,
         constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
         const dim3 grid(static_cast<unsigned>(epi_tiles(N, g.n_chan * n_img, plan->sm_count)), static_cast<unsigned>(g.n_chan),
                         static_cast<unsigned>(n_img));
-        const auto kfn = plan->nker > 1 ? epilogue_kernel<N, M, P, true> : epilogue_kernel<N, M, P, false>;
+        const auto kfn = plan->nker > 1                                                    ? epilogue_kernel<N, M, P, kAntennas>
+                         : (plan->flags & EPIC_KERNEL_TAPER) && g.wscale != 1.0 ? epilogue_kernel<N, M, P, kTaper64>
+                                                                                : epilogue_kernel<N, M, P, kShared>;
         kfn<<<grid, kThreads, 0, stream>>>(
-            g.d_partial, n_tau, g.n_items, g.R1, g.R2, g.d_chans, g.d_out_off, g.d_wpow,
+            g.d_partial, n_tau, g.n_items, g.R1, g.R2, g.d_chans, g.d_out_off, g.d_wpow, g.wscale,
             plan->d_apq, nullptr, 0, 0, gains, plan->A, plan->C, T, plan->flags, out, static_cast<long long>(plan->out_floats / 2),
             g.d_Y, g.d_twp, plan->K);
         return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
@@ -513,9 +532,10 @@ int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, int
     return epi_dispatch(r.N, r.M, r.P, [&](auto n_, auto m_, auto p_) {
         constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
         const dim3 grid(static_cast<unsigned>(epi_tiles(N, r.C, sm_count)), static_cast<unsigned>(r.C));
-        epilogue_kernel<N, M, P, false><<<grid, kThreads, 0, stream>>>(r.partial, r.n_tau, r.n_items, 8, M / 8, r.chans, r.out_off,
-                                                                r.wpow, nullptr, r.autoint, 1, 0, gains, r.A, r.C, r.T, r.flags,
-                                                                out, 0, nullptr, nullptr, 0);
+        const auto kfn = (r.flags & EPIC_KERNEL_TAPER) && r.wscale != 1.0 ? epilogue_kernel<N, M, P, kTaper64>
+                                                                          : epilogue_kernel<N, M, P, kShared>;
+        kfn<<<grid, kThreads, 0, stream>>>(r.partial, r.n_tau, r.n_items, 8, M / 8, r.chans, r.out_off, r.wpow, r.wscale, nullptr,
+                                           r.autoint, 1, 0, gains, r.A, r.C, r.T, r.flags, out, 0, nullptr, nullptr, 0);
         return cudaGetLastError() == cudaSuccess ? EPIC_OK : EPIC_ERR_CUDA;
     });
 }

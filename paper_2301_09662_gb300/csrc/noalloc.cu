@@ -94,7 +94,7 @@ extern "C" int epic_image_static(const double *ant_xy_m, int n_ant, int n_pol, c
     if (rc != EPIC_OK) return rc;
     const int N = grid_n, M = N / Q1, NP = n_pol == 2 ? 4 : 1, NPF = n_pol == 2 ? 4 : 1;
     std::vector<float2> wpow;
-    host_kernel_power(kernel_c64, K, N, wpow);
+    const double wscale = host_kernel_power(kernel_c64, K, N, (flags & EPIC_KERNEL_TAPER) != 0, wpow);
 
     // ---- scratch layout (all offsets 256-byte aligned)
     size_t off = 0;
@@ -168,6 +168,7 @@ extern "C" int epic_image_static(const double *ant_xy_m, int n_ant, int n_pol, c
     r.chans = reinterpret_cast<const int *>(scratch + o_chans);
     r.out_off = reinterpret_cast<const long long *>(scratch + o_outoff);
     r.wpow = reinterpret_cast<const float2 *>(scratch + o_wpow);
+    r.wscale = wscale;
     r.twN = reinterpret_cast<const float2 *>(scratch + o_twN);
     r.autoint = reinterpret_cast<int *>(scratch + o_auto);
     r.partial = reinterpret_cast<float *>(scratch + o_partial);

@@ -183,15 +183,26 @@ int host_cell_map(const double *ant_xy_m, int n_ant, const double *freq_hz, int 
     return EPIC_OK;
 }
 
-void host_kernel_power(const float *kern, int K, int N, std::vector<float2> &out)
+// |W^|^2 as FP32 pairs divided by a power of two, which is returned.  Without a taper it brings the largest
+// value to 1 .. 2 and goes into A_pq instead, in FP64 (epilogue_kernel), so that a pair of either holds
+// what FP64 did: their product has the scale of the image, but A_pq alone leaves FP32's exponents with
+// gains above about 1e17 or below 1e-18.  With a taper A_pq has the scale of the sums it is taken from,
+// and |W^|^2 is scaled only where it leaves 2^-40 .. 2^40.
+double host_kernel_power(const float *kern, int K, int N, bool taper, std::vector<float2> &out)
 {
     std::vector<double> w;
     kernel_power(kern, K, N, w);
+    double most = 0;
+    for (double x : w) most = std::max(most, x);
+    int e = most > 0 && std::isfinite(most) ? std::ilogb(most) : 0;
+    if (taper && std::abs(e) <= 40) e = 0;
     out.resize(w.size());
     for (size_t i = 0; i < w.size(); i++) {
-        const float hi = static_cast<float>(w[i]);
-        out[i] = make_float2(hi, static_cast<float>(w[i] - static_cast<double>(hi)));
+        const double x = std::ldexp(w[i], -e);
+        const float hi = static_cast<float>(x);
+        out[i] = make_float2(hi, static_cast<float>(x - static_cast<double>(hi)));
     }
+    return std::ldexp(1.0, e);
 }
 
 // A kernel's dynamic shared-memory cap holds for the whole process, so it is
@@ -799,7 +810,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
         std::vector<long long> offs(g.n_chan);
         for (int i = 0; i < g.n_chan; i++) offs[i] = p->out_off[g.chans[i]];
         std::vector<float2> wpow;
-        epic::host_kernel_power(kernel_c64, K, g.N, wpow);
+        g.wscale = epic::host_kernel_power(kernel_c64, K, g.N, taper, wpow);
         std::vector<float2> tw(g.N);
         for (int k = 0; k < g.N; k++) {
             const double ang = 2.0 * M_PI * k / g.N;
