@@ -233,7 +233,7 @@ int launch_tc_dual_fold(epic_plan_s *plan, const GroupCfg &g, const float2 *gain
 int launch_tc_dual(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
                    cudaStream_t stream);
 // grid sides 128 and 64: the gather-gridding pair kernel (tc_pair128.cu)
-void pair_origin(const std::vector<short2> &cells, int A, int K, const std::vector<int> &chans, int M,
+void pair_origin(const std::vector<short2> &cells, int A, int K, const std::vector<int> &chans, int M, bool move,
                  std::vector<short2> &moved, std::vector<int2> &kblk);
 int build_pair_tables(const std::vector<short2> &cells, int A, int K, const std::vector<int> &chans,
                       const std::vector<uint32_t> &tab32, const std::vector<int4> &idx32,

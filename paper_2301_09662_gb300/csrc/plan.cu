@@ -997,7 +997,10 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
             // 48-point DFTs in the 64-point operands; without the pair kernel it stays on the FP32
             // kernel); grid side 64: the same kernel with its one class
             const bool pair_side = (g.tensor && (g.N == 128 || g.N == 64)) || (tensor && g.N == 96 && g.reg64);
-            if (rc == EPIC_OK && pair_side && n_pol == 2 && p->nker == 1 && !(diag & EPIC_DIAG_NO_PAIR)) {
+            // (from the aperture's corner, or, should the lists only fit so, from where it lies: the pairing of
+            // adjacent cells differs)
+            const bool pair_ok = pair_side && n_pol == 2 && p->nker == 1 && !(diag & EPIC_DIAG_NO_PAIR);
+            for (int moved = 1; moved >= 0 && rc == EPIC_OK && pair_ok && !g.pair; moved--) {
                 std::vector<uint32_t> tab32;
                 std::vector<int4> idx32, pidx;
                 std::vector<int2> chan32, pchan;
@@ -1005,7 +1008,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 std::vector<uint16_t> ptab;
                 std::vector<short2> pcells;
                 std::vector<int2> pkblk;
-                epic::pair_origin(cells, n_ant, p->K, g.chans, g.M, pcells, pkblk);
+                epic::pair_origin(cells, n_ant, p->K, g.chans, g.M, moved != 0, pcells, pkblk);
                 if (epic::build_gather_table(pcells, n_ant, p->K, g.M, 2, g.chans, tab32, idx32, chan32, rows32) ==
                         EPIC_OK &&
                     epic::build_pair_tables(pcells, n_ant, p->K, g.chans, tab32, idx32, chan32, ptab, pidx, pchan,

@@ -694,12 +694,14 @@ const void *pair_kernel(int cls, int mf)
 // multiplies F(l) by one unit factor common to both polarisations, which cancels in every product;
 // an aperture that occupies 48 of 64 folded rows then leaves a k-block of zeros out of every column
 // stage (and out of the row stages by its columns), wherever on the grid it lies.
-void pair_origin(const std::vector<short2> &cells, int A, int K, const std::vector<int> &chans, int M,
+// Without `move` the cells stay, with all k-blocks.
+void pair_origin(const std::vector<short2> &cells, int A, int K, const std::vector<int> &chans, int M, bool move,
                  std::vector<short2> &moved, std::vector<int2> &kblk)
 {
     const int h = (K - 1) / 2;
     moved = cells;
     kblk.assign(chans.size(), make_int2(M / 16, M / 16));
+    if (!move) return;
     for (size_t ci = 0; ci < chans.size(); ci++) {
         short2 *cc = moved.data() + static_cast<size_t>(chans[ci]) * A;
         int x0 = 1 << 20, x1 = -1, y0 = 1 << 20, y1 = -1;

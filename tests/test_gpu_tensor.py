@@ -303,3 +303,15 @@ def test_pair_kernel_empty_integration_is_zero(N):
     assert p.status() == epic.EPIC_OK
     assert torch.count_nonzero(out) == 0
     p.close()
+
+
+@pytest.mark.parametrize("seed", [106, 132])
+def test_lists_that_fit_only_where_the_aperture_lies(seed):
+    """328 antennas whose lists exceed shared memory once the cells move to the aperture's corner
+    (another pairing of adjacent cells) but not as they lie; side 96 has no other tensor kernel."""
+    wl = synth.random_small(A=328, P=2, C=1, T=3, N=96, K=5, seed=seed)
+    wl.ant_xy = np.random.default_rng(seed).uniform(-9, 9, (328, 2)) * synth.C0 / 60e6 * 0.5
+    wl.freq_hz = np.array([60e6])
+    got, p = run_gpu(wl, precision=epic.EPIC_TC_SPLIT_FP16)
+    p.close()
+    assert peak_rel_err(got, oracle.workload_image(wl), wl.grid_n, 2).max() < 1e-5
