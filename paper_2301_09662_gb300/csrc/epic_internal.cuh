@@ -249,7 +249,7 @@ int launch_tc_pair(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const
 // built on up to `threads` host threads (0: automatic); the result does not depend on it.
 int build_gather_table(const std::vector<short2> &cells, int A, int K, int M, int P, const std::vector<int> &chans,
                        std::vector<uint32_t> &tab, std::vector<int4> &idx, std::vector<int2> &chan,
-                       std::vector<unsigned long long> &rowmask, int threads = 0);
+                       std::vector<unsigned long long> &rowmask, int threads = 0, bool search = true);
 // FP32 kernel for apertures of at most 64 x 64 cells, grid sides 64, 96, 128 (fp32_compact.cu)
 int build_compact_lists(const std::vector<short2> &cells, int A, int K, int P, const std::vector<int> &chans,
                         std::vector<uint16_t> &tab, std::vector<int2> &idx, std::vector<int4> &chan);

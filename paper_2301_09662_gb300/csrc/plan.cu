@@ -339,11 +339,12 @@ int build_reg64_schedule(const std::vector<short2> &cells, int A, int K, int M, 
 //   idx[ci * 8 + w] = (zero list offset, zero steps, first batch offset, batches), offsets from the
 //   channel block's start; chan[ci] = (block start, block words)
 // Channels are built in parallel on up to `threads` host threads (0: up to 16, or the hardware's
-// count); the table does not depend on the thread count.  A host allocation failure returns
+// count); the table does not depend on the thread count.  Without `search` the step order is the greedy
+// one (about half the time: for tables that only small calls read).  A host allocation failure returns
 // EPIC_ERR_NOMEM, a layout the format cannot hold EPIC_ERR_UNSUPPORTED.
 int build_gather_table(const std::vector<short2> &cells, int A, int K, int M, int P, const std::vector<int> &chans,
                        std::vector<uint32_t> &tab, std::vector<int4> &idx, std::vector<int2> &chan,
-                       std::vector<unsigned long long> &rowmask, int threads)
+                       std::vector<unsigned long long> &rowmask, int threads, bool search)
 {
     constexpr int W = 8;
     const int h = (K - 1) / 2, S = M + 1, MP = M / 2;
@@ -443,7 +444,9 @@ int build_gather_table(const std::vector<short2> &cells, int A, int K, int M, in
                     }
                     return mx;
                 };
-                bool improved = d <= 24;   // (bounded: plan time grows as d^2 per pass)
+                std::vector<int> cost(d);
+                for (int j = 0; j < d; j++) cost[j] = step_cost(j);
+                bool improved = search && d <= 24;   // (bounded: plan time grows as d^2 per pass)
                 for (int pass = 0; pass < 4 && improved; pass++) {
                     improved = false;
                     for (int l = 0; l < grp; l++)
@@ -451,10 +454,15 @@ int build_gather_table(const std::vector<short2> &cells, int A, int K, int M, in
                             for (int j2 = j1 + 1; j2 < d; j2++) {
                                 uint32_t &x = at(j1, l), &y = at(j2, l);
                                 if (x == y) continue;
-                                const int before = step_cost(j1) + step_cost(j2);
                                 std::swap(x, y);
-                                if (step_cost(j1) + step_cost(j2) < before) improved = true;
-                                else std::swap(x, y);
+                                const int c1 = step_cost(j1), c2 = step_cost(j2);
+                                if (c1 + c2 < cost[j1] + cost[j2]) {
+                                    cost[j1] = c1;
+                                    cost[j2] = c2;
+                                    improved = true;
+                                } else {
+                                    std::swap(x, y);
+                                }
                             }
                 }
             }
@@ -899,7 +907,8 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
                 std::vector<uint32_t> tab;
                 std::vector<int4> gidx;
                 std::vector<int2> gchan;
-                rc = epic::build_gather_table(cells, n_ant, p->K, g.M, n_pol, g.chans, tab, gidx, gchan, rows);
+                // (beside the compact lists, for small E-field calls: their latency does not ask for the search)
+                rc = epic::build_gather_table(cells, n_ant, p->K, g.M, n_pol, g.chans, tab, gidx, gchan, rows, 0, !g.cimage);
                 if (rc == EPIC_OK) rc = dev_upload(&g.d_gtab, tab.data(), tab.size());
                 if (rc == EPIC_OK) rc = dev_upload(&g.d_gidx, gidx.data(), gidx.size());
                 if (rc == EPIC_OK) rc = dev_upload(&g.d_gchan, gchan.data(), gchan.size());
