@@ -172,6 +172,7 @@ struct epic_plan_s {
     const void *g_v = nullptr, *g_gains = nullptr, *g_delays = nullptr;
     void *g_out = nullptr;
     int g_T = -1;
+    bool g_first = true;               // no call yet
     bool g_prof = false;
     // host-buffer entry point staging (allocated on first use)
     uint8_t *d_stage_v = nullptr;

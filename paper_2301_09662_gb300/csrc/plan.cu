@@ -561,18 +561,26 @@ void prof_mark(epic_plan_s *plan, cudaStream_t stream, int stage, bool start)
         }
         plan->events.push_back(e);
     }
-    // External records become event-record nodes when the stream is being
-    // captured (a plain record would only mark a dependency)
-    cudaEventRecordWithFlags(plan->events[2 * stage + (start ? 0 : 1)], stream, cudaEventRecordExternal);
+    // While the stream is being captured an external record becomes an event-record node (a plain one
+    // would only mark a dependency); otherwise only the plain one is allowed
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(stream, &st);
+    cudaEventRecordWithFlags(plan->events[2 * stage + (start ? 0 : 1)], stream,
+                             st == cudaStreamCaptureStatusActive ? cudaEventRecordExternal : cudaEventRecordDefault);
     if (!start && stage + 1 > plan->n_recorded) plan->n_recorded = stage + 1;
 }
 
 // One integration on `stream`: replay the plan's CUDA graph (captured on the
-// first call and again whenever T, a pointer or the profiling state changes),
-// or launch directly when graphs are disabled.
+// second call and again whenever T, a pointer or the profiling state changes),
+// or launch directly: when graphs are disabled, and on a plan's first call, which
+// need not be followed by one that could replay a graph (16 antennas, 4 channels
+// of 32 x 32: 96 us with the graph's instantiation, 63 without).
 int run_image(epic_plan_s *p, const uint8_t *v, const float2 *gains, int T, float2 *out, cudaStream_t stream)
 {
-    if (!p->use_graph) return image_fp32(p, v, gains, T, out, stream, false);
+    if (!p->use_graph || p->g_first) {
+        p->g_first = false;
+        return image_fp32(p, v, gains, T, out, stream, false);
+    }
     if (!p->gexec || p->g_v != v || p->g_gains != gains || p->g_delays != p->delays || p->g_out != out ||
         p->g_T != T || p->g_prof != p->profiling) {
         cudaGraph_t graph = nullptr;
