@@ -95,7 +95,8 @@ enum {
 #define EPIC_NO_AUTOSUB  2u     /* keep the autocorrelation term (diagnostics) */
 /* Apply the illumination kernel in the image domain: grid each calibrated
  * voltage into its single cell and multiply the finished image by |W^(l)|^2
- * (FP64).  Because every antenna shares one kernel, gridding through W is a
+ * (in pairs of FP32 numbers, about 48 bits; in FP64 where the kernel's power
+ * leaves 2^-40 .. 2^40).  Because every antenna shares one kernel, gridding through W is a
  * convolution and F(l) = W^(l) sum_a e~_a exp(+2 pi i k_a.l / N); the result
  * equals the default (literal gridding) form up to rounding, with K^2 times
  * fewer gridding operations. */
@@ -108,7 +109,8 @@ enum {
  * writes the gridding kernel W_a per antenna: heterogeneous beams,
  * A-projection, Sec. 3.1).  The autocorrelation term becomes
  * sum_a A_a,pq |W^_a(l)|^2, evaluated from the auto-correlation grid
- * sum_a A_a,pq (W_a (x) W_a^*) in FP64.  FP32 form only; not with
+ * sum_a A_a,pq (W_a (x) W_a^*): grid and first half of its transform in FP64,
+ * the second half in pairs of FP32 numbers.  FP32 form only; not with
  * EPIC_KERNEL_TAPER (which needs one shared kernel) or epic_image_series. */
 #define EPIC_ANTENNA_KERNELS 16u
 
@@ -212,8 +214,8 @@ int epic_image(epic_plan_t plan, const uint8_t *ci4, const float *gains_c64,
  * time-chunk counts -- the cost model's choice, its neighbours, and the counts
  * that fill whole waves of SMs -- and the fastest is kept for later epic_image /
  * epic_image_ex calls with the same n_spectra (other counts fall back to the
- * cost model; epic_image_series keeps one chunk per image).  The next call
- * re-captures its CUDA graph.  Blocks the host until the timing runs finish.
+ * cost model; epic_image_series chooses its own).  The next call
+ * captures its CUDA graph anew.  Blocks the host until the timing runs finish.
  * Results are unchanged up to the FP32 summation order of the time chunks.
  * EPIC_ERR_ARG for a null plan or n_spectra outside [1, max_spectra];
  * EPIC_ERR_NOMEM / EPIC_ERR_CUDA if the scratch buffers or launches fail.

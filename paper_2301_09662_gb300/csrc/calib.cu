@@ -16,7 +16,7 @@
 // E conj(e) to the sums of their own antennas in registers, so an iteration reads the voltages
 // once.  The CTAs' sums meet through distributed shared memory: each CTA finishes a slice of the
 // antennas and hands its gains to the others, so there is no workspace and one launch.  Bound by
-// issue and latency (about 20 instructions a voltage and iteration; 36 % issue).  256 antennas, 64 channels, two
+// issue and latency (about 20 instructions a voltage and iteration; 40 % issue).  256 antennas, 64 channels, two
 // polarisations, 1000 spectra, two iterations: 91 us, against 322 us for one CTA per channel and
 // polarisation, whose loads' latency was the limit.
 // gain_solve_kernel (larger arrays): one CTA per (channel, polarisation), E(t) of all samples in

@@ -32,7 +32,7 @@
 // 128 x 128, 1000 spectra 5.78 -> 3.10 ms; the same as 25 Stokes images with delays 8.30 -> 3.61 ms;
 // per-antenna kernels, 250 spectra 2.55 -> 0.99 ms with their auto image (image_common.cu);
 // 37 channels at 64, 96 and 128 0.67 -> 0.46 ms.  Bound by the transform warps' issue: the FMA
-// pipe is active 51 % of the time (42 % there, for half the work), 8 transform warps an SM.
+// pipe is active 55 % of the time (42 % there, for half the work), 8 transform warps an SM.
 //
 // Shared memory: G [P][rows][65], R [P][rows][N + 1], voltages of two samples,
 // gains, taps and gather lists (read through L1 where they do not fit).

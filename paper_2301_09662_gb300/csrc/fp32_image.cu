@@ -343,7 +343,8 @@ int fp32_pick_tau(int n_items, int T, int sms) { return pick_tau(n_items, T, sms
 
 // The compact kernel's CTA images all classes of a channel: n_chan CTAs per time chunk, each
 // writing Q times the partial image (set-up and write cost ~4 samples).  No chunk is longer than
-// the per-class kernel's would be, so FP32 sums run over no more samples than there.
+// the per-class kernel's would be, so FP32 sums run over no more samples than there (epic_autotune
+// also tries fewer chunks, for either kernel).
 int compact_pick_tau(int n_chan, int n_items, int T, int sms)
 {
     return pick_tau(n_chan, T, sms, fp32_pick_tau(n_items, T, sms), 4.0);

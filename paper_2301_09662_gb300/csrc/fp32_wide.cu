@@ -669,7 +669,10 @@ WideLayout wide_layout(int N, int n_chan, int rpad, int max_spectra, int cap_tb,
 // GB300, us wide / per class: side 256, 300 antennas, 5 x 5, 2 channels x 16 spectra 40 / 34, 4 x 16
 // 46 / 50; 2048 antennas, 7 x 7, 1 x 8 45 / 63; side 512, 2048 antennas, 7 x 7, 1 x 2 59 / 65, 1 x 4
 // 60 / 107; 1000 antennas, 7 x 7, 1 x 4 54 / 47, 1 x 8 58 / 72; 300 antennas, 5 x 5, 1 x 16 60 / 54,
-// 2 x 16 77 / 83; 64 antennas, 3 x 3, 2 x 16 109 / 97, 4 x 12 106 / 105.
+// 2 x 16 77 / 83; 64 antennas, 3 x 3, 2 x 16 109 / 97, 4 x 12 106 / 105.  (1 x 2 of 2048 antennas, 4.1e7
+// by this count, lies on the wrong side; 1 x 4 of 1000, 4.2e7, asks for the line above both.)  At side 512
+// the calls below the line went to the fold path before there were wide kernels: 84 us for 2048 antennas, 1 x 1
+// (63 per class now), 66 for 1000, 1 x 2 (45), 92 for 300, 1 x 16 (51).
 bool wide_pays(const epic_plan_s *plan, const GroupCfg &g, int T)
 {
     const double work = static_cast<double>(g.n_items) * T * (3.0 * plan->A * plan->K * plan->K + 16384.0);

@@ -984,7 +984,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
             // sample) and fold all classes (alias_fold.cu), for the FP32 and the two-stage tensor
             // kernel.  With one tap (the taper) re-gridding per class is cheaper than moving the
             // folded grids through HBM (measured at N = 512: 0.24 s against 0.44 s per dense
-            // integration).  EPIC_NO_ALIAS=1 keeps the per-class gridding.
+            // integration).  EPIC_DIAG_NO_ALIAS keeps the per-class gridding.
             if (rc == EPIC_OK && fold_ok && !g.wide) {
                 std::vector<short2> j0;
                 std::vector<uint32_t> bseg;

@@ -80,3 +80,13 @@ def test_efield_placements(N, left, right):
     p.close()
     ref = oracle.workload_efield(wl)
     assert np.max(np.abs(got - ref)) / np.max(np.abs(ref)) < TOL
+
+
+def test_autotuned_long_call():
+    """The tuner may keep fewer time chunks than the cost model (FP32 sums of up to 600 spectra)."""
+    wl = synth.random_small(A=36, P=2, C=3, T=600, N=128, K=3, seed=11)
+    p = epic.Plan.from_workload(wl)
+    p.autotune(wl.T)
+    got, _ = run_gpu(wl, plan=p)
+    p.close()
+    assert peak_rel_err(got, oracle.workload_image(wl), wl.grid_n, 2).max() < TOL
