@@ -260,6 +260,7 @@ int prepare_compact(const epic_plan_s *plan, const GroupCfg &g);
 size_t efield_smem_bytes(int N, int P, int rows, int rrows, int A, int K, int nker, bool taps, int words);
 int efield_rows(int N, const std::vector<int4> &lchan);   // most rows of R where every channel is placed on a quarter
 bool efield_per_class(int N, int P, int n_items, int T, int sms);   // an E-field call so small that the per-class kernel is faster
+bool efield_tables(int N, int P, int n_items, int max_spectra, int sms);
 int prepare_efield(const epic_plan_s *plan, const GroupCfg &g);
 int launch_compact(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const float2 *gains, int T, int *n_tau,
                    cudaStream_t stream);

@@ -443,6 +443,13 @@ bool efield_per_class(int N, int P, int n_items, int T, int sms)
     return (N == 96 || N == 128) && n_items <= sms && 4 * ctas <= 7LL * sms;
 }
 
+// Whether a plan keeps the per-class tables for such calls: for few channels, where they cost little, and
+// where its longest call is one (37 channels at three sides, 16 ms of plan, would pay 2 ms for them).
+bool efield_tables(int N, int P, int n_items, int max_spectra, int sms)
+{
+    return efield_per_class(N, P, n_items, n_items <= 16 ? 1 : std::max(1, max_spectra), sms);
+}
+
 int prepare_efield(const epic_plan_s *plan, const GroupCfg &g)
 {
     const size_t need = efield_smem_bytes(g.N, plan->P, g.crows, g.erows, plan->A, plan->K, plan->nker, g.etaps, g.estage ? g.cwords : 0);

@@ -888,7 +888,7 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
             // images per class where that is faster (and possible)
             int ccols = 0;
             for (size_t i = 0; i < lchan.size(); i += 2) ccols = std::max(ccols, lchan[i].w);
-            g.eclass = g.compact && g.reg64 && epic::efield_per_class(g.N, n_pol, g.n_items, 1, p->sm_count);
+            g.eclass = g.compact && g.reg64 && epic::efield_tables(g.N, n_pol, g.n_items, max_spectra, p->sm_count);
             g.cimage = g.compact && (!g.reg64 || epic::compact_pays(g.N, n_pol, n_ant, p->K, g.crows, ccols));
             if (g.compact) {
                 g.R1 = 1;

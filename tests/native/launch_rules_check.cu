@@ -167,8 +167,15 @@ static void tuning()
     CHECK(!epic::tunable(&plan, g, 16), "fold path");
 }
 
+static void efield_plans()
+{
+    CHECK(epic::efield_tables(128, 2, 16, 1000, 152) && epic::efield_tables(128, 2, 32, 8, 152), "few channels, short calls");
+    CHECK(!epic::efield_tables(128, 2, 32, 1000, 152) && !epic::efield_tables(64, 2, 4, 1, 152), "more channels, long calls; side 64");
+}
+
 int main()
 {
+    efield_plans();
     tuning();
     stage_time();
     wide();
