@@ -29,7 +29,7 @@
 //    transformed.  G is free as soon as the row transforms hold their inputs.
 //
 // Measured against the per-class kernel (one GB300, whole calls): 256 antennas, 64 channels of
-// 128 x 128, 1000 spectra 5.78 -> 3.10 ms; the same as 25 Stokes images with delays 8.30 -> 3.61 ms;
+// 128 x 128, 1000 spectra 5.78 -> 3.10 ms; the same as 25 Stokes images with delays 8.30 -> 3.55 ms;
 // per-antenna kernels, 250 spectra 2.55 -> 0.99 ms with their auto image (image_common.cu);
 // 37 channels at 64, 96 and 128 0.67 -> 0.46 ms.  Bound by the transform warps' issue: the FMA
 // pipe is active 55 % of the time (42 % there, for half the work), 8 transform warps an SM.
