@@ -436,7 +436,7 @@ int epic_image_static(const double *ant_xy_m, int n_ant, int n_pol,
  *   gains_out   device complex64 [n_chan][n_ant][n_pol], overwritten
  *
  * FP32 sums, exact integer |e|^2 sums; one thread-block cluster per channel (for n_ant n_pol
- * above 1024 one CTA per channel and polarisation).
+ * above 1024, and for short calls, one CTA per channel and polarisation).
  * Asynchronous on the stream; allocates nothing.  EPIC_ERR_ARG for null
  * pointers or out-of-range arguments, EPIC_ERR_TOO_LARGE when the per-CTA
  * shared memory (8 n_spectra + 20 n_ant bytes) exceeds 200 KB.

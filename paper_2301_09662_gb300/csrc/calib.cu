@@ -10,7 +10,7 @@
 // (lx, ly) = (l N du, m N du) pixels (a source there has e_a ~ phi_a and appears
 // at +(lx, ly) in the image).
 //
-// gain_solve_cluster_kernel (n_ant n_pol <= 1024): one thread-block cluster per channel, each CTA
+// gain_solve_cluster_kernel (n_ant n_pol <= 1024, but for the shortest calls): one thread-block cluster per channel, each CTA
 // a share of the samples.  A warp takes a sample at a time: its lanes hold the row's voltages
 // (words lane, lane + 32, ..), form E(t) of both polarisations by one warp reduction and add
 // E conj(e) to the sums of their own antennas in registers, so an iteration reads the voltages
@@ -19,7 +19,7 @@
 // issue and latency (about 20 instructions a voltage and iteration; 40 % issue).  256 antennas, 64 channels, two
 // polarisations, 1000 spectra, two iterations: 91 us, against 322 us for one CTA per channel and
 // polarisation, whose loads' latency was the limit.
-// gain_solve_kernel (larger arrays): one CTA per (channel, polarisation), E(t) of all samples in
+// gain_solve_kernel (larger arrays, short calls): one CTA per (channel, polarisation), E(t) of all samples in
 // shared memory, the voltages read twice per iteration.
 #include <algorithm>
 #include <cmath>
@@ -365,17 +365,14 @@ gain_solve_cluster_kernel(const uint8_t *__restrict__ v, const short2 *__restric
 }
 
 template <int R>
-int launch_cal_cluster(const epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, int T, double lx, double ly, int n_iter,
-                       float2 *gains, cudaStream_t s)
+int launch_cal_cluster(const epic_plan_s *plan, const GroupCfg &g, int cl, const uint8_t *v, int T, double lx, double ly,
+                       int n_iter, float2 *gains, cudaStream_t s)
 {
     const size_t smem = cal_cluster_smem(plan->A * plan->P);
     const auto kfn = gain_solve_cluster_kernel<R>;
     if (cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(cal_cluster_smem(128 * R))) !=
         cudaSuccess)
         return EPIC_ERR_CUDA;
-    // up to two CTAs an SM, in one wave; a CTA keeps at least a sample per warp
-    int cl = 1;
-    while (cl < 8 && cl * g.n_chan <= plan->sm_count && 2 * cl * kCalWarps <= T) cl *= 2;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(g.n_chan * cl));
     cfg.blockDim = dim3(kCalThreads);
@@ -392,6 +389,28 @@ int launch_cal_cluster(const epic_plan_s *plan, const GroupCfg &g, const uint8_t
                ? EPIC_OK
                : EPIC_ERR_CUDA;
 }
+
+}  // namespace
+
+// CTAs of a channel's cluster, or 0 for one CTA per channel and polarisation.  One wave of CTAs (two an SM
+// up to 512 values a row, one above), each with at least a sample per warp.  The cluster's barriers and
+// gain exchange take about 20 us (30 above 512 values) that short calls do not earn back, nor do long rows of both
+// polarisations read by bytes where the clusters come to more than a wave.  One GB300, us one CTA per channel and polarisation / cluster, two iterations:
+// 256 antennas x 2, 61 channels, 8 spectra 10 / 21, 20: 14 / 19, 66: 27 / 25; 200 channels, 66: 47 / 47; 34 x 1, 8
+// channels, 20: 11 / 12; 512 x 2, 8 channels, 20: 23 / 27, 200 channels, 66: 84 / 98; 297 x 2, 200 channels,
+// 1000: 1044 / 1266; 600 x 1, 8 channels, 8: 19 / 25.
+int cal_cluster_size(int AP, int P, int n_chan, int T, int sms)
+{
+    const bool wide = AP > 512, bytes = (AP & 3) != 0 && P == 2;
+    int t_min = !wide ? 48 : P == 1 ? 16 : bytes ? 96 : 64;
+    if (n_chan > sms) t_min = !wide ? 64 : bytes ? 1 << 30 : 128;
+    if (AP > 1024 || T < t_min) return 0;
+    int cl = 1;
+    while (cl < 8 && 2 * cl * n_chan <= (wide ? 1 : 2) * sms && 2 * cl * kCalWarps <= T) cl *= 2;
+    return cl;
+}
+
+namespace {
 
 size_t cal_smem(int A, int T) { return sizeof(float2) * (2 * static_cast<size_t>(A) + T) + sizeof(int) * A; }
 
@@ -413,12 +432,13 @@ extern "C" int epic_solve_gains(epic_plan_t plan, const uint8_t *ci4, int n_spec
     for (const auto &g : plan->groups) {
         const double lx = l * g.N * plan->du, ly = m * g.N * plan->du;
         const int AP = plan->A * plan->P;
-        if (AP <= 1024) {
+        const int cl = epic::cal_cluster_size(AP, plan->P, g.n_chan, n_spectra, plan->sm_count);
+        if (cl > 0) {
             auto *out = reinterpret_cast<float2 *>(gains_out);
-            const int rc = AP <= 128   ? epic::launch_cal_cluster<1>(plan, g, ci4, n_spectra, lx, ly, n_iter, out, s)
-                           : AP <= 256 ? epic::launch_cal_cluster<2>(plan, g, ci4, n_spectra, lx, ly, n_iter, out, s)
-                           : AP <= 512 ? epic::launch_cal_cluster<4>(plan, g, ci4, n_spectra, lx, ly, n_iter, out, s)
-                                       : epic::launch_cal_cluster<8>(plan, g, ci4, n_spectra, lx, ly, n_iter, out, s);
+            const int rc = AP <= 128   ? epic::launch_cal_cluster<1>(plan, g, cl, ci4, n_spectra, lx, ly, n_iter, out, s)
+                           : AP <= 256 ? epic::launch_cal_cluster<2>(plan, g, cl, ci4, n_spectra, lx, ly, n_iter, out, s)
+                           : AP <= 512 ? epic::launch_cal_cluster<4>(plan, g, cl, ci4, n_spectra, lx, ly, n_iter, out, s)
+                                       : epic::launch_cal_cluster<8>(plan, g, cl, ci4, n_spectra, lx, ly, n_iter, out, s);
             if (rc != EPIC_OK) return rc;
             continue;
         }

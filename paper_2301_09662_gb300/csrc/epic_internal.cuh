@@ -254,6 +254,7 @@ int build_gather_table(const std::vector<short2> &cells, int A, int K, int M, in
 // FP32 kernel for apertures of at most 64 x 64 cells, grid sides 64, 96, 128 (fp32_compact.cu)
 int build_compact_lists(const std::vector<short2> &cells, int A, int K, int P, const std::vector<int> &chans,
                         std::vector<uint16_t> &tab, std::vector<int2> &idx, std::vector<int4> &chan);
+int cal_cluster_size(int AP, int P, int n_chan, int T, int sms);   // gain solver (calib.cu)
 bool compact_pays(int N, int P, int A, int K, int rows, int cols);
 size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words);
 int prepare_compact(const epic_plan_s *plan, const GroupCfg &g);

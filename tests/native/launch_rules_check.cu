@@ -173,8 +173,29 @@ static void efield_plans()
     CHECK(!epic::efield_tables(128, 2, 32, 1000, 152) && !epic::efield_tables(64, 2, 4, 1, 152), "more channels, long calls; side 64");
 }
 
+// Gain solver: clusters where they are the faster form (measured pairs), in one wave where that is possible
+static void gains()
+{
+    const struct {
+        int A, P, C, T;
+        bool cluster;
+    } at[] = {{256, 2, 61, 8, false}, {256, 2, 61, 20, false}, {256, 2, 61, 66, true},    {256, 2, 64, 1000, true}, {34, 1, 8, 20, false},
+              {512, 2, 8, 20, false}, {512, 2, 200, 66, false}, {512, 2, 200, 200, true}, {297, 2, 200, 1000, false},
+              {600, 1, 8, 8, false},  {600, 1, 8, 20, true},   {1001, 1, 200, 200, true}, {297, 2, 61, 66, false},    {513, 2, 4, 1000, false}};
+    for (const auto &c : at)
+        CHECK((epic::cal_cluster_size(c.A * c.P, c.P, c.C, c.T, 152) > 0) == c.cluster, "%d x %d, %d channels, %d spectra", c.A, c.P, c.C,
+              c.T);
+    for (int AP : {64, 512, 600, 1024})
+        for (int C : {1, 19, 38, 61, 64, 76, 77, 152, 153, 304})
+            for (int T : {64, 128, 1000}) {
+                const int cl = epic::cal_cluster_size(AP, 2, C, T, 152), room = AP > 512 ? 152 : 304;
+                CHECK(cl <= 1 || cl * C <= room, "%d values, %d channels: clusters of %d", AP, C, cl);
+            }
+}
+
 int main()
 {
+    gains();
     efield_plans();
     tuning();
     stage_time();

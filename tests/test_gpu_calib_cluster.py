@@ -1,6 +1,6 @@
 """The gain solver's cluster form (n_ant n_pol <= 1024) at the edges of its row
 widths, with few samples and odd rows, and the one-CTA form just past it,
-against the FP64 oracle.  FP32 sums of T <= 70 samples and A <= 513 antennas:
+against the FP64 oracle.  FP32 sums of T <= 70 samples and A <= 601 antennas:
 relative rounding below 2^-24 sqrt(T A) ~ 1e-5 of the unit RMS gain."""
 import numpy as np
 import pytest
@@ -20,8 +20,15 @@ pytestmark = pytest.mark.gpu
     (128, 2, 70, 40),   # 256 values, many channels: small clusters
     (256, 2, 2, 7),     # fewer samples than warps
     (257, 1, 1, 1),     # one sample, odd row
-    (512, 2, 1, 50),    # 1024 values, the widest
-    (513, 2, 1, 20),    # past it: the one-CTA form
+    (512, 2, 1, 50),    # 1024 values
+    (513, 2, 1, 20),    # past the widest: the one-CTA form
+    # the calls above of fewer than 48 spectra (64 past 512 values) take the one-CTA form; clusters:
+    (65, 2, 2, 49),     # rows read by bytes, a sample more than a multiple of the warps
+    (128, 2, 70, 48),   # the shortest, many channels: small clusters
+    (257, 1, 1, 51),    # odd row
+    (512, 2, 1, 67),    # the widest
+    (300, 2, 61, 64),   # 600 values: one CTA an SM
+    (601, 1, 2, 17),    # past 512 values of one polarisation
 ])
 def test_edges(A, P, C, T):
     wl = synth.random_small(A=A, P=P, C=C, T=T, N=128, K=1, seed=A + T, gains=False)
