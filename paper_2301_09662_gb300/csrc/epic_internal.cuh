@@ -256,6 +256,7 @@ int build_compact_lists(const std::vector<short2> &cells, int A, int K, int P, c
                         std::vector<uint16_t> &tab, std::vector<int2> &idx, std::vector<int4> &chan);
 int cal_cluster_size(int AP, int P, int n_chan, int T, int sms);   // gain solver (calib.cu)
 bool compact_pays(int N, int P, int A, int K, int rows, int cols);
+bool compact_pays_odd(int N, int P, int K);
 size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words);
 int prepare_compact(const epic_plan_s *plan, const GroupCfg &g);
 size_t efield_smem_bytes(int N, int P, int rows, int rrows, int A, int K, int nker, bool taps, int words);

@@ -658,6 +658,11 @@ bool compact_pays(int N, int P, int A, int K, int rows, int cols)
     return N != 64 || per_row > (P == 2 ? 5.0 : 60.0);
 }
 
+// The same against the shared-memory kernel, where n_ant n_pol is not a multiple of 4: its atomics cost
+// little for one tap.  Side 64, one polarisation, us there / here: 34 antennas, 1 x 1, 60 channels x 74 spectra
+// 76 / 90, 32 x 300 139 / 147, 255 antennas 82 / 92 and 152 / 150; 17 antennas, 3 x 3 92 / 90.
+bool compact_pays_odd(int N, int P, int K) { return !(N == 64 && P == 1 && K == 1); }
+
 size_t compact_smem_bytes(int N, int P, int rows, int A, int K, int nker, bool taps, int words)
 {
     return compact_smem(P, N == 64 ? 2 : 1, N, rows, A, K, nker, taps, words).total;

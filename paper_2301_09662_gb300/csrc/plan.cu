@@ -889,7 +889,9 @@ int epic_plan(epic_plan_t *out, const double *ant_xy_m, int n_ant, int n_pol,
             int ccols = 0;
             for (size_t i = 0; i < lchan.size(); i += 2) ccols = std::max(ccols, lchan[i].w);
             g.eclass = g.compact && g.reg64 && epic::efield_tables(g.N, n_pol, g.n_items, max_spectra, p->sm_count);
-            g.cimage = g.compact && (!g.reg64 || epic::compact_pays(g.N, n_pol, n_ant, p->K, g.crows, ccols));
+            g.cimage = g.compact && (g.reg64 ? epic::compact_pays(g.N, n_pol, n_ant, p->K, g.crows, ccols)
+                                             : p->nker > 1 || epic::compact_pays_odd(g.N, n_pol, p->K));
+            if (!g.reg64) g.compact = g.cimage;   // (no E-field images without it)
             if (g.compact) {
                 g.R1 = 1;
                 g.R2 = g.M;

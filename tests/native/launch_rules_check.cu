@@ -46,6 +46,8 @@ static void side64()
         bool compact;
     } at[] = {{1, 64, 5, 56, false}, {1, 64, 7, 56, false}, {1, 64, 3, 15, false}, {1, 32, 5, 15, false}, {1, 64, 5, 16, true},
               {1, 256, 3, 15, true},  {2, 16, 1, 14, false}, {2, 16, 1, 56, false}, {2, 32, 3, 15, true},  {2, 256, 5, 40, true}};
+    CHECK(!epic::compact_pays_odd(64, 1, 1) && epic::compact_pays_odd(64, 1, 3) && epic::compact_pays_odd(64, 2, 1) &&
+              epic::compact_pays_odd(96, 1, 1), "odd rows");
     for (const auto &c : at) {
         CHECK(epic::compact_pays(64, c.P, c.A, c.K, c.span, c.span) == c.compact, "side 64, P %d, %d antennas, K %d, %d cells", c.P,
               c.A, c.K, c.span);

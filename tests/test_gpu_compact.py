@@ -33,7 +33,8 @@ def _span(wl, span, K):
     (96, 2, 50, 6, 3, 49),      # folds one position past 48
     (96, 1, 30, 2, 5, 64),
     (64, 2, 24, 7, 3, 40),      # two samples at a time, the last one absent
-    (64, 1, 23, 8, 1, 33),
+    (64, 1, 23, 8, 1, 33),      # one tap, odd row: the shared-memory kernel
+    (64, 1, 23, 8, 3, 33),
     (64, 2, 40, 3, 5, 60),      # planes of two samples do not fit: the per-class kernel
     (64, 1, 104, 9, 5, 40),     # 65 footprint cells a row: compact with a single polarisation
     (64, 1, 92, 9, 5, 40),      # 57.5: the per-class kernel
