@@ -316,7 +316,7 @@ struct RawImage {
 };
 int fp32_pick_tau(int n_items, int T, int sms);
 int compact_pick_tau(int n_chan, int n_items, int T, int sms);
-bool fork_pays(int n_items, int n_tau, int T, int sms);   // side 32: auto sums beside the imaging
+bool fork_pays(int n_items, int n_tau, int T, int sms, int P, int AKK);   // side 32: auto sums beside the imaging
 int series_chunks(int items, int n_img, int spi, int tau_cap, int sms);   // compact groups: time chunks per image
 // time chunks of one launch: forced (image series), else autotuned for this T, else the cost model
 bool tunable(const epic_plan_s *plan, const GroupCfg &g, int T);   // epic_autotune has something to measure

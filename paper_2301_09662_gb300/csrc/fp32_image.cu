@@ -435,15 +435,18 @@ int launch_imaging(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const
 }
 
 // Whether the auto sums of a plan with one group of side 32 run beside its imaging.  That kernel's CTAs
-// share SMs, so where they come to one wave of long chunks (n_tau chunks of T spectra) blocks of the auto
-// sums placed among them can leave two on an SM and none on another for the whole call, and which are
-// placed first varies in a row of calls.  Two polarisations, ms one after the other / beside each other:
-// 256 antennas, 152 channels x 500 spectra (chunks of 500) 4.12 / 4.11 .. 5.00; 16 antennas, 8 channels x
-// 1000 (of 53) 0.271 / 0.263 .. 0.306, 16 channels x 200 (of 23) 0.127 / 0.121; 4 channels x 64, one
-// polarisation (of 2) 0.0205 / 0.0164.
-bool fork_pays(int n_items, int n_tau, int T, int sms)
+// share SMs, so where they come to one wave (n_tau chunks of T spectra) blocks of the auto sums placed
+// among them can leave two on an SM and none on another for the whole call: with the imaging started first
+// in about one row of calls of ten.  The fork gains the auto sums' 4 to 25 us, a bad placement costs a tenth
+// of the wave, so it pays for all but long ones: a CTA's samples take about P (1.4 + 0.0018 A K^2) us each.  3
+// x 3, us one after the other / beside each other: two polarisations, 256 antennas, 152 channels x 500 spectra
+// (4100 by that count) 4120 / 4110 .. 5000, 8 x 200 (60) 139 / 130, 16 antennas, 8 x 1000 (170) 271 / 263 ..
+// 306; one polarisation, 414 antennas, 20 x 81 (100) 146 / 136 .. 152, 1024 antennas, 8 x 200 (215) 251 / 233, 16
+// antennas, 4 x 64 (3) 20.5 / 16.4.
+bool fork_pays(int n_items, int n_tau, int T, int sms, int P, int AKK)
 {
-    return static_cast<long long>(n_items) * n_tau > sms || (T + n_tau - 1) / n_tau < 48;
+    const double wave = (T + n_tau - 1) / n_tau * P * (1.4 + 0.0018 * AKK);
+    return static_cast<long long>(n_items) * n_tau > sms || wave < 1000.0;
 }
 
 // Launch every kernel of one integration.  With fork, the auto-power kernel
@@ -463,7 +466,8 @@ int image_fp32(epic_plan_s *plan, const uint8_t *v, const float2 *gains, int T, 
     const bool autosub = !(plan->flags & EPIC_NO_AUTOSUB);
     const bool side32 = plan->groups.size() == 1 && plan->groups[0].M == 32;
     fork = fork && !plan->side.empty() &&
-           !(side32 && !fork_pays(plan->groups[0].n_items, choose_tau(plan, plan->groups[0], T), T, plan->sm_count));
+           !(side32 && !fork_pays(plan->groups[0].n_items, choose_tau(plan, plan->groups[0], T), T, plan->sm_count,
+                                   plan->P, plan->A * plan->K * plan->K));
     int rc = EPIC_OK;
     const int lead = autosub ? 1 : 0;    // stages: the auto sums, then imaging and epilogue of each group
     prof_begin(plan);

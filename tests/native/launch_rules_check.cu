@@ -69,9 +69,9 @@ static void tiles()
 // Side 32 alone: no fork beside one wave of long chunks (measured pairs).
 static void fork32()
 {
-    CHECK(!epic::fork_pays(152, 1, 500, 152) && !epic::fork_pays(8, 19, 1000, 152), "one wave of long chunks");
-    CHECK(epic::fork_pays(4, 32, 64, 152) && epic::fork_pays(64, 7, 200, 152) && epic::fork_pays(16, 9, 200, 152),
-          "short chunks, several waves");
+    CHECK(!epic::fork_pays(152, 1, 500, 152, 2, 2304) && !epic::fork_pays(152, 1, 500, 152, 2, 144), "one long wave");
+    CHECK(epic::fork_pays(4, 32, 64, 152, 1, 144) && epic::fork_pays(64, 7, 200, 152, 2, 144) && epic::fork_pays(20, 7, 81, 152, 1, 3726),
+          "short wave, several waves");
 }
 
 // E-field calls: per class while its CTAs fit on the SMs at once (measured pairs).
