@@ -51,7 +51,7 @@ L2_FLUSH_BYTES = 256 << 20
 # source changes.  Filled in from the committed profiles/ summaries.
 NCU_TRAFFIC = {
     ("lwa", "tc_split_fp16"): (196.63e6, "758209b70c6bc67f"),     # profiles/tc_pair128_kernel_lwa.md
-    ("lwa", "fp32"): (207.50e6, "b80d18a305ac77be"),              # profiles/fp32_compact_kernel_lwa.md
+    ("lwa", "fp32"): (207.50e6, "8aedfd0f46376679"),              # profiles/fp32_compact_kernel_lwa.md
 }
 # What the same capture shows about the kernel's limits (same keys and hashes).
 NCU_LIMITER = {
@@ -62,7 +62,7 @@ NCU_LIMITER = {
     ("lwa", "fp32"): ({"fma_pipe_active_pct": 55.1, "issue_active_pct": 54.7, "warps_active_pct": 18.7,
                       "registers_per_thread": 162, "smem_conflict_wavefront_share": 0.15,
                       "top_stalls": "wait 0.95, long_scoreboard 0.84, barrier 0.68"},
-                     "b80d18a305ac77be"),
+                     "8aedfd0f46376679"),
 }
 
 
