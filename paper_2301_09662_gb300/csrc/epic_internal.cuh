@@ -333,7 +333,7 @@ int launch_alias(epic_plan_s *plan, const GroupCfg &g, const uint8_t *v, const f
 size_t fp32_smem_bytes(int M, int P, int A, int K);
 int launch_fp32_raw(const RawImage &r, const uint8_t *v, const float2 *gains, cudaStream_t stream);
 int launch_autopower_raw(const RawImage &r, const uint8_t *v, int sm_count, cudaStream_t stream);
-int epi_tiles(int N, int images, int sms);          // pixel tiles of the epilogue
+int epi_tiles(int N, int P, int images, int sms);          // pixel tiles of the epilogue
 int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, int sm_count, cudaStream_t stream);
 // host tables shared by the plan and the static-scratch entry point
 int host_cell_map(const double *ant_xy_m, int n_ant, const double *freq_hz, int n_chan, const int *grid_n,

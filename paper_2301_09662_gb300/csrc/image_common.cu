@@ -464,7 +464,7 @@ int launch_epi(epic_plan_s *plan, const GroupCfg &g, const float2 *gains, int T,
 {
     return epi_dispatch(g.N, g.M, plan->P, [&](auto n_, auto m_, auto p_) {
         constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
-        const dim3 grid(static_cast<unsigned>(epi_tiles(N, g.n_chan * n_img, plan->sm_count)), static_cast<unsigned>(g.n_chan),
+        const dim3 grid(static_cast<unsigned>(epi_tiles(N, P, g.n_chan * n_img, plan->sm_count)), static_cast<unsigned>(g.n_chan),
                         static_cast<unsigned>(n_img));
         const auto kfn = plan->nker > 1                                                    ? epilogue_kernel<N, M, P, kAntennas>
                          : (plan->flags & EPIC_KERNEL_TAPER) && g.wscale != 1.0 ? epilogue_kernel<N, M, P, kTaper64>
@@ -510,14 +510,16 @@ __global__ void delay_prep_kernel(const double *__restrict__ delays, int n, doub
 
 }  // namespace
 
-// Pixel tiles: four pixels a thread, one where that would leave SMs without a block.  One GB300, whole
+// Pixel tiles: four pixels a thread, one where that would leave SMs without a block (with one polarisation,
+// a quarter of the work a pixel, below 1.6 blocks an SM).  One GB300, whole
 // calls of 16 spectra, us with four / one: two polarisations, 16 antennas, 128 x 128, 4 channels (64 /
 // 256 blocks) 32 / 29, 16 channels (256 / 1024) 39 / 49, 32 channels 57 / 82; one polarisation, 100
-// antennas, 64 x 64, 32 channels (128 / 512) 27 / 24, 64 channels 33 / 33; two of 512 x 512 (512 / 2048) 41 / 49.
-int epi_tiles(int N, int images, int sms)
+// antennas, 64 x 64, 32 channels (128 / 512) 27 / 24, 64 channels 33 / 33, 16 antennas, 128 x 128, 10 channels
+// (160 / 640) 33 / 29; two of 512 x 512 (512 / 2048) 41 / 49.
+int epi_tiles(int N, int P, int images, int sms)
 {
     const int one = (N * N + kThreads - 1) / kThreads, four = (one + 3) / 4;
-    return four * images >= sms ? four : one;
+    return four * images * 5 >= sms * (P == 2 ? 5 : 8) ? four : one;
 }
 
 int launch_autopower_raw(const RawImage &r, const uint8_t *v, int sm_count, cudaStream_t stream)
@@ -531,7 +533,7 @@ int launch_epilogue_raw(const RawImage &r, const float2 *gains, float2 *out, int
 {
     return epi_dispatch(r.N, r.M, r.P, [&](auto n_, auto m_, auto p_) {
         constexpr int N = decltype(n_)::value, M = decltype(m_)::value, P = decltype(p_)::value;
-        const dim3 grid(static_cast<unsigned>(epi_tiles(N, r.C, sm_count)), static_cast<unsigned>(r.C));
+        const dim3 grid(static_cast<unsigned>(epi_tiles(N, P, r.C, sm_count)), static_cast<unsigned>(r.C));
         const auto kfn = (r.flags & EPIC_KERNEL_TAPER) && r.wscale != 1.0 ? epilogue_kernel<N, M, P, kTaper64>
                                                                           : epilogue_kernel<N, M, P, kShared>;
         kfn<<<grid, kThreads, 0, stream>>>(r.partial, r.n_tau, r.n_items, 8, M / 8, r.chans, r.out_off, r.wpow, r.wscale, nullptr,

@@ -62,8 +62,10 @@ static void tiles()
         int N, images, want;
     } at[] = {{32, 4, 4}, {128, 4, 64}, {128, 16, 16}, {128, 32, 16}, {64, 32, 16}, {64, 64, 4}, {64, 150, 4}, {512, 1, 256}, {128, 8, 64}};
     for (const auto &c : at)
-        CHECK(epic::epi_tiles(c.N, c.images, 152) == c.want, "side %d, %d images: %d tiles", c.N, c.images,
-              epic::epi_tiles(c.N, c.images, 152));
+        CHECK(epic::epi_tiles(c.N, 2, c.images, 152) == c.want, "side %d, %d images: %d tiles", c.N, c.images,
+              epic::epi_tiles(c.N, 2, c.images, 152));
+    CHECK(epic::epi_tiles(128, 1, 10, 152) == 64 && epic::epi_tiles(64, 1, 38, 152) == 16 && epic::epi_tiles(128, 1, 16, 152) == 16,
+          "one polarisation");
 }
 
 // Side 32 alone: no fork beside one wave of long chunks (measured pairs).
