@@ -50,7 +50,7 @@ L2_FLUSH_BYTES = 256 << 20
 # with the hash of the kernel source it was taken on; ignored (null) once the
 # source changes.  Filled in from the committed profiles/ summaries.
 NCU_TRAFFIC = {
-    ("lwa", "tc_split_fp16"): (196.63e6, "758209b70c6bc67f"),     # profiles/tc_pair128_kernel_lwa.md
+    ("lwa", "tc_split_fp16"): (196.63e6, "dc9001e266e5d34a"),     # profiles/tc_pair128_kernel_lwa.md
     ("lwa", "fp32"): (207.50e6, "8aedfd0f46376679"),              # profiles/fp32_compact_kernel_lwa.md
 }
 # What the same capture shows about the kernel's limits (same keys and hashes).
@@ -58,7 +58,7 @@ NCU_LIMITER = {
     ("lwa", "tc_split_fp16"): ({"tensor_pipe_active_pct": 46.9, "issue_active_pct": 51.4, "warps_active_pct": 18.7,
                                "smem_conflict_wavefront_share": 0.37,
                                "top_stalls": "short_scoreboard 1.04, wait 1.04, not_selected 0.66"},
-                              "758209b70c6bc67f"),
+                              "dc9001e266e5d34a"),
     ("lwa", "fp32"): ({"fma_pipe_active_pct": 55.1, "issue_active_pct": 54.7, "warps_active_pct": 18.7,
                       "registers_per_thread": 162, "smem_conflict_wavefront_share": 0.15,
                       "top_stalls": "wait 0.95, long_scoreboard 0.84, barrier 0.68"},
@@ -317,8 +317,8 @@ def occupied_k_blocks(wl, c, fold, K):
 def tensor_roofline(wl, form, img_ms, peaks, pair=True, taper=False):
     """Executed tensor FLOPs of the tensor-core imaging launch over its time.
     Each 64-point DFT stage of one sample is 8 k-blocks x terms MMAs of
-    128 x 128 x 16, of which the pair kernel (grid sides 128, 96 and 64) issues
-    those with occupied columns (row stage) or rows (column stages).  Sides 128
+    128 x 128 x 16, of which the pair kernel issues those with occupied columns (row
+    stage) or rows (column stages) at grid sides 128 and 64, and six at 96.  Sides 128
     and 96 run two CTAs per channel, each a row stage and two column stages; side
     64 one CTA, a row and a column stage; other sides (and these with
     EPIC_DIAG_NO_PAIR) 2 stages per class.  Also the method's algorithmic FLOPs
@@ -332,7 +332,7 @@ def tensor_roofline(wl, form, img_ms, peaks, pair=True, taper=False):
         fold = 48 if n == 96 else 64                    # side 96: 48-point DFTs
         classes = max(1, n // fold) ** 2
         if pair and n in (128, 96, 64):
-            kx, ky = occupied_k_blocks(wl, c, fold, K)
+            kx, ky = (3, 3) if n == 96 else occupied_k_blocks(wl, c, fold, K)
             ctas = 1 if n == 64 else 2
             stages += ctas * (2 * kx + ctas * 2 * ky) / 8.0
         else:
