@@ -434,13 +434,14 @@ int efield_rows(int N, const std::vector<int4> &lchan)
 // where the per-class kernel has a CTA for each.  Where those find room on the SMs at
 // once (a CTA takes one sample, or two of one polarisation) the call is its latency.  One GB300, us per
 // class / here: side 128, two polarisations, 4 channels x 8 spectra (128 CTAs) 12.3 / 18.4, 4 x 12 (192) 15.4
-// / 18.5, 8 x 8 with 1000 antennas (256) 35 / 39, 4 x 20 (320) 22.5 / 18.5, 64 x 2 (512) 28.7 / 20.5; one, 4
+// / 18.5, 8 x 8 with 1000 antennas (256) 35 / 39, 5 x 14 (280) 14.4 / 18.5,
+// 4 x 20 (320) 22.5 / 18.5, 64 x 2 (512) 28.7 / 20.5; one, 4
 // x 8 (64) 10.3 / 16.4, 16 x 8 (256) 16.4 / 18.5, 64 x 2 (256 in one sample's classes) 20.7 / 18.5; side
 // 96, two, 4 x 12 14.4 / 15.4, 4 x 20 19.5 / 16.0.  At side 64 this kernel is not the slower one.
 bool efield_per_class(int N, int P, int n_items, int T, int sms)
 {
     const long long ctas = static_cast<long long>(n_items) * (P == 1 ? (T + 1) / 2 : T);
-    return (N == 96 || N == 128) && n_items <= sms && 4 * ctas <= 7LL * sms;
+    return (N == 96 || N == 128) && n_items <= sms && ctas <= 2LL * sms;
 }
 
 // Whether a plan keeps the per-class tables for such calls: for few channels, where they cost little, and

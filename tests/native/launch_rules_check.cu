@@ -82,7 +82,7 @@ static void efield()
     const struct {
         int N, P, items, T;
         bool classes;
-    } at[] = {{128, 2, 16, 8, true}, {128, 2, 16, 12, true}, {128, 2, 32, 8, true}, {128, 2, 16, 20, false}, {128, 2, 256, 1, false},
+    } at[] = {{128, 2, 16, 8, true}, {128, 2, 16, 12, true}, {128, 2, 32, 8, true}, {128, 2, 20, 14, true},  {128, 2, 16, 20, false}, {128, 2, 256, 1, false},
               {128, 1, 16, 8, true}, {128, 1, 64, 8, true},  {128, 1, 256, 2, false}, {96, 2, 16, 12, true}, {96, 2, 16, 20, false},
               {64, 2, 4, 1, false}};
     for (const auto &c : at)
